@@ -55,7 +55,8 @@ typedef enum gpe_status {
 
 typedef enum gpe_precision {
     GPE_C64 = 0,   /* complex64 bulk arithmetic, FP64 reductions and tables */
-    GPE_C128 = 1   /* complex128 throughout                                 */
+    GPE_C128 = 1   /* complex128 state; the 2D/3D sweeps hold each line in 64-bit
+                      fixed point with a scale of its own (no less exact)    */
 } gpe_precision;
 
 /* Problem description (copied by gpe_plan_create). */

@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/gpe.h"
+#include "fx.cuh"
 #include "gpe_internal.h"
 
 namespace gpe {
@@ -91,6 +92,10 @@ struct gpe_plan {
     int device = 0;
     bool trap[3] = {false, false, false};
     void *tw[3] = {}, *kt[3] = {}, *ki[3] = {}, *vh[3] = {}, *vf[3] = {}, *vi[3] = {};
+    // complex128 sweeps (fixed point, see PassArgs::gq): unit factors, decay
+    // factors and their exponents, trap angles and exponents per instance
+    void *twx[3] = {}, *ktx[3] = {}, *kix[3] = {}, *vq[3] = {}, *viq[3] = {}, *gq = nullptr;
+    int kix_e[3] = {0, 0, 0};
     void *vsamp = nullptr;       // sampled potential [N] in the bulk real type, or NULL
     double *g_dev = nullptr, *gamma_dev = nullptr, *scale = nullptr, *partials = nullptr;
     double *sums = nullptr, *out6 = nullptr, *out4 = nullptr;
@@ -141,6 +146,8 @@ struct gpe_plan {
     void *sched[3] = {nullptr, nullptr, nullptr};
     void *sched_last = nullptr;
     double *dtab = nullptr;                 // dither angles and offsets per step (resident kernel)
+    // complex128 sweeps of 2D and 3D steps run in fixed point, on tables of their own
+    bool fxp() const { return prec == GPE_C128 && ndim >= 2; }
 };
 
 static gpe_status check_err(gpe_plan *p);
@@ -223,6 +230,117 @@ static void destroy(gpe_plan *p)
             if (e) cudaEventDestroy(e);
     if (p->copy_st) cudaStreamDestroy(p->copy_st);
     delete p;
+}
+
+static gpe_status upload_raw(gpe_plan *p, void **dst, const void *src, size_t bytes)
+{
+    GPE_TRY(dalloc(p, dst, bytes));
+    GPE_CUDA(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
+    return GPE_OK;
+}
+
+// ------------------------------------------------------------------ fixed-point tables (complex128)
+// exp(-2 pi i t / n), t < n, as 62-bit unit factors.  n is a power of two, so
+// every angle is one of the first octant up to exact symmetries; there sine and
+// cosine are summed from their Maclaurin series in two-double arithmetic
+// (error below 2^-100), because a factor rounded to a double would carry a
+// modulus error of 2^-54 into every step.
+namespace {
+struct TwoDouble {
+    double h, l;
+};
+TwoDouble td_add(TwoDouble a, TwoDouble b)
+{
+    const double s = a.h + b.h, v = s - a.h;
+    const double e = (a.h - (s - v)) + (b.h - v) + a.l + b.l;
+    const double h = s + e;
+    return {h, e - (h - s)};
+}
+TwoDouble td_mul(TwoDouble a, TwoDouble b)
+{
+    const double p = a.h * b.h;
+    const double e = fma(a.h, b.h, -p) + a.h * b.l + a.l * b.h;
+    const double h = p + e;
+    return {h, e - (h - p)};
+}
+TwoDouble td_div(TwoDouble a, double d)
+{
+    const double q = a.h / d;
+    const double r = (fma(-q, d, a.h) + a.l) / d;
+    const double h = q + r;
+    return {h, r - (h - q)};
+}
+int64_t td_fixed62(TwoDouble a) { return (int64_t)ldexp(a.h, 62) + llrint(ldexp(a.l, 62)); }
+}  // namespace
+static void unit_circle_fx(int64_t n, std::vector<int4> &out)
+{
+    const TwoDouble two_pi = {6.283185307179586, 2.4492935982947064e-16};
+    const int64_t one = (int64_t)1 << 62;
+    std::vector<int64_t> c(n / 8 + 1), s(n / 8 + 1);
+    for (int64_t t = 0; t <= n / 8; ++t) {
+        const TwoDouble x = td_mul(two_pi, {(double)t / (double)n, 0.0}), x2 = td_mul(x, x);
+        TwoDouble ct = {1.0, 0.0}, st = x, cs = ct, ss = st;
+        for (int k = 1; k <= 16; ++k) {
+            ct = td_div(td_mul(ct, x2), -(double)((2 * k - 1) * (2 * k)));
+            st = td_div(td_mul(st, x2), -(double)((2 * k) * (2 * k + 1)));
+            cs = td_add(cs, ct);
+            ss = td_add(ss, st);
+        }
+        c[t] = t ? td_fixed62(cs) : one;
+        s[t] = t ? td_fixed62(ss) : 0;
+    }
+    out.resize(n);
+    for (int64_t t = 0; t < n; ++t) {
+        // t = quarter turns + r, r folded into the first octant
+        const int quad = (int)(4 * t / n);
+        const int64_t r = t - quad * (n / 4);          // n < 4 has no quarter turns: r = 0 or n/2 handled below
+        int64_t cr, sr;
+        if (n < 4) {
+            cr = t ? -one : one;
+            sr = 0;
+        } else {
+            const bool fold = 8 * r > n;
+            const int64_t k = fold ? n / 4 - r : r;
+            const int64_t c0 = fold ? s[k] : c[k], s0 = fold ? c[k] : s[k];
+            cr = quad == 0 ? c0 : quad == 1 ? -s0 : quad == 2 ? -c0 : s0;
+            sr = quad == 0 ? s0 : quad == 1 ? c0 : quad == 2 ? -s0 : -c0;
+        }
+        out[t] = fx_pack(cr, -sr);
+    }
+}
+// sqrt(|g| c / 2 pi) = m 2^e, m of 62 bits
+static FxCoupling coupling_fx(double g, double c)
+{
+    FxCoupling r = {0, 0, 0};
+    const double a = g * c;
+    r.neg = a < 0.0;
+    const double v = sqrt(fabs(a) / (2.0 * M_PI));
+    if (!(v > 0.0)) return r;
+    int ex = 0;
+    const double f = frexp(v, &ex);                    // [1/2, 1)
+    r.m = std::min((int64_t)ldexp(f, 62), ((int64_t)1 << 62) - 1);
+    r.e = ex - 62;
+    return r;
+}
+// an angle in radians as a multiple of 2^-64 turns
+static int64_t turns_fx(double th)
+{
+    double t = th / (2.0 * M_PI);
+    t -= rint(t);                                      // [-1/2, 1/2]
+    return (int64_t)((uint64_t)(int64_t)ldexp(t, 63) << 1);
+}
+// an exponent V c (natural) in powers of two, to 53 fraction bits; beyond 2^+-200 the factor stays there
+static int64_t exponent_fx(double th) { return llrint(ldexp(std::max(-200.0, std::min(200.0, th * M_LOG2E)), 53)); }
+
+// half-step trap angles and exponents of one instance on axis a, or of a sampled 1D potential
+static void trap_fx(const gpe_plan *p, int a, double gamma, int64_t *vq, int64_t *viq)
+{
+    for (int64_t j = 0; j < p->n[a]; ++j) {
+        const double x = p->lo[a] + (double)j * p->h[a];
+        const double th = 0.5 * gamma * gamma * x * x * p->dt;
+        vq[j] = turns_fx(0.5 * th);
+        viq[j] = exponent_fx(0.5 * th);
+    }
 }
 
 // Trap tables of one instance on axis a (V_a = gamma^2 x^2 / 2, th = V_a dt):
@@ -346,9 +464,38 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
             kt[2 * t + 1] = -sin(th);
             ki[t] = exp(-th) / (double)na;
         }
+        PLAN_TRY(upload_real(p, &p->ki[a], ki));
+        if (p->prec == GPE_C128) {
+            std::vector<int4> ux;
+            unit_circle_fx(na, ux);
+            PLAN_TRY(upload_raw(p, &p->twx[a], ux.data(), ux.size() * sizeof(int4)));
+        }
+        if (p->fxp()) {
+            std::vector<int4> ux(na);
+            std::vector<int64_t> kx(na);
+            const int64_t one = (int64_t)1 << 62;
+            // decay factors relative to a power of two that bounds them (1, unless dt < 0)
+            double kmax = 1.0;
+            for (int64_t t = 0; t < na; ++t) kmax = std::max(kmax, ki[t] * (double)na);
+            int ex = 0;
+            if (kmax > 1.0) frexp(kmax, &ex);
+            p->kix_e[a] = ex;
+            for (int64_t t = 0; t < na; ++t) {
+                ux[t] = fx_pack(one + llrint(ldexp(kt[2 * t], 62)), llrint(ldexp(kt[2 * t + 1], 62)));
+                kx[t] = (int64_t)ldexp(ki[t] * (double)na, 62 - ex);
+            }
+            PLAN_TRY(upload_raw(p, &p->ktx[a], ux.data(), ux.size() * sizeof(int4)));
+            PLAN_TRY(upload_raw(p, &p->kix[a], kx.data(), kx.size() * sizeof(int64_t)));
+            if (p->trap[a]) {
+                std::vector<int64_t> vq(na * B), viq(na * B);
+                for (int64_t b = 0; b < B; ++b) trap_fx(p, a, gam[3 * b + a], &vq[b * na], &viq[b * na]);
+                PLAN_TRY(upload_raw(p, &p->vq[a], vq.data(), vq.size() * sizeof(int64_t)));
+                PLAN_TRY(upload_raw(p, &p->viq[a], viq.data(), viq.size() * sizeof(int64_t)));
+            }
+            continue;
+        }
         PLAN_TRY(upload_cplx(p, &p->tw[a], tw));
         PLAN_TRY(upload_cplx(p, &p->kt[a], kt));
-        PLAN_TRY(upload_real(p, &p->ki[a], ki));
         if (p->trap[a]) {
             std::vector<double> vh(2 * na * B), vf(2 * na * B), vi(na * B);
             for (int64_t b = 0; b < B; ++b)
@@ -400,6 +547,12 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
     PLAN_TRY(dalloc(p, (void **)&p->out4, sizeof(double) * 4 * B));
     PLAN_TRY(dalloc(p, (void **)&p->err, sizeof(int)));
     PLAN_TRY(dalloc(p, (void **)&p->ones, sizeof(double) * B));
+    if (p->fxp()) {
+        std::vector<FxCoupling> gq(2 * B);
+        for (int64_t b = 0; b < B; ++b)
+            for (int full = 0; full < 2; ++full) gq[2 * b + full] = coupling_fx(gs[b], full ? p->dt : 0.5 * p->dt);
+        PLAN_TRY(upload_raw(p, &p->gq, gq.data(), gq.size() * sizeof(FxCoupling)));
+    }
 #undef PLAN_TRY
     p->gamma_host = gam;
     {
@@ -595,17 +748,22 @@ static PassArgs make_pass(const gpe_plan *p, int axis, const void *src, void *ds
     a.lines_total = batch * lpi;
     const int L = pass_lines_per_tile(p->prec, axis == 0, a.nax, p->tile_var[axis]);
     a.ntiles = (a.lines_total + L - 1) / L;
-    a.tw = p->tw[axis];
+    const bool fxp = p->fxp();
+    a.tw = p->prec == GPE_C128 ? p->twx[axis] : p->tw[axis];
     const bool h0 = o0 < p->ndim, h1 = o1 < p->ndim;
-    a.kt_ax = p->kt[axis];
-    a.kt_o0 = h0 ? p->kt[o0] : nullptr;
-    a.kt_o1 = h1 ? p->kt[o1] : nullptr;
-    a.ki_ax = p->ki[axis];
+    void *const *kt = fxp ? p->ktx : p->kt, *const *vi = fxp ? p->viq : p->vi;
+    a.kt_ax = kt[axis];
+    a.kt_o0 = h0 ? kt[o0] : nullptr;
+    a.kt_o1 = h1 ? kt[o1] : nullptr;
+    a.ki_ax = fxp ? p->kix[axis] : p->ki[axis];
+    a.kiq_e = p->kix_e[axis];
     a.ki_o0 = h0 ? p->ki[o0] : nullptr;
     a.ki_o1 = h1 ? p->ki[o1] : nullptr;
-    a.vi_ax = p->vi[axis];
-    a.vi_o0 = h0 ? p->vi[o0] : nullptr;
-    a.vi_o1 = h1 ? p->vi[o1] : nullptr;
+    a.vi_ax = vi[axis];
+    a.vi_o0 = h0 ? vi[o0] : nullptr;
+    a.vi_o1 = h1 ? vi[o1] : nullptr;
+    a.gq = p->gq;
+    a.lg_n = ilog2_64(p->N);
     a.vsamp = p->ndim >= 2 ? p->vsamp : nullptr;
     a.vsamp_diag = p->vsamp;
     a.g = p->g_dev;
@@ -640,7 +798,8 @@ static PassArgs make_pass(const gpe_plan *p, int axis, const void *src, void *ds
 // select the real-time trap tables for a nonlinear substep of length c*dt (c = 1/2 or 1)
 static void set_nreal(const gpe_plan *p, PassArgs &a, bool full)
 {
-    void *const *vt = full ? p->vf : p->vh;
+    void *const *vt = p->fxp() ? p->vq : full ? p->vf : p->vh;
+    a.vq_full = full ? 1 : 0;
     const int axis = a.axis;
     const int o0 = axis == 0 ? 1 : 0, o1 = axis == 2 ? 1 : 2;
     a.vt_ax = vt[axis];
@@ -773,7 +932,7 @@ static gpe_status trap_level(gpe_plan *p, void *const *dst, const double *gamma_
 {
     double gm[3] = {0, 0, 0};
     for (int a = 0; a < p->ndim; ++a) gm[a] = gamma_t[3 * lev + a];
-    cudaError_t e = launch_trap_level(p->prec == GPE_C64 ? 0 : 1, dst, p->ndim, p->n, p->lo, p->h, gm, c * p->dt,
+    cudaError_t e = launch_trap_level(p->fxp() ? 2 : p->prec == GPE_C64 ? 0 : 1, dst, p->ndim, p->n, p->lo, p->h, gm, c * p->dt,
                                       p->batch, p->st);
     if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("trap tables: ") + cudaGetErrorString(e));
     return GPE_OK;
@@ -889,7 +1048,8 @@ static gpe_status step_real_dev(gpe_plan *p, void *psi, int64_t nsteps, const do
         x.op_mid = OP_NREAL;
         set_nreal(p, x, !last);
         if (gamma_t) {
-            GPE_TRY(trap_level(p, p->sched, gamma_t, s + 1, last ? 0.5 : 1.0));
+            // (fixed-point tables hold the half step's angles; the sweep doubles them)
+            GPE_TRY(trap_level(p, p->sched, gamma_t, s + 1, last || p->fxp() ? 0.5 : 1.0));
             use_sched(p, x);
         }
         x.dphi = phi;
@@ -914,7 +1074,7 @@ extern "C" gpe_status gpe_step_real_trap(gpe_plan *p, void *psi, int64_t nsteps,
         if (!isfinite(gamma_host[i])) return fail(GPE_EINVAL, "trap frequencies must be finite");
     DeviceGuard dg(p->device);
     if (!dg.ok) return fail(GPE_ECUDA, "cannot select the plan's device");
-    const size_t ce = p->prec == GPE_C64 ? sizeof(float4) : sizeof(double2);
+    const size_t ce = p->fxp() ? sizeof(int64_t) : p->prec == GPE_C64 ? sizeof(float4) : sizeof(double2);
     for (int a = 0; a < p->ndim; ++a)
         if (!p->sched[a]) GPE_TRY(dalloc(p, &p->sched[a], ce * (size_t)p->n[a] * (size_t)p->batch));
     if (p->ndim == 1 && !p->sched_last) GPE_TRY(dalloc(p, &p->sched_last, ce * (size_t)p->n[0] * (size_t)p->batch));
@@ -1708,9 +1868,24 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
     double gm[3] = {0, 0, 0};
     for (int a = 0; a < p->ndim; ++a) gm[a] = gamma[a];
     GPE_CUDA(cudaMemcpyAsync(p->gamma_dev + 3 * slot, gm, sizeof(gm), cudaMemcpyHostToDevice, p->st));
+    if (p->fxp()) {
+        FxCoupling gq[2];
+        for (int full = 0; full < 2; ++full) gq[full] = coupling_fx(g, full ? p->dt : 0.5 * p->dt);
+        GPE_CUDA(cudaMemcpyAsync((FxCoupling *)p->gq + 2 * slot, gq, sizeof(gq), cudaMemcpyHostToDevice, p->st));
+        GPE_CUDA(cudaStreamSynchronize(p->st));        // host staging goes out of scope
+    }
     for (int a = 0; a < p->ndim; ++a) {
         if (!p->trap[a]) continue;
         const int64_t na = p->n[a];
+        if (p->fxp()) {
+            std::vector<int64_t> vq(na), viq(na);
+            trap_fx(p, a, gm[a], vq.data(), viq.data());
+            const size_t len = (size_t)na * sizeof(int64_t);
+            GPE_CUDA(cudaMemcpyAsync((int64_t *)p->vq[a] + slot * na, vq.data(), len, cudaMemcpyHostToDevice, p->st));
+            GPE_CUDA(cudaMemcpyAsync((int64_t *)p->viq[a] + slot * na, viq.data(), len, cudaMemcpyHostToDevice, p->st));
+            GPE_CUDA(cudaStreamSynchronize(p->st));
+            continue;
+        }
         std::vector<double> vh(2 * na), vf(2 * na), vi(na);
         trap_tables_host(p, a, gm[a], vh.data(), vf.data(), vi.data());
         std::vector<unsigned char> bh, bf;

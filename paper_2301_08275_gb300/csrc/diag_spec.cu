@@ -393,6 +393,10 @@ __global__ void k_trap_level(int prec, void *t0, void *t1, void *t2, int ndim, i
         const double x = (a == 0 ? lo0 : (a == 1 ? lo1 : lo2)) + (double)j * (a == 0 ? h0 : (a == 1 ? h1 : h2));
         const double gm = a == 0 ? g0 : (a == 1 ? g1 : g2);
         const double th = 0.5 * gm * gm * x * x * c;
+        if (prec == 2) {
+            static_cast<long long *>(a == 0 ? t0 : (a == 1 ? t1 : t2))[b * na + j] = fx_turns(th / 6.283185307179586477);
+            continue;
+        }
         const double sh = sin(0.5 * th);
         const double wx = -2.0 * sh * sh, wy = -sin(th);
         void *t = a == 0 ? t0 : (a == 1 ? t1 : t2);

@@ -34,12 +34,15 @@
 #include <stdint.h>
 #include <string.h>
 
+#include "fx.cuh"
+
 namespace gpe {
 
 // ---------------------------------------------------------------- complex
 template <typename R> struct CT;
 template <> struct CT<float> { using C = float2; };
 template <> struct CT<double> { using C = double2; };
+template <> struct CT<fx> { using C = fx2; };
 
 __device__ __forceinline__ float2 mk(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
@@ -75,6 +78,7 @@ template <typename C> __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x
 template <typename R> struct UT;
 template <> struct UT<float> { using U = float4; };
 template <> struct UT<double> { using U = double2; };
+template <> struct UT<fx> { using U = int4; };
 
 // v * u for a unit factor u (conj(u) when CONJ), rounding only the result
 template <bool CONJ = false> __device__ __forceinline__ float2 umul(float2 v, float4 u)
@@ -89,6 +93,11 @@ template <bool CONJ = false> __device__ __forceinline__ double2 umul(double2 v, 
     const double uy = CONJ ? -u.y : u.y;
     return mk(fma(v.x, u.x, -v.y * uy), fma(v.x, uy, v.y * u.x));
 }
+
+// what a butterfly's first input (twiddle 1) gets in place of umul: fixed-point
+// twiddles carry a scale (fx.cuh), floating ones none
+__device__ __forceinline__ float2 tw_first(float2 v) { return v; }
+__device__ __forceinline__ double2 tw_first(double2 v) { return v; }
 
 // v * (1 + w) for a unit factor close to one, stored as its offset w: the
 // small product v*w is formed first and v is added last, so each component is
@@ -177,6 +186,7 @@ template <int M, int DIR, typename C> __device__ __forceinline__ C twc(C a, int 
         const R sy = ((idx == 4 || idx == 12) ? (R)1 : (R)-1) * (R)DIR;
         return mk(mul_rsqrt2(cx * a.x - sy * a.y), mul_rsqrt2(sy * a.x + cx * a.y));
     }
+    if constexpr (M > 8) {
     // angle 2 pi idx / 32 = q pi/2 + j pi/16 with j in 1..3 (first quadrant
     // reference angle j or 8 - j)
     const int q = idx >> 3, j = idx & 7;          // j in {1,2,3,5,6,7}
@@ -192,6 +202,9 @@ template <int M, int DIR, typename C> __device__ __forceinline__ C twc(C a, int 
     if (jj == 1) return cconst_mul<1>(a, swap_cs, sgn_c, sgn_s);
     if (jj == 2) return cconst_mul<2>(a, swap_cs, sgn_c, sgn_s);
     return cconst_mul<3>(a, swap_cs, sgn_c, sgn_s);
+    } else {
+        return a;      // M <= 8 has no other angle
+    }
 }
 
 // one radix-2 step of the M-point DFT: lo = e + W^k o, hi = e - W^k o with
@@ -578,6 +591,8 @@ template <typename R, int N, int L, int LPT, bool SW = false, int EPT = 0, bool 
 #pragma unroll
                     for (int ln = 0; ln < LPT; ++ln) x[ln][m] = umul<(DIR > 0)>(x[ln][m], w);
                 }
+#pragma unroll
+                for (int ln = 0; ln < LPT; ++ln) x[ln][0] = tw_first(x[ln][0]);
             }
 #pragma unroll
             for (int ln = 0; ln < LPT; ++ln) Dft<r, DIR, C>::run(x[ln]);
@@ -643,5 +658,29 @@ __device__ __forceinline__ void sweep_transforms(typename T::C (&v)[T::LPT_][T::
         if (h == 0) mid();
     }
 }
+
+// Bits of growth of a transform of a pass plan relative to |x|_2, times two:
+// after pass p the values are at most sqrt(points so far) |x|_2 / 4^p.
+template <typename PL, int LG> struct FxGrowth {
+    __host__ __device__ static constexpr int lg_to(int p)
+    {
+        int n = 1;
+        for (int i = 0; i <= p; ++i) n *= PL::radix(i);
+        return ilog2c(n);
+    }
+    __host__ __device__ static constexpr int peak2()
+    {
+        int m = 0;
+        for (int p = 0; p < PL::P; ++p) {
+            const int g = lg_to(p) - 4 * p;
+            m = g > m ? g : m;
+        }
+        return m;
+    }
+    static constexpr int DROP = 2 * (PL::P - 1);          // bits the twiddles of one transform divide by
+    static constexpr int END2 = LG - 2 * DROP;            // growth at the end, times two
+    // two transforms with a unit factor between them that keeps the scale
+    static constexpr int BITS = ((peak2() > END2 + peak2() ? peak2() : END2 + peak2()) + 1) / 2;
+};
 
 }  // namespace gpe

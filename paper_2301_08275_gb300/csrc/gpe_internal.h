@@ -57,6 +57,14 @@ struct PassArgs {
     // substeps, vsamp_diag the potential energy (both set for 2D/3D; 1D steps
     // take the same values through the trap tables, so only vsamp_diag is set)
     const void *vsamp, *vsamp_diag;
+    // complex128 sweeps run in fixed point (fx.cuh) and take their tables in
+    // that form: tw and kt_* as 62-bit unit factors (int4), vt_* the half-step
+    // trap angles in 2^-64 turns (int64; the full step doubles them, vq_full),
+    // vi_* the half-step trap exponents V_a c log2(e) to 53 fraction bits
+    // (int64), ki_ax exp(-k^2 dt/2) 2^-kiq_e to 62 bits (int64; ki_o0 and ki_o1
+    // stay double), gq the nonlinear coupling ([batch][half, full])
+    const void *gq;
+    int vq_full, kiq_e, lg_n;      // lg_n: log2 of the points of an instance
     const double *g;       // per-instance interaction
     double nl_c;           // theta = g * nl_c * |psi|^2
     // per-step phase dither of the complex64 real-time step: the kinetic
@@ -164,7 +172,7 @@ cudaError_t launch_line1d_cluster(const Line1DArgs &a, cudaStream_t st);
 // trap tables of one time level of a time-dependent harmonic trap (diag_spec.cu):
 // for every axis a < ndim and every instance, tab[a][b*n[a] + j] = exp(-i V_a c) - 1
 // with V_a = gamma[a]^2 x_j^2 / 2, x_j = lo[a] + j h[a] (float4 hi/lo pairs for
-// prec 0, double2 for prec 1)
+// prec 0, double2 for prec 1), or the angles V_a c in 2^-64 turns (int64) for prec 2
 cudaError_t launch_trap_level(int prec, void *const *tab, int ndim, const int64_t *n, const double *lo,
                               const double *h, const double *gamma, double c, int64_t batch, cudaStream_t st);
 

@@ -61,13 +61,14 @@ __global__ void k_noalloc_twiddles_f(float4 *tw, int n)
     const float hx = (float)c, hy = (float)(-s);
     tw[t] = make_float4(hx, hy, (float)(c - (double)hx), (float)(-s - (double)hy));
 }
-__global__ void k_noalloc_twiddles_d(double2 *tw, int n)
+// complex128 sweeps take 62-bit unit factors (fx.cuh)
+__global__ void k_noalloc_twiddles_d(int4 *tw, int n)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     double s, c;
     sincospi(2.0 * (double)t / (double)n, &s, &c);
-    tw[t] = make_double2(c, -s);
+    tw[t] = fx_pack(llrint(ldexp(c, 62)), -llrint(ldexp(s, 62)));
 }
 
 __global__ void k_noalloc_params(double *p, double g, double g0, double g1, double g2)
@@ -193,7 +194,7 @@ extern "C" gpe_status gpe_norm_energy_noalloc(const gpe_plan_desc *d, const void
             k_noalloc_twiddles_f<<<nb, 128, 0, st>>>(reinterpret_cast<float4 *>(base + kTwOff) + (size_t)a * kMaxN,
                                                      (int)n[a]);
         else
-            k_noalloc_twiddles_d<<<nb, 128, 0, st>>>(reinterpret_cast<double2 *>(base + kTwOff) + (size_t)a * kMaxN,
+            k_noalloc_twiddles_d<<<nb, 128, 0, st>>>(reinterpret_cast<int4 *>(base + kTwOff) + (size_t)a * kMaxN,
                                                      (int)n[a]);
         NA_CUDA(cudaGetLastError());
     }

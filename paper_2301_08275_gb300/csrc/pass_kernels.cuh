@@ -540,13 +540,19 @@ template <typename R, int N, bool ROWS, int VAR>
 using PassTile = GTile<R, N, pick_lines<R, N, ROWS, VAR>(), lines_per_thread<R>(), pass_swizzle<R, N, ROWS, VAR>(),
                        pass_points_per_thread<R, N, ROWS>(), pass_pad<R, N, ROWS>()>;
 
+// complex128 sweeps: the same tile with fixed-point values (fx.cuh)
+template <int N, bool ROWS, int VAR>
+using PassTileFx = GTile<fx, N, pick_lines<double, N, ROWS, VAR>(), 1, pass_swizzle<double, N, ROWS, VAR>(),
+                         pass_points_per_thread<double, N, ROWS>(), pass_pad<double, N, ROWS>()>;
+
 // dynamic shared memory of one CTA without the transform scratch: two staging
 // buffers, per-line reduction scratch, twiddles, two mbarriers
 template <typename R, int N, bool ROWS, int VAR> __host__ __device__ constexpr size_t pass_smem_base()
 {
     using T = PassTile<R, N, ROWS, VAR>;
     return 2 * sizeof(typename T::C) * T::BUF_POINTS + sizeof(double) * (size_t)(T::SMEM_POINTS / T::E) +
-           sizeof(typename T::U) * N + 2 * sizeof(uint64_t);
+           sizeof(typename T::U) * N + 2 * sizeof(uint64_t) +
+           (sizeof(R) == 8 ? 2 * sizeof(unsigned) * pick_lines<R, N, ROWS, VAR>() : 0);   // line scales
 }
 // CTAs per SM the registers are budgeted for: 4 per SM for split rows (1024 /
 // threads per CTA, at most 16), else 2 (1 for CTAs of more than 512 threads),
@@ -577,6 +583,164 @@ template <typename R, int N, bool ROWS, int VAR> __host__ __device__ constexpr s
     using T = PassTile<R, N, ROWS, VAR>;
     return pass_smem_base<R, N, ROWS, VAR>() +
            (pass_ping<R, N, ROWS, VAR>() ? sizeof(typename T::C) * T::BUF_POINTS : 0);
+}
+
+// ------------------------------------------------------------------ complex128 in fixed point
+// The complex128 sweeps transform and turn their lines in 64-bit fixed point
+// (fx.cuh): FP64 arithmetic bounded them at 0.4 of the FP64 rate, integer
+// multiply-adds run 32 times faster.  There is no FP64 variant beside them:
+// every grid, option and substep goes through here.
+//
+// nonlinear substep (real time) on a line held as v 2^q: the interaction's
+// angle and the trap's are added in turns and applied as one rotation
+template <int E, int TPL>
+__device__ __forceinline__ void fx_nreal(fx2 (&v)[E], int q, const PassArgs &a, const LineGeom &g, int tl)
+{
+    const FxCoupling *gq = static_cast<const FxCoupling *>(a.gq) + 2 * g.ti + a.vq_full;
+    const long long gm = gq->m;
+    const Limbs m = limbs(gm);
+    const bool neg = gq->neg != 0;
+    const int sh = 62 + 54 + gq->e + q;
+    const long long *vax = static_cast<const long long *>(a.vt_ax);
+    const long long *v0 = static_cast<const long long *>(a.vt_o0), *v1 = static_cast<const long long *>(a.vt_o1);
+    const double *vs = static_cast<const double *>(a.vsamp);
+    long long line = 0;
+    if (v0) line += v0[(int64_t)g.ti * a.o0n + g.c0];
+    if (v1) line += v1[(int64_t)g.ti * a.o1n + g.c1];
+    const double cs = a.nl_c * 0.15915494309189533577;      // per turn
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        long long t;
+        if (gm == 0) t = 0;
+        else if (sh <= 0) {
+            t = fx_angle(v[e], m, sh);
+            if (neg) t = -t;
+        } else {
+            // angles that may pass a turn: in FP64, reduced there
+            const double x = fx_to(v[e].x, q), y = fx_to(v[e].y, q);
+            t = fx_turns(a.g[g.ti] * cs * (x * x + y * y));
+        }
+        long long w = line;
+        if (vax) w += vax[(int64_t)g.ti * a.nax + tl + TPL * e];
+        t += (long long)((unsigned long long)w << a.vq_full);
+        if (vs) t += fx_turns(cs * vs[g.off + (int64_t)(tl + TPL * e) * a.estride]);
+        v[e] = fx_rotate(v[e], t);
+    }
+}
+
+// nonlinear substep (imaginary time) on the line's doubles: the exponents of
+// interaction and trap are added to 53 fraction bits; s scales the values first
+template <int E, int TPL>
+__device__ __forceinline__ void fx_nimag(double2 (&d)[E], double s, const PassArgs &a, const LineGeom &g, int tl)
+{
+    const long long *vax = static_cast<const long long *>(a.vi_ax);
+    const long long *v0 = static_cast<const long long *>(a.vi_o0), *v1 = static_cast<const long long *>(a.vi_o1);
+    const double *vs = static_cast<const double *>(a.vsamp);
+    long long line = 0;
+    if (v0) line += v0[(int64_t)g.ti * a.o0n + g.c0];
+    if (v1) line += v1[(int64_t)g.ti * a.o1n + g.c1];
+    const double cl = a.nl_c * 1.4426950408889634074;
+    const double gc = a.g[g.ti] * cl * (s * s);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        double x = gc * (d[e].x * d[e].x + d[e].y * d[e].y);
+        if (vs) x += cl * vs[g.off + (int64_t)(tl + TPL * e) * a.estride];
+        // beyond 2^+-300 the factor is what it is there
+        const int hx = __double2hiint(x);
+        if ((hx & 0x7fffffff) > 0x4072c000) x = hx < 0 ? -300.0 : 300.0;
+        long long ex = fx_from(x, -53) + line;
+        if (vax) ex += vax[(int64_t)g.ti * a.nax + tl + TPL * e];
+        const double f = s * fx_exp2m(ex);
+        d[e] = mk(d[e].x * f, d[e].y * f);
+    }
+}
+
+// One sweep of a line: substep, transform, substep, transform (see SweepProg),
+// on doubles in and out.  Scaling exponents: q falls by the bits that the
+// twiddles divide by, the kinetic substep carries the 1/N of the inverse.
+template <int N, bool ROWS, int VAR, bool PING>
+__device__ __forceinline__ void fx_sweep(double2 (&d)[PassTileFx<N, ROWS, VAR>::E], const PassArgs &a,
+                                         const LineGeom &g, double2 *sm, double2 *ss, int tl, int l, const double2 *tw,
+                                         unsigned *lsc, int op_pre, int fft1, int op_mid, int fft2)
+{
+    using T = PassTileFx<N, ROWS, VAR>;
+    using G = FxGrowth<typename T::PL, ilog2c(N)>;
+    constexpr int E = T::E, TPL = T::TPL, L = T::NP;
+    if (op_pre == OP_SCALE || op_pre == OP_SCALE_NIMAG) {
+        const double s = a.scale[g.inst];
+        if (op_pre == OP_SCALE_NIMAG) {
+            fx_nimag<E, TPL>(d, s, a, g, tl);
+        } else {
+#pragma unroll
+            for (int e = 0; e < E; ++e) d[e] = mk(d[e].x * s, d[e].y * s);
+        }
+    }
+    if (fft1 == 0) return;
+    const LineScale ls = line_scale<L, T::NT, E>(d, lsc, lsc + L, l, G::BITS);
+    int q = ls.q;
+    fx2 v[1][E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[0][e] = mk(fx_from(d[e].x, q), fx_from(d[e].y, q));
+    if (op_pre == OP_NREAL) fx_nreal<E, TPL>(v[0], q, a, g, tl);
+    sweep_transforms<T, PING>(v, reinterpret_cast<fx2 *>(sm), reinterpret_cast<fx2 *>(ss), tl, l,
+                              reinterpret_cast<const int4 *>(tw), fft1, fft2, [&]() {
+        q += G::DROP;
+        if (op_mid == OP_NREAL) {
+            fx_nreal<E, TPL>(v[0], q, a, g, tl);
+        } else if (op_mid == OP_KREAL) {
+            const int4 *kt = static_cast<const int4 *>(a.kt_ax);
+            const int4 *k0 = static_cast<const int4 *>(a.kt_o0), *k1 = static_cast<const int4 *>(a.kt_o1);
+            int4 fl = k0[g.c0];
+            if (k1) fl = fx_unit(fx_mul<2>(fx_value(fl), k1[g.c1]));
+            const fx2 flv = fx_value(fl);
+#pragma unroll
+            for (int e = 0; e < E; ++e) v[0][e] = fx_mul<2>(v[0][e], fx_unit(fx_mul<2>(flv, kt[tl + TPL * e])));
+            q -= a.lg_n;
+        } else if (op_mid == OP_KIMAG) {
+            const long long *ki = static_cast<const long long *>(a.ki_ax);
+            double f = static_cast<const double *>(a.ki_o0)[g.c0];
+            if (a.ki_o1) f *= static_cast<const double *>(a.ki_o1)[g.c1];
+            // f = fm 2^fe, fm of 62 bits
+            const int fe = max(((__double2hiint(f) >> 20) & 0x7ff) - 1023 - 61, -1021);
+            const Limbs fm = limbs(fx_from(f, fe));
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const Limbs w = limbs(fx_mulr<2>(ki[tl + TPL * e], fm));
+                v[0][e] = mk(fx_mulr<2>(v[0][e].x, w), fx_mulr<2>(v[0][e].y, w));
+            }
+            q += fe + 62 + a.kiq_e - ilog2c(N);
+        }
+    });
+    if (fft2) q += G::DROP;
+    if (q < -1021 || q > 950 || ls.bad) {
+        // values below the range of doubles are zero; an infinity or a NaN anywhere in a line fills it
+        const double x = ls.bad || q > 950 ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) d[e] = mk(x, x);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) d[e] = mk(fx_to(v[0][e].x, q), fx_to(v[0][e].y, q));
+    }
+    if (op_mid == OP_NIMAG) fx_nimag<E, TPL>(d, 1.0, a, g, tl);
+}
+// forward transform of a line alone (diagnostics)
+template <int N, bool ROWS, int VAR, bool PING>
+__device__ __forceinline__ void fx_forward(double2 (&d)[PassTileFx<N, ROWS, VAR>::E], double2 *sm, double2 *ss, int tl,
+                                           int l, const double2 *tw, unsigned *lsc)
+{
+    using T = PassTileFx<N, ROWS, VAR>;
+    using G = FxGrowth<typename T::PL, ilog2c(N)>;
+    constexpr int E = T::E;
+    const LineScale ls = line_scale<T::NP, T::NT, E>(d, lsc, lsc + T::NP, l, G::BITS);
+    fx2 v[1][E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[0][e] = mk(fx_from(d[e].x, ls.q), fx_from(d[e].y, ls.q));
+    T::template fft<-1, PING>(v, reinterpret_cast<fx2 *>(sm), reinterpret_cast<fx2 *>(ss), tl, l,
+                              reinterpret_cast<const int4 *>(tw));
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        d[e] = ls.bad ? mk(__longlong_as_double(0x7ff8000000000000ll), 0.0)
+                      : mk(fx_to(v[0][e].x, ls.q + G::DROP), fx_to(v[0][e].y, ls.q + G::DROP));
 }
 
 // Sweep programs compiled with their slots fixed: the passes of the real- and
@@ -639,7 +803,13 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
     U *tw = reinterpret_cast<U *>(smraw + tiles_bytes + sizeof(double) * N * L / E);
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smraw + tiles_bytes + sizeof(double) * N * L / E + sizeof(U) * N);
     const int t = threadIdx.x, l0 = (t % T::NP) * LPT, tl = t / T::NP;
-    T::load_twiddles(tw, static_cast<const U *>(a.tw), t, T::NT);
+    unsigned *const lsc = reinterpret_cast<unsigned *>(mbar + 2);    // line scales (complex128)
+    if constexpr (sizeof(R) == 8) {
+        using F = PassTileFx<N, ROWS, VAR>;
+        F::load_twiddles(reinterpret_cast<int4 *>(tw), static_cast<const int4 *>(a.tw), t, T::NT);
+    } else {
+        T::load_twiddles(tw, static_cast<const U *>(a.tw), t, T::NT);
+    }
 
     // Strided tiles (point i of line l at i*L + l, the layout of a box of L
     // lines by tma_box points) can be fetched by the copy engine: thread 0
@@ -707,6 +877,10 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
     bool aborted = false;
     for (; tile < a.ntiles; ++it, tile += gridDim.x) {
         C *sm = (it & 1) ? buf1 : buf0;
+        if constexpr (sizeof(R) == 8) {
+            if (t < 2 * L) lsc[t] = 0;       // published by the barrier that follows
+            if (T::NT < 2 * L && t + T::NT < 2 * L) lsc[t + T::NT] = 0;
+        }
         if (tma) {
             // this tile's boxes have landed (the next tile's may still fly)
             const bool ok = mbar_wait_bounded(&mbar[it & 1], (unsigned)(it >> 1) & 1u);
@@ -756,7 +930,10 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
 #pragma unroll
             for (int ln = 0; ln < LPT; ++ln) sk[ln] = (R)0;
             if (rmode == RED_DIAG_X) {
-                T::template fft<-1, PING>(v, sm, PING ? scr : sm, tl, l0, tw);
+                if constexpr (sizeof(R) == 8)
+                    fx_forward<N, ROWS, VAR, PING>(v[0], sm, PING ? scr : sm, tl, l0, tw, lsc);
+                else
+                    T::template fft<-1, PING>(v, sm, PING ? scr : sm, tl, l0, tw);
                 const R kf = (R)a.kf[0];
 #pragma unroll
                 for (int ln = 0; ln < LPT; ++ln) {
@@ -845,7 +1022,10 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
                 }
             }
         } else if (rmode == RED_DIAG_K) {
-            T::template fft<-1, PING>(v, sm, PING ? scr : sm, tl, l0, tw);
+            if constexpr (sizeof(R) == 8)
+                fx_forward<N, ROWS, VAR, PING>(v[0], sm, PING ? scr : sm, tl, l0, tw, lsc);
+            else
+                T::template fft<-1, PING>(v, sm, PING ? scr : sm, tl, l0, tw);
             const R kf = (R)a.kf[a.axis];
             R acc[LPT];
 #pragma unroll
@@ -875,17 +1055,22 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
             for (int ln = 0; ln < LPT; ++ln)
                 if (tl == 0 && g[ln].valid) a.partials[(int64_t)(6 + a.axis) * a.lines_cap + g[ln].lg] = sk[ln];
         } else {
-#pragma unroll
-            for (int ln = 0; ln < LPT; ++ln)
-                point_op<R, E, TPL>(op_pre, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
-            sweep_transforms<T, PING>(v, sm, PING ? scr : sm, tl, l0, tw, fft1, fft2, [&]() {
+            if constexpr (sizeof(R) == 8) {
+                fx_sweep<N, ROWS, VAR, PING>(v[0], a, g[0], sm, PING ? scr : sm, tl, l0, tw, lsc, op_pre, fft1, op_mid,
+                                             fft2);
+            } else {
 #pragma unroll
                 for (int ln = 0; ln < LPT; ++ln)
-                    point_op<R, E, TPL>(op_mid, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
-            });
+                    point_op<R, E, TPL>(op_pre, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
+                sweep_transforms<T, PING>(v, sm, PING ? scr : sm, tl, l0, tw, fft1, fft2, [&]() {
 #pragma unroll
-            for (int ln = 0; ln < LPT; ++ln)
-                point_op<R, E, TPL>(op_post, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
+                    for (int ln = 0; ln < LPT; ++ln)
+                        point_op<R, E, TPL>(op_mid, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
+                });
+#pragma unroll
+                for (int ln = 0; ln < LPT; ++ln)
+                    point_op<R, E, TPL>(op_post, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
+            }
             if (rmode == RED_NORM) {
                 if constexpr (sizeof(R) == 4) {
                     float nh[LPT], nl[LPT];
