@@ -111,8 +111,6 @@ struct gpe_plan {
     size_t pin_len = 0;
     void *work[4] = {};
     double *hist = nullptr, *spec_out = nullptr;
-    int hist_blocks = 0;
-    int64_t nshells = 0;
     void *host_buf = nullptr;    // device copy for gpe_step_real_host
     // slab pipeline of gpe_step_real_host: a copy stream and one event per slab and direction
     cudaStream_t copy_st = nullptr;
@@ -1757,14 +1755,16 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
     if (!p->work[0]) {
         for (int w = 0; w <= p->ndim; ++w) GPE_TRY(dalloc(p, &p->work[w], field));
     }
-    const int nb = bin_blocks(sa);
-    if (!p->hist || p->nshells < ns || p->hist_blocks < nb) {
-        // block histograms, then the fixed-point total partials and scale
-        GPE_TRY(dalloc(p, (void **)&p->hist, sizeof(double) * (2 * (size_t)ns * nb + nb + 1)));
+    for (int a = 0; a < 3; ++a) sa.lg[a] = ilog2_64(p->n[a]);
+    sa.cubic = 1;
+    for (int a = 0; a < p->ndim; ++a) sa.cubic = sa.cubic && sa.lratio[a] == 1.0;
+    const int nv = velocity_blocks(sa);
+    if (!p->hist) {
+        // histogram and scale, then the partial sums of every component
+        GPE_TRY(dalloc(p, (void **)&p->hist, sizeof(double) * (2 * (size_t)ns + 1 + 3 * (size_t)nv)));
         GPE_TRY(dalloc(p, (void **)&p->spec_out, sizeof(double) * 2 * (size_t)ns));
-        p->nshells = ns;
-        p->hist_blocks = nb;
     }
+    double *const partial = p->hist + 2 * ns + 1;
     // output slot of each kind: requested kinds in bit order
     double *slot[4] = {nullptr, nullptr, nullptr, nullptr};
     std::vector<double> tmp(2 * ns);
@@ -1773,10 +1773,7 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
         SpecArgs sb = sa;
         sb.split = split;
         sb.ncomp = ncomp;
-        double *aux = p->hist + 2 * (size_t)ns * nb;
-        cudaError_t e = launch_bin(sb, uh, ns, p->hist, nb, aux, p->st);
-        if (e == cudaSuccess)
-            e = launch_hist_reduce(p->hist, nb, ns, p->dv / (double)p->N, aux, p->spec_out, p->spec_out + ns,
+        cudaError_t e = launch_bin(sb, uh, ns, partial, ncomp * nv, p->hist, 0.5 * p->dv / (double)p->N, p->spec_out,
                                    p->st);
         if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
         GPE_CUDA(cudaMemcpyAsync(tmp.data(), p->spec_out, sizeof(double) * 2 * ns, cudaMemcpyDeviceToHost, p->st));
@@ -1795,7 +1792,7 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
             cudaError_t e = launch_deriv(sa, p->work[0], p->work[1 + a], a, p->st);
             if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
             GPE_TRY(fft_nd(p, p->work[1 + a], p->work[1 + a], +1));
-            e = launch_velocity(sv, pb, p->work[1 + a], p->st);
+            e = launch_velocity(sv, pb, p->work[1 + a], partial + (size_t)a * nv, p->st);
             if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
             GPE_TRY(fft_nd(p, p->work[1 + a], p->work[1 + a], -1));
         }
@@ -1813,6 +1810,10 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
         if (slot[3]) {
             // the bins carry 1/2 dV/N; the number spectrum has no 1/2
             void *ph[3] = {p->work[0], nullptr, nullptr};
+            SpecArgs sn = sa;
+            sn.part = 2;
+            cudaError_t e = launch_velocity(sn, pb, nullptr, partial, p->st);
+            if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
             GPE_TRY(bin_out(ph, 0, 1, 2.0, slot[3], nullptr));
         }
         if (slot[0] || slot[1]) {

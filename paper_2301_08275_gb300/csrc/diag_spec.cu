@@ -183,11 +183,11 @@ cudaError_t launch_finish_diag(const double *sums, int64_t batch, int ndim, cons
 }
 
 // ------------------------------------------------------------------ spectra
-__device__ __forceinline__ int64_t axis_index(int64_t i, const SpecArgs &s, int axis)
+// coordinate of point i on an axis (all extents are powers of two)
+__device__ __forceinline__ int axis_index(int64_t i, const SpecArgs &s, int axis)
 {
-    int64_t stride = 1;
-    for (int a = 0; a < axis; ++a) stride *= s.n[a];
-    return (i / stride) % s.n[axis];
+    const int sh = axis == 0 ? 0 : axis == 1 ? s.lg[0] : s.lg[0] + s.lg[1];
+    return (int)(i >> sh) & ((1 << s.lg[axis]) - 1);
 }
 
 // dst = i k_axis src, with the Nyquist mode of i k_axis set to zero.
@@ -196,144 +196,280 @@ __global__ void k_deriv(const SpecArgs s, const typename CT<R>::C *__restrict__ 
                         int axis)
 {
     using C = typename CT<R>::C;
-    const int64_t na = s.n[axis];
+    const int na = 1 << s.lg[axis];
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = axis_index(i, s, axis);
+        const int j = axis_index(i, s, axis);
         const R k = (2 * j == na) ? (R)0 : (R)(s.kf[axis] * (double)(j < na / 2 ? j : j - na));
         const C v = src[i];
         dst[i] = mk(-k * v.y, k * v.x);
     }
 }
 
+// sum of one double per thread of a 256-thread block, in a fixed order; thread 0 has it
+__device__ __forceinline__ double block_sum(double s, double *sh)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    return ((sh[0] + sh[1]) + (sh[2] + sh[3])) + ((sh[4] + sh[5]) + (sh[6] + sh[7]));
+}
+
 // w <- u = Im(conj(psi) * w / N) / |psi| (part 0) or Re(...) / |psi| (part 1: the
-// gradient of |psi|), 0 where |psi|^2 < 1e-30, stored as (u, 0).
+// gradient of |psi|), 0 where |psi|^2 < 1e-30, stored as (u, 0); part 2 leaves w
+// alone and takes |psi|.  partial[block] = sum of the squares, which fixes the
+// scale of the shell sums (below): a few per mille suffice, so single
+// precision adds them, and double precision where those leave its range.
 template <typename R>
-__global__ void k_velocity(const SpecArgs s, const typename CT<R>::C *__restrict__ psi, typename CT<R>::C *__restrict__ w)
+__global__ void __launch_bounds__(256) k_velocity(const SpecArgs s, const typename CT<R>::C *__restrict__ psi,
+                                                  typename CT<R>::C *__restrict__ w, double *__restrict__ partial)
 {
     using C = typename CT<R>::C;
+    __shared__ double sh[8];
     const R invn = (R)(1.0 / (double)s.N);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.N; i += (int64_t)gridDim.x * blockDim.x) {
+    auto value = [&](int64_t i) -> R {
         const C p = psi[i];
-        const C d = w[i];
         const R rho = p.x * p.x + p.y * p.y;
+        if (s.part == 2) return sqrt(rho);
+        const C d = w[i];
         R u = (R)0;
         if (rho >= (R)1e-30) u = (s.part ? (p.x * d.x + p.y * d.y) : (p.x * d.y - p.y * d.x)) * invn / sqrt(rho);
-        w[i] = mk(u, (R)0);
+        return u;
+    };
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    float acc = 0.0f;
+    for (int64_t i = first; i < s.N; i += step) {
+        const R u = value(i);
+        const float f = (float)u;
+        acc = fmaf(f, f, acc);
+        if (s.part != 2) w[i] = mk(u, (R)0);
     }
+    double t = (double)acc;
+    if (!(acc > 1e-30f && acc < 1e37f)) {
+        t = 0.0;
+        for (int64_t i = first; i < s.N; i += step) {
+            const double u = s.part == 2 ? (double)value(i) : (double)w[i].x;
+            t += u * u;
+        }
+    }
+    t = block_sum(t, sh);
+    if (threadIdx.x == 0) partial[blockIdx.x] = t;
 }
 
 // Shell histogram of |u_i|^2 and |u_c|^2 (split) or of sum_a |u_a|^2 (slot 0)
-// over the k grid, one partial histogram per block (hist[block][2][nshells]).
-// Shell sums are accumulated in 64-bit fixed point so that they do not depend
-// on the order in which threads add (integer addition is associative): a
-// deterministic pre-pass sums |u|^2 over the field in a fixed tree order,
-// the scale is the power of two that maps that total below 2^62, and every
-// point's contribution is rounded to an integer multiple of 1/scale before
-// the (integer) atomic additions.  Rounding costs at most total * 2^-63 per
-// point; the errors are of either sign and far below the FP64 sums' own.
-template <typename R>
-__global__ void k_field_total(const SpecArgs s, const typename CT<R>::C *__restrict__ u0,
-                              const typename CT<R>::C *__restrict__ u1, const typename CT<R>::C *__restrict__ u2,
-                              double *__restrict__ partial)
+// over the k grid.  Shell sums are accumulated in 64-bit fixed point so that
+// they do not depend on the order in which threads and blocks add (integer
+// addition is associative).  The scale is the power of two that maps the
+// field's total, N sum u^2 (Parseval, from k_velocity's partial sums), below
+// 2^61; rounding costs at most total * 2^-62 per point, of either sign.
+//
+// FP64 arithmetic bounded this kernel (about 100 FP64 operations a point with
+// three divisions: 202 us for a 1024^2 complex64 field), so
+//  * the parts come from |k x u|^2 / k^2 and |k . u|^2 / k^2, one division
+//    each, for any scale of k: q_a = m_a L_max / L_a in place of k_a;
+//  * complex64 fields take them in two-float arithmetic (error-free products
+//    and sums, 2^-44 relative; the fields themselves carry 2^-24);
+//  * shells of cubic boxes are exact integer tests, of other boxes a single
+//    precision root, in double only next to a shell's edge;
+//  * neighbouring lanes of one shell add through shuffles, the first of them
+//    adds to the block's histogram, and the blocks add theirs to one in global
+//    memory (no per-block copies to sum afterwards).
+// Spectra of a 1024^2 complex64 field, the whole call: 458 -> 219 us.
+struct Pf {
+    float h, l;
+};
+__device__ __forceinline__ Pf pf_norm(float h, float l)
 {
-    using C = typename CT<R>::C;
-    __shared__ double red[256];
-    const C *u[3] = {u0, u1, u2};
-    const int nc = s.split ? s.ndim : s.ncomp;
-    double acc = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.N; i += (int64_t)gridDim.x * blockDim.x)
-        for (int a = 0; a < nc; ++a) {
-            const C v = u[a][i];
-            acc += (double)v.x * (double)v.x + (double)v.y * (double)v.y;
-        }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
+    const float s = h + l;
+    return {s, l - (s - h)};
 }
-// fixed-order sum of the block partials; scale = 2^(61 - ceil(log2 total))
-__global__ void k_fixed_scale(double *aux, int nblocks)
+__device__ __forceinline__ Pf pf_add(Pf a, Pf b)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += aux[b];
+    const float s = a.h + b.h, v = s - a.h;
+    return pf_norm(s, ((a.h - (s - v)) + (b.h - v)) + (a.l + b.l));
+}
+__device__ __forceinline__ Pf pf_neg(Pf a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Pf pf_mul(Pf a, float b)
+{
+    const float p = a.h * b;
+    return {p, fmaf(a.h, b, -p) + a.l * b};
+}
+__device__ __forceinline__ Pf pf_sq(Pf a)
+{
+    const float p = a.h * a.h;
+    return pf_norm(p, fmaf(a.h, a.h, -p) + 2.0f * a.h * a.l);
+}
+__device__ __forceinline__ Pf pf_div(Pf a, Pf b)
+{
+    const float r = 1.0f / b.h, z = a.h * r;
+    return pf_norm(z, (fmaf(-z, b.h, a.h) + (a.l - z * b.l)) * r);
+}
+// the same operations on doubles, so that one kernel serves both precisions
+template <typename R> struct Wide;
+template <> struct Wide<float> {
+    using T = Pf;
+    __device__ static T make(double v) { return {(float)v, (float)(v - (double)(float)v)}; }
+    __device__ static T whole(float v) { return {v, 0.0f}; }
+    __device__ static T mul(T a, float b) { return pf_mul(a, b); }
+    __device__ static T add(T a, T b) { return pf_add(a, b); }
+    __device__ static T neg(T a) { return pf_neg(a); }
+    __device__ static T sq(T a) { return pf_sq(a); }
+    __device__ static T div(T a, T b) { return pf_div(a, b); }
+    __device__ static float hi(T a) { return a.h; }
+    // round(v 2^61), 0 <= v <= 1
+    __device__ static long long fixed(T a)
+    {
+        return __float2ll_rn(a.h * 2305843009213693952.0f) + __float2ll_rn(a.l * 2305843009213693952.0f);
+    }
+};
+template <> struct Wide<double> {
+    using T = double;
+    __device__ static T make(double v) { return v; }
+    __device__ static T whole(double v) { return v; }
+    __device__ static T mul(T a, double b) { return a * b; }
+    __device__ static T add(T a, T b) { return a + b; }
+    __device__ static T neg(T a) { return -a; }
+    __device__ static T sq(T a) { return a * a; }
+    __device__ static T div(T a, T b) { return a / b; }
+    __device__ static float hi(T a) { return (float)a; }
+    __device__ static long long fixed(T a) { return __double2ll_rn(a * 2305843009213693952.0); }
+};
+
+// power of two that scales the fields so that their squares sum to at most one
+__device__ __forceinline__ double field_scale(double total, int prec)
+{
+    if (!(total > 0.0) || !isfinite(total)) return 1.0;
     int ex = 0;
-    frexp(t > 0.0 ? t : 1.0, &ex);               // t < 2^ex
-    aux[nblocks] = ldexp(1.0, 61 - ex);
+    frexp(total * 1.002, &ex);
+    int h = (ex + 1) >> 1;                        // total < 2^ex <= 4^h
+    if (prec == 0) h = max(-126, min(126, h));
+    return ldexp(1.0, -h);
 }
 
 template <typename R>
-__global__ void k_bin(const SpecArgs s, const typename CT<R>::C *__restrict__ u0, const typename CT<R>::C *__restrict__ u1,
-                      const typename CT<R>::C *__restrict__ u2, int64_t nshells, const double *__restrict__ scale_p,
-                      unsigned long long *__restrict__ hist)
+__global__ void __launch_bounds__(256) k_bin(const SpecArgs s, const typename CT<R>::C *__restrict__ u0,
+                                             const typename CT<R>::C *__restrict__ u1,
+                                             const typename CT<R>::C *__restrict__ u2, int nshells,
+                                             const double *__restrict__ partial, int npartial,
+                                             unsigned long long *__restrict__ hist, double *__restrict__ scale_out)
 {
     using C = typename CT<R>::C;
+    using W = Wide<R>;
+    using T = typename W::T;
     extern __shared__ unsigned long long shq[];   // [2][nshells]
-    for (int64_t i = threadIdx.x; i < 2 * nshells; i += blockDim.x) shq[i] = 0ull;
+    __shared__ double shd[8], shs;
+    const int nsum = (s.split ? 2 : 1) * nshells;
+    for (int i = threadIdx.x; i < nsum; i += 256) shq[i] = 0ull;
+    double t = 0.0;
+    for (int i = threadIdx.x; i < npartial; i += 256) t += partial[i];
+    t = block_sum(t, shd);
+    if (threadIdx.x == 0) {
+        shs = field_scale(t * (double)s.N, s.prec);
+        // a field that is not finite has no spectrum
+        if (blockIdx.x == 0) *scale_out = isfinite(t) ? shs : __longlong_as_double(0x7ff8000000000000ll);
+    }
     __syncthreads();
-    const double scale = *scale_p;
-    auto fx = [scale](double v) { return (unsigned long long)(v * scale + 0.5); };
-    const C *u[3] = {u0, u1, u2};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.N; i += (int64_t)gridDim.x * blockDim.x) {
-        double kv[3] = {0.0, 0.0, 0.0}, q2 = 0.0, k2 = 0.0;
-        int64_t rem = i;
-        for (int a = 0; a < s.ndim; ++a) {
-            const int64_t j = rem % s.n[a];
-            rem /= s.n[a];
-            const int64_t m = j < s.n[a] / 2 ? j : j - s.n[a];
-            kv[a] = s.kf[a] * (double)m;
-            k2 += kv[a] * kv[a];
-            const double qa = (double)m * s.lratio[a];
-            q2 += qa * qa;
-        }
-        const int64_t sh_i = (int64_t)floor(sqrt(q2) + 0.5);
-        if (!s.split) {
-            double et = 0.0;
-            for (int a = 0; a < s.ncomp; ++a) {
-                const C v = u[a][i];
-                et += (double)v.x * (double)v.x + (double)v.y * (double)v.y;
+    const R sc = (R)shs;
+    const C *const u[3] = {u0, u1, u2};
+    const int lane = threadIdx.x & 31;
+    const T lr[3] = {W::make(s.lratio[0]), W::make(s.lratio[1]), W::make(s.lratio[2])};
+    // whole warps run every iteration (the shuffles below)
+    const int64_t step = (int64_t)gridDim.x * 256;
+    for (int64_t i0 = blockIdx.x * (int64_t)256 + (threadIdx.x & ~31); i0 < s.N; i0 += step) {
+        const int64_t i = i0 + lane;
+        const bool on = i < s.N;
+        long long ei = 0, ec = 0;
+        int shell = -1;
+        if (on) {
+            int m[3] = {0, 0, 0};
+            for (int a = 0; a < s.ndim; ++a) {
+                const int j = axis_index(i, s, a), na = 1 << s.lg[a];
+                m[a] = j < na / 2 ? j : j - na;
             }
-            atomicAdd(&shq[sh_i], fx(et));
-            continue;
+            T q[3], q2;
+            if (s.cubic) {
+                const int k2 = m[0] * m[0] + m[1] * m[1] + m[2] * m[2];
+                // floor(sqrt(k2) + 1/2) = n  <=>  n^2 - n < k2 <= n^2 + n (or n = 0 = k2)
+                int n = (int)(sqrtf((float)k2) + 0.5f);
+                if (n > 0 && k2 <= n * n - n) --n;
+                if (k2 > n * n + n) ++n;
+                shell = n;
+                q2 = W::whole((R)k2);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) q[a] = W::whole((R)m[a]);
+            } else {
+                q2 = W::whole((R)0);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    q[a] = W::mul(lr[a], (R)m[a]);
+                    q2 = W::add(q2, W::sq(q[a]));
+                }
+                const float r = sqrtf(W::hi(q2)) + 0.5f, tol = 1e-6f * r + 1e-6f;
+                shell = (int)r;
+                if (r - (float)shell < tol || (float)shell + 1.0f - r < tol) {
+                    double d2 = 0.0;
+                    for (int a = 0; a < s.ndim; ++a) {
+                        const double qa = (double)m[a] * s.lratio[a];
+                        d2 += qa * qa;
+                    }
+                    shell = (int)floor(sqrt(d2) + 0.5);
+                }
+            }
+            R re[3] = {(R)0, (R)0, (R)0}, im[3] = {(R)0, (R)0, (R)0};
+            const int nc = s.split ? s.ndim : s.ncomp;
+            for (int a = 0; a < nc; ++a) {
+                const C v = u[a][i];
+                re[a] = v.x * sc;
+                im[a] = v.y * sc;
+            }
+            if (!s.split || (m[0] | m[1] | m[2]) == 0) {
+                T e = W::whole((R)0);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) e = W::add(e, W::add(W::sq(W::whole(re[a])), W::sq(W::whole(im[a]))));
+                ei = W::fixed(e);
+            } else {
+                auto cross = [&](const R *v, int a, int b) { return W::add(W::mul(q[a], v[b]), W::neg(W::mul(q[b], v[a]))); };
+                auto dot = [&](const R *v) { return W::add(W::add(W::mul(q[0], v[0]), W::mul(q[1], v[1])), W::mul(q[2], v[2])); };
+                T in = W::add(W::sq(cross(re, 0, 1)), W::sq(cross(im, 0, 1)));
+                if (s.ndim > 2) {
+                    in = W::add(in, W::add(W::sq(cross(re, 0, 2)), W::sq(cross(im, 0, 2))));
+                    in = W::add(in, W::add(W::sq(cross(re, 1, 2)), W::sq(cross(im, 1, 2))));
+                }
+                ei = W::fixed(W::div(in, q2));
+                ec = W::fixed(W::div(W::add(W::sq(dot(re)), W::sq(dot(im))), q2));
+            }
         }
-        double ur[3] = {0, 0, 0}, ui[3] = {0, 0, 0}, kdr = 0.0, kdi = 0.0;
-        for (int a = 0; a < s.ndim; ++a) {
-            const C v = u[a][i];
-            ur[a] = (double)v.x;
-            ui[a] = (double)v.y;
-            kdr += kv[a] * ur[a];
-            kdi += kv[a] * ui[a];
+        // sums over runs of lanes with one shell; the first lane of a run adds them
+        const int up = __shfl_up_sync(0xffffffffu, shell, 1);
+        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || up != shell);
+        const unsigned later = lane == 31 ? 0u : heads >> (lane + 1);
+        const int run = later ? __ffs((int)later) : 32 - lane;       // lanes from here to the run's end
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long a = __shfl_down_sync(0xffffffffu, ei, o);
+            if (o < run) ei += a;
+            if (s.split) {
+                const long long c = __shfl_down_sync(0xffffffffu, ec, o);
+                if (o < run) ec += c;
+            }
         }
-        double ec = 0.0, ei = 0.0;
-        for (int a = 0; a < s.ndim; ++a) {
-            const double cr = k2 > 0.0 ? kv[a] * kdr / k2 : 0.0;
-            const double ci = k2 > 0.0 ? kv[a] * kdi / k2 : 0.0;
-            ec += cr * cr + ci * ci;
-            ei += (ur[a] - cr) * (ur[a] - cr) + (ui[a] - ci) * (ui[a] - ci);
+        if (on && ((heads >> lane) & 1u)) {
+            atomicAdd(&shq[shell], (unsigned long long)ei);
+            if (s.split) atomicAdd(&shq[nshells + shell], (unsigned long long)ec);
         }
-        atomicAdd(&shq[sh_i], fx(ei));
-        atomicAdd(&shq[nshells + sh_i], fx(ec));
     }
     __syncthreads();
-    for (int64_t i = threadIdx.x; i < 2 * nshells; i += blockDim.x) hist[(int64_t)blockIdx.x * 2 * nshells + i] = shq[i];
+    for (int i = threadIdx.x; i < nsum; i += 256)
+        if (shq[i]) atomicAdd(&hist[i], shq[i]);
 }
-__global__ void k_hist_reduce(const unsigned long long *__restrict__ hist, int nblocks, int64_t nshells,
-                              const double *__restrict__ scale_p, double half_dv_over_n, double *__restrict__ out_inc,
-                              double *__restrict__ out_comp)
+// shells out of the histogram (second slot only when split)
+__global__ void k_hist_out(const unsigned long long *__restrict__ hist, int nshells, int split,
+                           const double *__restrict__ scale_p, double half_dv_over_n, double *__restrict__ out)
 {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= nshells) return;
-    unsigned long long a = 0ull, c = 0ull;
-    for (int b = 0; b < nblocks; ++b) {
-        a += hist[(int64_t)b * 2 * nshells + s];
-        c += hist[(int64_t)b * 2 * nshells + nshells + s];
-    }
-    const double inv = 1.0 / *scale_p;            // a power of two: exact
-    out_inc[s] = half_dv_over_n * ((double)a * inv);
-    out_comp[s] = half_dv_over_n * ((double)c * inv);
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= 2 * nshells) return;
+    const double inv = 1.0 / *scale_p;            // powers of two: exact
+    out[s] = !split && s >= nshells ? 0.0 : half_dv_over_n * ((double)hist[s] * 4.3368086899420177e-19 * inv * inv);
 }
 
 static int grid_for(int64_t N)
@@ -343,11 +479,10 @@ static int grid_for(int64_t N)
     return (int)(b < 1 ? 1 : b);
 }
 
-int bin_blocks(const SpecArgs &s)
+int velocity_blocks(const SpecArgs &s)
 {
-    int64_t b = (s.N + 255) / 256;
-    if (b > 152 * 2) b = 152 * 2;
-    return (int)(b < 1 ? 1 : b);
+    const int64_t b = (s.N + 255) / 256;
+    return (int)(b < 1 ? 1 : b > 152 * 8 ? 152 * 8 : b);
 }
 
 cudaError_t launch_deriv(const SpecArgs &s, const void *src, void *dst, int axis, cudaStream_t st)
@@ -359,12 +494,11 @@ cudaError_t launch_deriv(const SpecArgs &s, const void *src, void *dst, int axis
     return cudaGetLastError();
 }
 
-cudaError_t launch_velocity(const SpecArgs &s, const void *psi, void *w, cudaStream_t st)
+cudaError_t launch_velocity(const SpecArgs &s, const void *psi, void *w, double *partial, cudaStream_t st)
 {
-    if (s.prec == 0)
-        k_velocity<float><<<grid_for(s.N), 256, 0, st>>>(s, (const float2 *)psi, (float2 *)w);
-    else
-        k_velocity<double><<<grid_for(s.N), 256, 0, st>>>(s, (const double2 *)psi, (double2 *)w);
+    const int nb = velocity_blocks(s);
+    if (s.prec == 0) k_velocity<float><<<nb, 256, 0, st>>>(s, (const float2 *)psi, (float2 *)w, partial);
+    else k_velocity<double><<<nb, 256, 0, st>>>(s, (const double2 *)psi, (double2 *)w, partial);
     return cudaGetLastError();
 }
 
@@ -421,38 +555,32 @@ cudaError_t launch_trap_level(int prec, void *const *tab, int ndim, const int64_
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, double *block_hist, int nblocks,
-                       double *aux, cudaStream_t st)
+// histogram and shells of the fields uh; work: 2 nshells + 1 doubles (histogram
+// and scale), partial: npartial sums of squares from launch_velocity
+cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, const double *partial, int npartial,
+                       double *work, double half_dv_over_n, double *out, cudaStream_t st)
 {
-    const size_t smem = sizeof(unsigned long long) * 2 * (size_t)nshells;
-    unsigned long long *hq = reinterpret_cast<unsigned long long *>(block_hist);
-    cudaError_t e;
+    unsigned long long *hist = reinterpret_cast<unsigned long long *>(work);
+    double *scale = work + 2 * nshells;
+    const size_t smem = sizeof(unsigned long long) * (s.split ? 2 : 1) * (size_t)nshells;
+    // blocks of at least two iterations, as many as fit beside one another
+    const int64_t want = (s.N + 511) / 512, fit = smem > 64 * 1024 ? 2 : smem > 32 * 1024 ? 3 : 6;
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(want, 152 * fit));
+    cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * 2 * (size_t)nshells, st);
+    if (e != cudaSuccess) return e;
     if (s.prec == 0) {
-        k_field_total<float><<<nblocks, 256, 0, st>>>(s, (const float2 *)uh[0], (const float2 *)uh[1],
-                                                      (const float2 *)uh[2], aux);
-        k_fixed_scale<<<1, 32, 0, st>>>(aux, nblocks);
         e = cudaFuncSetAttribute(k_bin<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_bin<float><<<nblocks, 256, smem, st>>>(s, (const float2 *)uh[0], (const float2 *)uh[1],
-                                                 (const float2 *)uh[2], nshells, aux + nblocks, hq);
+        k_bin<float><<<nb, 256, smem, st>>>(s, (const float2 *)uh[0], (const float2 *)uh[1], (const float2 *)uh[2],
+                                            (int)nshells, partial, npartial, hist, scale);
     } else {
-        k_field_total<double><<<nblocks, 256, 0, st>>>(s, (const double2 *)uh[0], (const double2 *)uh[1],
-                                                       (const double2 *)uh[2], aux);
-        k_fixed_scale<<<1, 32, 0, st>>>(aux, nblocks);
         e = cudaFuncSetAttribute(k_bin<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_bin<double><<<nblocks, 256, smem, st>>>(s, (const double2 *)uh[0], (const double2 *)uh[1],
-                                                  (const double2 *)uh[2], nshells, aux + nblocks, hq);
+        k_bin<double><<<nb, 256, smem, st>>>(s, (const double2 *)uh[0], (const double2 *)uh[1], (const double2 *)uh[2],
+                                             (int)nshells, partial, npartial, hist, scale);
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_hist_reduce(const double *block_hist, int nblocks, int64_t nshells, double dv_over_n,
-                               const double *aux, double *out_inc, double *out_comp, cudaStream_t st)
-{
-    const int nb = (int)((nshells + 127) / 128);
-    k_hist_reduce<<<nb, 128, 0, st>>>(reinterpret_cast<const unsigned long long *>(block_hist), nblocks, nshells,
-                                      aux + nblocks, 0.5 * dv_over_n, out_inc, out_comp);
+    k_hist_out<<<(unsigned)((2 * nshells + 127) / 128), 128, 0, st>>>(hist, (int)nshells, s.split, scale,
+                                                                     half_dv_over_n, out);
     return cudaGetLastError();
 }
 

@@ -211,16 +211,16 @@ struct SpecArgs {
     double kf[3];       // 2 pi / len
     double lratio[3];   // max_len / len
     int64_t N;
-    int part;           // k_velocity: 0 u = Im(conj(psi) d psi)/|psi|, 1 w = Re(...)/|psi| = d|psi|
+    int lg[3];          // log2 of the points per axis
+    int cubic;          // all axes of one length: shells from whole numbers
+    int part;           // k_velocity: 0 u = Im(conj(psi) d psi)/|psi|, 1 w = Re(...)/|psi| = d|psi|, 2 |psi|
     int split;          // k_bin: 1 incompressible / compressible parts, 0 total of the components
     int ncomp;          // k_bin: field components summed (ndim, or 1 for psi_hat itself)
 };
 cudaError_t launch_deriv(const SpecArgs &s, const void *src, void *dst, int axis, cudaStream_t st);
-cudaError_t launch_velocity(const SpecArgs &s, const void *psi, void *w, cudaStream_t st);
-cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, double *block_hist, int nblocks,
-                       double *aux, cudaStream_t st);
-cudaError_t launch_hist_reduce(const double *block_hist, int nblocks, int64_t nshells, double dv_over_n,
-                               const double *aux, double *out_inc, double *out_comp, cudaStream_t st);
-int bin_blocks(const SpecArgs &s);
+int velocity_blocks(const SpecArgs &s);     // partial sums that launch_velocity writes
+cudaError_t launch_velocity(const SpecArgs &s, const void *psi, void *w, double *partial, cudaStream_t st);
+cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, const double *partial, int npartial,
+                       double *work, double half_dv_over_n, double *out, cudaStream_t st);
 
 }  // namespace gpe
