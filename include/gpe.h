@@ -205,8 +205,8 @@ gpe_status gpe_spectrum(gpe_plan *plan, const void *psi_dev, unsigned kinds, dou
  *   GPE_OPT_LINE_CLUSTER 1 (default): complex128 real-time steps of 1D
  *                        plans with lines of 64, 128 or 256 points and at
  *                        most 32 instances spread each line over a cluster
- *                        of 4, 8 or 16 CTAs (a latency path: FP64 work on
- *                        one SM is slow on this GPU); 0: one CTA per line.
+ *                        of 2, 4 or 8 CTAs (a latency path); 0: one CTA per
+ *                        line.
  *                        The two factor the transform differently, so their
  *                        results differ in rounding (both agree with the
  *                        FP64 reference to about 1e-14 per step).

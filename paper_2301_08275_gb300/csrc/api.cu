@@ -341,6 +341,13 @@ static void trap_fx(const gpe_plan *p, int a, double gamma, int64_t *vq, int64_t
     }
 }
 
+static void trap_decay_host(const gpe_plan *p, int a, double gamma, double *vi)
+{
+    for (int64_t j = 0; j < p->n[a]; ++j) {
+        const double x = p->lo[a] + (double)j * p->h[a];
+        vi[j] = exp(-0.5 * (0.5 * gamma * gamma * x * x * p->dt));
+    }
+}
 // Trap tables of one instance on axis a (V_a = gamma^2 x^2 / 2, th = V_a dt):
 // vh = exp(-i th/2) - 1, vf = exp(-i th) - 1 (interleaved re, im), vi = exp(-th/2).
 static void trap_tables_host(const gpe_plan *p, int a, double gamma, double *vh, double *vf, double *vi)
@@ -468,7 +475,7 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
             unit_circle_fx(na, ux);
             PLAN_TRY(upload_raw(p, &p->twx[a], ux.data(), ux.size() * sizeof(int4)));
         }
-        if (p->fxp()) {
+        if (p->prec == GPE_C128) {
             std::vector<int4> ux(na);
             std::vector<int64_t> kx(na);
             const int64_t one = (int64_t)1 << 62;
@@ -490,11 +497,15 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
                 PLAN_TRY(upload_raw(p, &p->vq[a], vq.data(), vq.size() * sizeof(int64_t)));
                 PLAN_TRY(upload_raw(p, &p->viq[a], viq.data(), viq.size() * sizeof(int64_t)));
             }
-            continue;
+            if (p->ndim > 1) continue;
         }
         PLAN_TRY(upload_cplx(p, &p->tw[a], tw));
-        PLAN_TRY(upload_cplx(p, &p->kt[a], kt));
-        if (p->trap[a]) {
+        if (p->prec == GPE_C64) PLAN_TRY(upload_cplx(p, &p->kt[a], kt));
+        if (p->trap[a] && p->prec == GPE_C128) {          // 1D imaginary time
+            std::vector<double> vi(na * B);
+            for (int64_t b = 0; b < B; ++b) trap_decay_host(p, a, gam[3 * b + a], &vi[b * na]);
+            PLAN_TRY(upload_real(p, &p->vi[a], vi));
+        } else if (p->trap[a]) {
             std::vector<double> vh(2 * na * B), vf(2 * na * B), vi(na * B);
             for (int64_t b = 0; b < B; ++b)
                 trap_tables_host(p, a, gam[3 * b + a], &vh[2 * b * na], &vf[2 * b * na], &vi[b * na]);
@@ -519,8 +530,15 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
                     vf[2 * (b * na + j) + 1] = -sin(th);
                     vi[b * na + j] = exp(-0.5 * th);
                 }
-            PLAN_TRY(upload_cplx(p, &p->vh[0], vh));
-            PLAN_TRY(upload_cplx(p, &p->vf[0], vf));
+            if (p->prec == GPE_C128) {
+                std::vector<int64_t> vq(na * B);
+                for (int64_t b = 0; b < B; ++b)
+                    for (int64_t j = 0; j < na; ++j) vq[b * na + j] = turns_fx(0.5 * d->V_host[j] * p->dt);
+                PLAN_TRY(upload_raw(p, &p->vq[0], vq.data(), vq.size() * sizeof(int64_t)));
+            } else {
+                PLAN_TRY(upload_cplx(p, &p->vh[0], vh));
+                PLAN_TRY(upload_cplx(p, &p->vf[0], vf));
+            }
             PLAN_TRY(upload_real(p, &p->vi[0], vi));
             p->trap[0] = true;
         }
@@ -545,7 +563,7 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
     PLAN_TRY(dalloc(p, (void **)&p->out4, sizeof(double) * 4 * B));
     PLAN_TRY(dalloc(p, (void **)&p->err, sizeof(int)));
     PLAN_TRY(dalloc(p, (void **)&p->ones, sizeof(double) * B));
-    if (p->fxp()) {
+    if (p->prec == GPE_C128) {
         std::vector<FxCoupling> gq(2 * B);
         for (int64_t b = 0; b < B; ++b)
             for (int full = 0; full < 2; ++full) gq[2 * b + full] = coupling_fx(gs[b], full ? p->dt : 0.5 * p->dt);
@@ -930,7 +948,7 @@ static gpe_status trap_level(gpe_plan *p, void *const *dst, const double *gamma_
 {
     double gm[3] = {0, 0, 0};
     for (int a = 0; a < p->ndim; ++a) gm[a] = gamma_t[3 * lev + a];
-    cudaError_t e = launch_trap_level(p->fxp() ? 2 : p->prec == GPE_C64 ? 0 : 1, dst, p->ndim, p->n, p->lo, p->h, gm, c * p->dt,
+    cudaError_t e = launch_trap_level(p->prec == GPE_C64 ? 0 : 2, dst, p->ndim, p->n, p->lo, p->h, gm, c * p->dt,
                                       p->batch, p->st);
     if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("trap tables: ") + cudaGetErrorString(e));
     return GPE_OK;
@@ -942,6 +960,15 @@ static void use_sched(const gpe_plan *p, PassArgs &a)
     a.vt_ax = p->sched[axis];
     a.vt_o0 = o0 < p->ndim ? p->sched[o0] : nullptr;
     a.vt_o1 = o1 < p->ndim ? p->sched[o1] : nullptr;
+}
+
+// fixed-point tables of a complex128 line
+static void line_fx(const gpe_plan *p, Line1DArgs &l, const void *vq)
+{
+    l.twx = p->twx[0];
+    l.ktx = p->ktx[0];
+    l.vq = vq;
+    l.gq = p->gq;
 }
 
 // nsteps real-time steps; with gamma_t (nsteps + 1 rows of three trap
@@ -966,6 +993,8 @@ static gpe_status step_real_dev(gpe_plan *p, void *psi, int64_t nsteps, const do
             l.kt = p->kt[0];
             l.vh = p->sched[0];
             l.vh_last = p->sched_last;
+            line_fx(p, l, p->sched[0]);
+            l.vq_last = p->sched_last;
             l.g = p->g_dev;
             l.dt = p->dt;
             l.err = p->err;
@@ -995,6 +1024,7 @@ static gpe_status step_real_dev(gpe_plan *p, void *psi, int64_t nsteps, const do
             l.kt = p->kt[0];
             l.vh = p->vh[0];
             l.vf = p->vf[0];
+            line_fx(p, l, p->vq[0]);
             l.g = p->g_dev;
             l.dt = p->dt;
             l.err = p->err;
@@ -1072,7 +1102,7 @@ extern "C" gpe_status gpe_step_real_trap(gpe_plan *p, void *psi, int64_t nsteps,
         if (!isfinite(gamma_host[i])) return fail(GPE_EINVAL, "trap frequencies must be finite");
     DeviceGuard dg(p->device);
     if (!dg.ok) return fail(GPE_ECUDA, "cannot select the plan's device");
-    const size_t ce = p->fxp() ? sizeof(int64_t) : p->prec == GPE_C64 ? sizeof(float4) : sizeof(double2);
+    const size_t ce = p->prec == GPE_C64 ? sizeof(float4) : sizeof(int64_t);
     for (int a = 0; a < p->ndim; ++a)
         if (!p->sched[a]) GPE_TRY(dalloc(p, &p->sched[a], ce * (size_t)p->n[a] * (size_t)p->batch));
     if (p->ndim == 1 && !p->sched_last) GPE_TRY(dalloc(p, &p->sched_last, ce * (size_t)p->n[0] * (size_t)p->batch));
@@ -1869,7 +1899,7 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
     double gm[3] = {0, 0, 0};
     for (int a = 0; a < p->ndim; ++a) gm[a] = gamma[a];
     GPE_CUDA(cudaMemcpyAsync(p->gamma_dev + 3 * slot, gm, sizeof(gm), cudaMemcpyHostToDevice, p->st));
-    if (p->fxp()) {
+    if (p->prec == GPE_C128) {
         FxCoupling gq[2];
         for (int full = 0; full < 2; ++full) gq[full] = coupling_fx(g, full ? p->dt : 0.5 * p->dt);
         GPE_CUDA(cudaMemcpyAsync((FxCoupling *)p->gq + 2 * slot, gq, sizeof(gq), cudaMemcpyHostToDevice, p->st));
@@ -1878,12 +1908,18 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
     for (int a = 0; a < p->ndim; ++a) {
         if (!p->trap[a]) continue;
         const int64_t na = p->n[a];
-        if (p->fxp()) {
+        if (p->prec == GPE_C128) {
             std::vector<int64_t> vq(na), viq(na);
             trap_fx(p, a, gm[a], vq.data(), viq.data());
             const size_t len = (size_t)na * sizeof(int64_t);
             GPE_CUDA(cudaMemcpyAsync((int64_t *)p->vq[a] + slot * na, vq.data(), len, cudaMemcpyHostToDevice, p->st));
             GPE_CUDA(cudaMemcpyAsync((int64_t *)p->viq[a] + slot * na, viq.data(), len, cudaMemcpyHostToDevice, p->st));
+            std::vector<double> vi(na);
+            if (p->ndim == 1) {
+                trap_decay_host(p, a, gm[a], vi.data());
+                GPE_CUDA(cudaMemcpyAsync((double *)p->vi[a] + slot * na, vi.data(), na * sizeof(double),
+                                         cudaMemcpyHostToDevice, p->st));
+            }
             GPE_CUDA(cudaStreamSynchronize(p->st));
             continue;
         }
@@ -1895,16 +1931,10 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
         const size_t ce = bh.size() / (size_t)na;      // bytes per complex entry
         GPE_CUDA(cudaMemcpyAsync((char *)p->vh[a] + slot * na * ce, bh.data(), bh.size(), cudaMemcpyHostToDevice, p->st));
         GPE_CUDA(cudaMemcpyAsync((char *)p->vf[a] + slot * na * ce, bf.data(), bf.size(), cudaMemcpyHostToDevice, p->st));
-        if (p->prec == GPE_C64) {
-            std::vector<float> f(vi.begin(), vi.end());
-            GPE_CUDA(cudaMemcpyAsync((float *)p->vi[a] + slot * na, f.data(), f.size() * sizeof(float),
-                                     cudaMemcpyHostToDevice, p->st));
-            GPE_CUDA(cudaStreamSynchronize(p->st));    // host staging goes out of scope
-        } else {
-            GPE_CUDA(cudaMemcpyAsync((double *)p->vi[a] + slot * na, vi.data(), vi.size() * sizeof(double),
-                                     cudaMemcpyHostToDevice, p->st));
-            GPE_CUDA(cudaStreamSynchronize(p->st));
-        }
+        std::vector<float> f(vi.begin(), vi.end());
+        GPE_CUDA(cudaMemcpyAsync((float *)p->vi[a] + slot * na, f.data(), f.size() * sizeof(float),
+                                 cudaMemcpyHostToDevice, p->st));
+        GPE_CUDA(cudaStreamSynchronize(p->st));    // host staging goes out of scope
     }
     GPE_CUDA(cudaStreamSynchronize(p->st));
     return GPE_OK;

@@ -533,14 +533,9 @@ __global__ void k_trap_level(int prec, void *t0, void *t1, void *t2, int ndim, i
         }
         const double sh = sin(0.5 * th);
         const double wx = -2.0 * sh * sh, wy = -sin(th);
-        void *t = a == 0 ? t0 : (a == 1 ? t1 : t2);
-        if (prec == 0) {
-            const float hx = (float)wx, hy = (float)wy;
-            static_cast<float4 *>(t)[b * na + j] =
-                make_float4(hx, hy, (float)(wx - (double)hx), (float)(wy - (double)hy));
-        } else {
-            static_cast<double2 *>(t)[b * na + j] = make_double2(wx, wy);
-        }
+        const float hx = (float)wx, hy = (float)wy;
+        static_cast<float4 *>(a == 0 ? t0 : (a == 1 ? t1 : t2))[b * na + j] =
+            make_float4(hx, hy, (float)(wx - (double)hx), (float)(wy - (double)hy));
     }
 }
 

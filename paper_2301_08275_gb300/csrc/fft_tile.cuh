@@ -81,14 +81,14 @@ template <> struct UT<double> { using U = double2; };
 template <> struct UT<fx> { using U = int4; };
 
 // v * u for a unit factor u (conj(u) when CONJ), rounding only the result
-template <bool CONJ = false> __device__ __forceinline__ float2 umul(float2 v, float4 u)
+template <bool CONJ = false, int SH = 0> __device__ __forceinline__ float2 umul(float2 v, float4 u)
 {
     const float uy = CONJ ? -u.y : u.y, wy = CONJ ? -u.w : u.w;
     const float tx = fmaf(v.x, u.z, -v.y * wy);
     const float ty = fmaf(v.x, wy, v.y * u.z);
     return mk(fmaf(v.x, u.x, fmaf(-v.y, uy, tx)), fmaf(v.x, uy, fmaf(v.y, u.x, ty)));
 }
-template <bool CONJ = false> __device__ __forceinline__ double2 umul(double2 v, double2 u)
+template <bool CONJ = false, int SH = 0> __device__ __forceinline__ double2 umul(double2 v, double2 u)
 {
     const double uy = CONJ ? -u.y : u.y;
     return mk(fma(v.x, u.x, -v.y * uy), fma(v.x, uy, v.y * u.x));
@@ -96,8 +96,8 @@ template <bool CONJ = false> __device__ __forceinline__ double2 umul(double2 v, 
 
 // what a butterfly's first input (twiddle 1) gets in place of umul: fixed-point
 // twiddles carry a scale (fx.cuh), floating ones none
-__device__ __forceinline__ float2 tw_first(float2 v) { return v; }
-__device__ __forceinline__ double2 tw_first(double2 v) { return v; }
+template <int SH = 0> __device__ __forceinline__ float2 tw_first(float2 v) { return v; }
+template <int SH = 0> __device__ __forceinline__ double2 tw_first(double2 v) { return v; }
 
 // v * (1 + w) for a unit factor close to one, stored as its offset w: the
 // small product v*w is formed first and v is added last, so each component is
@@ -269,6 +269,7 @@ __host__ __device__ constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c
 template <int N> struct Radix {
     static constexpr int LG = ilog2c(N);
     static constexpr int E = N >= 8 ? 8 : N;           // points per thread
+    static constexpr int TWSH = 0;                     // fixed point: a twiddle divides by 4 (see fx.cuh)
     static constexpr int REM = N >= 8 ? LG % 3 : 0;    // log2 of the first pass when not 8
     static constexpr int P = N < 8 ? 1 : LG / 3 + (REM ? 1 : 0);
     __host__ __device__ static constexpr int radix(int p) { return N < 8 ? N : ((REM && p == 0) ? (1 << REM) : 8); }
@@ -283,6 +284,7 @@ template <int N> struct Radix {
 template <int N> struct Radix32 {
     static constexpr int LG = ilog2c(N);
     static constexpr int E = 32;
+    static constexpr int TWSH = 0;
     static constexpr int REST = LG - 5;
     static constexpr int P = REST <= 0 ? 1 : (REST <= 5 ? 2 : 3);
     __host__ __device__ static constexpr int radix(int p)
@@ -292,7 +294,20 @@ template <int N> struct Radix32 {
     }
     __host__ __device__ static constexpr int ns(int p) { return p == 0 ? 1 : ns(p - 1) * radix(p - 1); }
 };
+// Pass plan for threads holding 4 points (N >= 4): radix 4, a radix-2 first
+// pass when log2 N is odd.  More threads per line and so a shorter chain of
+// instructions per thread, at one exchange more per transform: for 1D lines
+// too few to fill the GPU.
+template <int N> struct Radix4 {
+    static constexpr int LG = ilog2c(N);
+    static constexpr int E = 4;
+    static constexpr int TWSH = 1;                     // fixed point: a twiddle divides by 2
+    static constexpr int P = (LG + 1) / 2;
+    __host__ __device__ static constexpr int radix(int p) { return (LG & 1) && p == 0 ? 2 : 4; }
+    __host__ __device__ static constexpr int ns(int p) { return p == 0 ? 1 : ns(p - 1) * radix(p - 1); }
+};
 template <int N, int E> struct PassPlan { using T = Radix<N>; };
+template <int N> struct PassPlan<N, 4> { using T = Radix4<N>; };
 template <int N> struct PassPlan<N, 32> { using T = Radix32<N>; };
 
 // ---------------------------------------------------------------- tile engine
@@ -589,10 +604,10 @@ template <typename R, int N, int L, int LPT, bool SW = false, int EPT = 0, bool 
                 for (int m = 1; m < r; ++m) {
                     const U w = twk[(m - 1) * Ns];
 #pragma unroll
-                    for (int ln = 0; ln < LPT; ++ln) x[ln][m] = umul<(DIR > 0)>(x[ln][m], w);
+                    for (int ln = 0; ln < LPT; ++ln) x[ln][m] = umul<(DIR > 0), PL::TWSH>(x[ln][m], w);
                 }
 #pragma unroll
-                for (int ln = 0; ln < LPT; ++ln) x[ln][0] = tw_first(x[ln][0]);
+                for (int ln = 0; ln < LPT; ++ln) x[ln][0] = tw_first<PL::TWSH>(x[ln][0]);
             }
 #pragma unroll
             for (int ln = 0; ln < LPT; ++ln) Dft<r, DIR, C>::run(x[ln]);
@@ -660,8 +675,10 @@ __device__ __forceinline__ void sweep_transforms(typename T::C (&v)[T::LPT_][T::
 }
 
 // Bits of growth of a transform of a pass plan relative to |x|_2, times two:
-// after pass p the values are at most sqrt(points so far) |x|_2 / 4^p.
+// after pass p the values are at most sqrt(points so far) |x|_2 / 2^(D p), D =
+// 2 - TWSH the bits a twiddle divides by.
 template <typename PL, int LG> struct FxGrowth {
+    static constexpr int D = 2 - PL::TWSH;
     __host__ __device__ static constexpr int lg_to(int p)
     {
         int n = 1;
@@ -672,15 +689,22 @@ template <typename PL, int LG> struct FxGrowth {
     {
         int m = 0;
         for (int p = 0; p < PL::P; ++p) {
-            const int g = lg_to(p) - 4 * p;
+            const int g = lg_to(p) - 2 * D * p;
             m = g > m ? g : m;
         }
         return m;
     }
-    static constexpr int DROP = 2 * (PL::P - 1);          // bits the twiddles of one transform divide by
+    static constexpr int DROP = D * (PL::P - 1);          // bits the twiddles of one transform divide by
     static constexpr int END2 = LG - 2 * DROP;            // growth at the end, times two
-    // two transforms with a unit factor between them that keeps the scale
-    static constexpr int BITS = ((peak2() > END2 + peak2() ? peak2() : END2 + peak2()) + 1) / 2;
+    // two transforms with a unit factor between them that scales by 2^mid
+    __host__ __device__ static constexpr int bits(int mid)
+    {
+        const int second = END2 + 2 * mid + peak2(), m = second > peak2() ? second : peak2();
+        return ((m > 0 ? m : 0) + 1) / 2;
+    }
+    static constexpr int BITS = bits(0);
+    // the kinetic factor's scale 2^MID that makes transform, factor and inverse a unitary step
+    static constexpr int MID = 2 * DROP - LG;
 };
 
 }  // namespace gpe

@@ -143,15 +143,20 @@ __device__ __forceinline__ fx2 fx_madd1(fx2 v, fx2 w)
 // the tile engine's operations: a twiddle divides by 4 (the growth of the
 // radix-8 pass that follows it is at most 8, sqrt(8) in the mean), so the
 // butterfly's first input, which has no twiddle, is divided alike
-template <bool CONJ = false> __device__ __forceinline__ fx2 umul(fx2 v, int4 w)
+// (radix-4 plans divide by 2)
+template <bool CONJ = false, int SH = 0> __device__ __forceinline__ fx2 umul(fx2 v, int4 w)
 {
     static_assert(!CONJ, "the sweeps run one copy of the forward transform");
-    return fx_mul<0>(v, w);
+    return fx_mul<SH>(v, w);
 }
 // (ties to even: rounding them up would shift every mode alike by 1/8 of the
 // last place, which the inverse transform gathers at the line's first point)
-__device__ __forceinline__ long long fx_quarter(long long a) { return (a + 1 + ((a >> 2) & 1)) >> 2; }
-__device__ __forceinline__ fx2 tw_first(fx2 v) { return mk(fx_quarter(v.x), fx_quarter(v.y)); }
+template <int SH> __device__ __forceinline__ long long fx_down(long long a)
+{
+    constexpr int d = 2 - SH;
+    return (a + ((1 << (d - 1)) - 1) + ((a >> d) & 1)) >> d;
+}
+template <int SH = 0> __device__ __forceinline__ fx2 tw_first(fx2 v) { return mk(fx_down<SH>(v.x), fx_down<SH>(v.y)); }
 // x / sqrt(2) = x - x (1 - 1/sqrt(2)): the constant has 64 fraction bits, the result keeps the scale
 __device__ __forceinline__ long long mul_rsqrt2(long long a)
 {
@@ -381,6 +386,36 @@ __device__ __forceinline__ long long fx_turns(double t)
 {
     t -= rint(t);
     return (long long)((unsigned long long)(long long)(t * 9223372036854775808.0) << 1);
+}
+
+// The interaction's angle for values held as v 2^q: coupling entry gq (half or
+// full step), g c / 2 pi as a double for angles that may pass a turn.
+struct FxNonlinear {
+    Limbs m;
+    int sh, q;
+    bool none, neg;
+};
+__device__ __forceinline__ FxNonlinear fx_nonlinear(const FxCoupling *gq, int q)
+{
+    FxNonlinear r;
+    const long long m = gq->m;
+    r.m = limbs(m);
+    r.none = m == 0;
+    r.neg = gq->neg != 0;
+    r.sh = 62 + 54 + gq->e + q;
+    r.q = q;
+    return r;
+}
+__device__ __forceinline__ long long fx_nl_angle(fx2 v, const FxNonlinear &f, double g, double c_turn)
+{
+    if (f.none) return 0;
+    if (f.sh <= 0) {
+        const long long t = fx_angle(v, f.m, f.sh);
+        return f.neg ? -t : t;
+    }
+    // in FP64, reduced there
+    const double x = fx_to(v.x, f.q), y = fx_to(v.y, f.q);
+    return fx_turns(g * c_turn * (x * x + y * y));
 }
 
 }  // namespace gpe

@@ -151,6 +151,9 @@ struct Line1DArgs {
     const void *vh, *vf;    // offsets exp(-i V dt/2) - 1, exp(-i V dt) - 1 ([batch][n]) or NULL
     const void *vh_last;    // optional: the last half-step's table instead of vh (time-dependent trap)
     const void *vi;         // real decay table (imag) or NULL
+    // complex128 real time (fixed point): unit factors, half-step trap angles in
+    // 2^-64 turns (or NULL), the last half-step's instead, and the coupling
+    const void *twx, *ktx, *vq, *vq_last, *gq;
     const double *g;
     double dt;
     double target_norm_over_dv;   // imag: target norm / cell volume
@@ -163,7 +166,7 @@ struct Line1DArgs {
 };
 cudaError_t launch_line1d(int prec, const Line1DArgs &a, cudaStream_t st);
 // complex128 real-time steps of at most LINE_CLUSTER_MAX_BATCH lines of 64,
-// 128 or 256 points, one line per cluster of 4, 8 or 16 CTAs (line_cluster.cu);
+// 128 or 256 points, one line per cluster of 2, 4 or 8 CTAs (line_cluster.cu);
 // cudaErrorNotSupported when the device cannot place such a cluster
 constexpr int64_t LINE_CLUSTER_MAX_BATCH = 32;
 bool line1d_cluster_applies(const Line1DArgs &a);
@@ -171,8 +174,8 @@ cudaError_t launch_line1d_cluster(const Line1DArgs &a, cudaStream_t st);
 
 // trap tables of one time level of a time-dependent harmonic trap (diag_spec.cu):
 // for every axis a < ndim and every instance, tab[a][b*n[a] + j] = exp(-i V_a c) - 1
-// with V_a = gamma[a]^2 x_j^2 / 2, x_j = lo[a] + j h[a] (float4 hi/lo pairs for
-// prec 0, double2 for prec 1), or the angles V_a c in 2^-64 turns (int64) for prec 2
+// with V_a = gamma[a]^2 x_j^2 / 2, x_j = lo[a] + j h[a] (float4 hi/lo pairs)
+// for prec 0, or the angles V_a c in 2^-64 turns (int64) for prec 2
 cudaError_t launch_trap_level(int prec, void *const *tab, int ndim, const int64_t *n, const double *lo,
                               const double *h, const double *gamma, double c, int64_t batch, cudaStream_t st);
 

@@ -596,11 +596,7 @@ template <typename R, int N, bool ROWS, int VAR> __host__ __device__ constexpr s
 template <int E, int TPL>
 __device__ __forceinline__ void fx_nreal(fx2 (&v)[E], int q, const PassArgs &a, const LineGeom &g, int tl)
 {
-    const FxCoupling *gq = static_cast<const FxCoupling *>(a.gq) + 2 * g.ti + a.vq_full;
-    const long long gm = gq->m;
-    const Limbs m = limbs(gm);
-    const bool neg = gq->neg != 0;
-    const int sh = 62 + 54 + gq->e + q;
+    const FxNonlinear nl = fx_nonlinear(static_cast<const FxCoupling *>(a.gq) + 2 * g.ti + a.vq_full, q);
     const long long *vax = static_cast<const long long *>(a.vt_ax);
     const long long *v0 = static_cast<const long long *>(a.vt_o0), *v1 = static_cast<const long long *>(a.vt_o1);
     const double *vs = static_cast<const double *>(a.vsamp);
@@ -610,16 +606,7 @@ __device__ __forceinline__ void fx_nreal(fx2 (&v)[E], int q, const PassArgs &a, 
     const double cs = a.nl_c * 0.15915494309189533577;      // per turn
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        long long t;
-        if (gm == 0) t = 0;
-        else if (sh <= 0) {
-            t = fx_angle(v[e], m, sh);
-            if (neg) t = -t;
-        } else {
-            // angles that may pass a turn: in FP64, reduced there
-            const double x = fx_to(v[e].x, q), y = fx_to(v[e].y, q);
-            t = fx_turns(a.g[g.ti] * cs * (x * x + y * y));
-        }
+        long long t = fx_nl_angle(v[e], nl, a.g[g.ti], cs);
         long long w = line;
         if (vax) w += vax[(int64_t)g.ti * a.nax + tl + TPL * e];
         t += (long long)((unsigned long long)w << a.vq_full);
@@ -1165,7 +1152,7 @@ __global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1D
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = valid ? psi[tl + TPL * e] : mk((R)0, (R)0);
         const double g = a.g[ib];
-        if (!a.imag) {
+        if (sizeof(R) == 4 && !a.imag) {        // complex128: k_line1d_fx
             const U *kt = static_cast<const U *>(a.kt);
             const U *vh = static_cast<const U *>(a.vh);
             const U *vf = static_cast<const U *>(a.vf);
@@ -1239,6 +1226,89 @@ __global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1D
 #pragma unroll
             for (int e = 0; e < E; ++e) psi[tl + TPL * e] = v[e];
         }
+    }
+}
+
+// complex128 real-time steps of 1D lines in fixed point (fx.cuh): the norm of a
+// line is conserved, so one scale taken when the line is loaded serves all steps
+// of the launch (transform, kinetic factor and inverse together keep it), and
+// the line is converted twice per launch.  L lines per CTA, interleaved in
+// shared memory.  Measured, us per step of 1 / 400 lines (FP64 before): 32
+// points 2.4 / 5.0 (17.2 / 17.3), 256 points 2.8 / 6.2 (22.6 / 99), 1024 points
+// 5.4 / 13 (30 / 118), 4096 points 23 / 54 (128 / 386).
+template <int N, int L, int EPT> struct Line1DFx {
+    using T = GTile<fx, N, L, 1, (L < 8), (N >= 16 ? EPT : 0)>;
+    using G = FxGrowth<typename T::PL, ilog2c(N)>;
+    static constexpr size_t smem = sizeof(fx2) * T::BUF_POINTS + sizeof(int4) * N + 2 * sizeof(unsigned) * L;
+};
+template <int N, int L, int EPT>
+__global__ void __launch_bounds__(Line1DFx<N, L, EPT>::T::NT) k_line1d_fx(const Line1DArgs a)
+{
+    using T = typename Line1DFx<N, L, EPT>::T;
+    using G = typename Line1DFx<N, L, EPT>::G;
+    constexpr int E = T::E, TPL = T::TPL, NT = T::NT;
+    constexpr int KSH = G::MID + 2;          // kinetic factors of 62 bits: product shifted by KSH - 64
+    extern __shared__ __align__(128) unsigned char smraw[];
+    fx2 *sm = reinterpret_cast<fx2 *>(smraw);
+    int4 *tw = reinterpret_cast<int4 *>(sm + T::BUF_POINTS);
+    unsigned *lsc = reinterpret_cast<unsigned *>(tw + N);
+    const int t = threadIdx.x, l = t % L, tl = t / L;
+    T::load_twiddles(tw, static_cast<const int4 *>(a.twx), t, NT);
+    const int4 *kt = static_cast<const int4 *>(a.ktx);
+    int4 kin[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        kin[e] = kt[tl + TPL * e];
+        if constexpr (KSH < 0) {
+            const fx2 w = fx_value(kin[e]);
+            kin[e] = fx_pack(w.x >> -KSH, w.y >> -KSH);
+        }
+    }
+    const int64_t ntiles = (a.batch + L - 1) / L;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t inst = tile * L + l;
+        const bool valid = inst < a.batch;
+        const int64_t ip = valid ? inst : 0;
+        double2 *psi = a.inst_ptr ? static_cast<double2 *>(a.inst_ptr[ip]) : static_cast<double2 *>(a.psi) + ip * N;
+        const int64_t ib = a.slot_of ? a.slot_of[ip] : ip;
+        double2 d[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) d[e] = valid ? psi[tl + TPL * e] : mk(0.0, 0.0);
+        for (int i = t; i < 2 * L; i += NT) lsc[i] = 0;
+        __syncthreads();
+        const LineScale ls = line_scale<L, NT, E>(d, lsc, lsc + L, l, G::bits(KSH - 2));
+        fx2 v[1][E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[0][e] = mk(fx_from(d[e].x, ls.q), fx_from(d[e].y, ls.q));
+        const FxCoupling *gq = static_cast<const FxCoupling *>(a.gq) + 2 * ib;
+        const double g = a.g[ib], ct = a.dt * 0.15915494309189533577;
+        const long long *vq = static_cast<const long long *>(a.vq);
+        const long long *vl = a.vq_last ? static_cast<const long long *>(a.vq_last) : vq;
+        auto substep = [&](const FxNonlinear &nl, int full, const long long *trap, double c) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                long long ang = fx_nl_angle(v[0][e], nl, g, c);
+                if (trap) ang += (long long)((unsigned long long)trap[ib * N + tl + TPL * e] << full);
+                v[0][e] = fx_rotate(v[0][e], ang);
+            }
+        };
+        substep(fx_nonlinear(gq, ls.q), 0, vq, 0.5 * ct);
+#pragma unroll 1
+        for (int64_t st = 0; st < a.nsteps; ++st) {
+            sweep_transforms<T, false>(v, sm, sm, tl, l, tw, -1, +1, [&]() {
+#pragma unroll
+                for (int e = 0; e < E; ++e) v[0][e] = fx_mul<(KSH > 0 ? KSH : 0)>(v[0][e], kin[e]);
+            });
+            const int full = st == a.nsteps - 1 ? 0 : 1;
+            substep(fx_nonlinear(gq + full, ls.q), full, full ? vq : vl, full ? ct : 0.5 * ct);
+        }
+        if (valid) {
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                psi[tl + TPL * e] = ls.bad ? mk(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll))
+                                           : mk(fx_to(v[0][e].x, ls.q), fx_to(v[0][e].y, ls.q));
+        }
+        __syncthreads();         // lsc and sm are reused
     }
 }
 
@@ -1358,11 +1428,37 @@ template <typename R, int N, int L> static cudaError_t launch_line1d_l(const Lin
     return cudaGetLastError();
 }
 
+template <int N, int L, int EPT> static cudaError_t launch_line1d_fx_l(const Line1DArgs &a, cudaStream_t st)
+{
+    using F = Line1DFx<N, L, EPT>;
+    static_assert(F::T::layout_consistent(), "shared layout of the exchanges");
+    static LaunchCache lc;
+    int cap = 0;
+    cudaError_t e = prepare(k_line1d_fx<N, L, EPT>, lc, F::T::NT, F::smem, &cap);
+    if (e != cudaSuccess) return e;
+    const int64_t ntiles = (a.batch + L - 1) / L;
+    if (ntiles <= 0) return cudaSuccess;
+    k_line1d_fx<N, L, EPT><<<(int)(ntiles < cap ? ntiles : cap), F::T::NT, F::smem, st>>>(a);
+    return cudaGetLastError();
+}
+// Lines that do not fill the SMs: one per CTA and 4 points per thread (shorter
+// chains); otherwise 8 points per thread, with several lines in a CTA when
+// they are short.
+template <int N> static cudaError_t launch_line1d_fx(const Line1DArgs &a, cudaStream_t st)
+{
+    constexpr int L = N >= 256 ? 1 : N >= 64 ? 4 : 8;
+    if (a.batch < 2 * sm_count()) return launch_line1d_fx_l<N, 1, 4>(a, st);
+    return launch_line1d_fx_l<N, L, 0>(a, st);
+}
+
 // Fewer instances than SMs: one line per CTA, so that no warp spends the SM's
 // pipes on the empty lines of a part-filled tile (the per-line arithmetic is
 // the same either way).
 template <typename R, int N> static cudaError_t launch_line1d_t(const Line1DArgs &a, cudaStream_t st)
 {
+    if constexpr (sizeof(R) == 8) {
+        if (!a.imag) return launch_line1d_fx<N>(a, st);
+    }
     constexpr int L = pick_lines_1d<R, N>();
     if constexpr (L > 1) {
         if (a.batch < sm_count()) return launch_line1d_l<R, N, 1>(a, st);
