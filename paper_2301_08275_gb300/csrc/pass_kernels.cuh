@@ -509,13 +509,17 @@ template <typename R> __host__ __device__ constexpr int lines_per_thread() { ret
 // i is transformed in the other.
 // points per thread: 16 for strided complex64 lines of at least 16 points (two
 // butterflies per thread and pass: the 512^3 y sweep 0.51 -> 0.45 ms, z 0.92 ->
-// 0.90 ms), else 8; rows keep 8 (16 measured slower there).  Every tile shape
+// 0.90 ms), else 8; rows keep 8 (16 measured slower there).  4 for complex128
+// (radix-4 passes of the fixed-point sweeps): the same work at 1024^2 (85 against
+// 88 us per step with 8), half the chain per thread on small grids (128^2
+// imaginary step 55 -> 37 us).  Every tile shape
 // of a pass kind uses the same count, so the per-line reductions add in the
 // same order whichever shape the tuner picks.
 template <typename R, int N, bool ROWS> __host__ __device__ constexpr int pass_points_per_thread()
 {
     return (!ROWS && sizeof(R) == 4 && N >= 256 && N <= 1024) ? 32
            : (!ROWS && sizeof(R) == 4 && N >= 16)              ? 16
+           : (sizeof(R) == 8 && N >= 16)                       ? 4
                                                                : Radix<N>::E;
 }
 
