@@ -138,6 +138,7 @@ struct gpe_plan {
     int tile_var[3] = {0, 0, 0};            // tile shape per axis
     int tx_extra = 0;                       // GPE_OPT_TEST_STALL_COPIES
     bool generic_passes = false;            // GPE_OPT_GENERIC_PASSES
+    bool sweeps_chosen = false;             // an option asked for particular sweeps
     bool line_cluster = true;               // GPE_OPT_LINE_CLUSTER
     bool no_dither = false;                 // GPE_OPT_NO_DITHER
     // trap tables of one time level (gpe_step_real_trap), allocated on first use
@@ -971,6 +972,55 @@ static void line_fx(const gpe_plan *p, Line1DArgs &l, const void *vq)
     l.gq = p->gq;
 }
 
+// ------------------------------------------------------------------ small planes on chip
+// Grids of 64 or 128 points per axis take the cluster kernel of plane_cluster.cu
+// unless an option asked for particular sweeps, a trap schedule gives every
+// step its own tables, or there are so many instances that sweeps over all of
+// them fill the GPU better.
+static bool plane_applies(const gpe_plan *p)
+{
+    return plane_shape(p->ndim, p->n) && !p->sweeps_chosen && !p->tx_extra &&
+           active_count(p) * p->N <= PLANE_MAX_POINTS;
+}
+// cudaErrorNotSupported: no such cluster on this device, nothing was enqueued
+static cudaError_t plane_steps(gpe_plan *p, void *psi, int64_t nsteps, bool imag, double target)
+{
+    PlaneArgs a;
+    memset(&a, 0, sizeof(a));
+    a.count = active_count(p);
+    a.rows = make_pass(p, 0, psi, psi, a.count);
+    a.cols = make_pass(p, 1, psi, psi, a.count);
+    set_nreal(p, a.rows, true);
+    a.rows.err = p->err;
+    a.imag = imag ? 1 : 0;
+    for (int i = 0; i < 2; ++i) {
+        a.vh[i] = p->prec == GPE_C128 ? p->vq[i] : p->vh[i];
+        a.vf[i] = p->prec == GPE_C128 ? p->vq[i] : p->vf[i];
+    }
+    a.dt = p->dt;
+    a.dv = p->dv;
+    a.target = target;
+    a.dither = !imag && p->prec == GPE_C64 && !p->no_dither;
+    const int64_t chunk = imag || p->prec == GPE_C128 ? 1 << 20 : PLANE_STEPS;
+    for (int64_t s0 = 0; s0 < nsteps; s0 += chunk) {
+        a.nsteps = (int)std::min(chunk, nsteps - s0);
+        a.first = s0 == 0;
+        a.last = s0 + a.nsteps == nsteps;
+        for (int s = 0; a.dither && s < a.nsteps; ++s) {
+            PassArgs k;
+            memset(&k, 0, sizeof(k));
+            a.dphi[s] = dither_angle(s0 + s);
+            set_dither(k, a.dphi[s]);
+            for (int q = 0; q < 4; ++q) a.dk[s][q] = (float)k.dk[q];
+        }
+        TraceScope ts(p, "plane" + std::to_string(p->n[0]) + "x" + std::to_string(p->n[1]) + (imag ? ":imag" : ":real"));
+        const cudaError_t e = p->prec == GPE_C64 ? launch_plane_f32((int)p->n[0], (int)p->n[1], a, p->st)
+                                                 : launch_plane_f64((int)p->n[0], (int)p->n[1], a, p->st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // nsteps real-time steps; with gamma_t (nsteps + 1 rows of three trap
 // frequencies) the harmonic trap follows that schedule instead of the plan's
 // static trap: the nonlinear half-steps next to time level n use gamma_t row n.
@@ -1039,6 +1089,12 @@ static gpe_status step_real_dev(gpe_plan *p, void *psi, int64_t nsteps, const do
             if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("1D launch: ") + cudaGetErrorString(e));
         }
         return GPE_OK;
+    }
+    if (!gamma_t && plane_applies(p)) {
+        const cudaError_t e = plane_steps(p, psi, nsteps, false, 0.0);
+        if (e == cudaSuccess) return GPE_OK;
+        if (e != cudaErrorNotSupported) return fail(GPE_ECUDA, std::string("plane launch: ") + cudaGetErrorString(e));
+        cudaGetLastError();
     }
     // prologue: first nonlinear half-step and forward transforms of all but the last axis
     PassArgs x0 = make_pass(p, 0, psi, psi, B);
@@ -1301,6 +1357,7 @@ extern "C" gpe_status gpe_plan_set_option(gpe_plan *p, int option, int64_t value
 {
     if (!p) return fail(GPE_EINVAL, "NULL plan");
     if (value != 0 && value != 1) return fail(GPE_EINVAL, "plan options take 0 or 1");
+    if (option >= GPE_OPT_TMA_STAGING && option <= GPE_OPT_GENERIC_PASSES) p->sweeps_chosen = true;
     if (option == GPE_OPT_TEST_STALL_COPIES) {
         p->tx_extra = value ? 16 : 0;
         return GPE_OK;
@@ -1399,6 +1456,7 @@ extern "C" gpe_status gpe_plan_autotune(gpe_plan *p, const void *psi, int reps, 
     if (reps < 1 || reps > 1000) return fail(GPE_EINVAL, "reps must be in [1, 1000]");
     if (flags & ~GPE_TUNE_NO_TMA) return fail(GPE_EINVAL, "unknown autotune flag");
     if (p->ndim == 1) return GPE_OK;
+    if (plane_applies(p)) return GPE_OK;       // stepped on chip: no sweeps to choose
     if (p->cur_count > 0) return fail(GPE_EINVAL, "plan is in use by a batch launch");
     DeviceGuard dg(p->device);
     if (!dg.ok) return fail(GPE_ECUDA, "cannot select the plan's device");
@@ -1613,6 +1671,12 @@ static gpe_status imag_steps(gpe_plan *p, void *psi, int64_t nsteps, double targ
         cudaError_t e = launch_line1d(p->prec, l, p->st);
         if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("1D launch: ") + cudaGetErrorString(e));
         return GPE_OK;
+    }
+    if (plane_applies(p)) {
+        const cudaError_t e = plane_steps(p, psi, nsteps, true, target);
+        if (e == cudaSuccess) return GPE_OK;
+        if (e != cudaErrorNotSupported) return fail(GPE_ECUDA, std::string("plane launch: ") + cudaGetErrorString(e));
+        cudaGetLastError();
     }
     GPE_TRY(fill_scale_one(p));
     const int piv = p->ndim - 1;
@@ -1876,6 +1940,17 @@ gpe_status plan_prepare(gpe_plan *p)
         t.ntiles = 0;
         cudaError_t e = launch_pass(p->prec, a == 0, t, p->st);
         if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
+    }
+    if (plane_shape(p->ndim, p->n)) {
+        PlaneArgs a;
+        memset(&a, 0, sizeof(a));
+        for (a.imag = 0; a.imag < 2; ++a.imag) {
+            const cudaError_t e = p->prec == GPE_C64 ? launch_plane_f32((int)p->n[0], (int)p->n[1], a, p->st)
+                                                     : launch_plane_f64((int)p->n[0], (int)p->n[1], a, p->st);
+            if (e != cudaSuccess && e != cudaErrorNotSupported)
+                return fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
+            if (e != cudaSuccess) cudaGetLastError();
+        }
     }
     if (p->ndim == 1) {
         Line1DArgs l;

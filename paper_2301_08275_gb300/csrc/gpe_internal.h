@@ -140,6 +140,34 @@ struct ResidentArgs {
 cudaError_t launch_resident2d(int n, const ResidentArgs &a, cudaStream_t st);
 bool resident2d_supported(int prec, int ndim, const int64_t *n);
 
+// Steps of 2D grids of 64 or 128 points per axis held on chip by one cluster
+// per instance (plane_cluster.cu); cudaErrorNotSupported when the device
+// cannot place such a cluster.  A call's steps come in launches of at most
+// PLANE_STEPS (complex64: the dither of each step is an argument); a launch that
+// is not the call's last leaves the state as it is between two steps (after
+// the forward row transform), and the next one takes it up there.
+constexpr int PLANE_STEPS = 64;
+// points of all instances of a call: beyond, sweeps over all of them at once are
+// about as fast (8 instances of 128^2 complex128: 20.6 us per step here, 22 as sweeps)
+constexpr int64_t PLANE_MAX_POINTS = 1 << 17;
+struct PlaneArgs {
+    PassArgs rows, cols;       // argument templates of the row (nonlinear) and column (kinetic) sweeps
+    const void *vh[2], *vf[2]; // trap tables of x and y for half and full steps (complex128: the same, see PassArgs)
+    int64_t count;             // instances
+    int nsteps, imag;
+    int first, last;           // this launch opens / closes the call's real-time steps
+    double dt, dv, target;     // imaginary time: cell volume and target norm
+    int dither;
+    double dphi[PLANE_STEPS];
+    float dk[PLANE_STEPS][4];
+};
+cudaError_t launch_plane_f32(int n0, int n1, const PlaneArgs &a, cudaStream_t st);
+cudaError_t launch_plane_f64(int n0, int n1, const PlaneArgs &a, cudaStream_t st);
+inline bool plane_shape(int ndim, const int64_t *n)
+{
+    return ndim == 2 && (n[0] == 64 || n[0] == 128) && (n[1] == 64 || n[1] == 128);
+}
+
 struct Line1DArgs {
     void *psi;
     int64_t batch;

@@ -647,19 +647,18 @@ __device__ __forceinline__ void fx_nimag(double2 (&d)[E], double s, const PassAr
 }
 
 // One sweep of a line: substep, transform, substep, transform (see SweepProg),
-// on doubles in and out.  Scaling exponents: q falls by the bits that the
+// on doubles in and out; s is the factor of OP_SCALE and OP_SCALE_NIMAG, one
+// otherwise.  Scaling exponents: q falls by the bits that the
 // twiddles divide by, the kinetic substep carries the 1/N of the inverse.
-template <int N, bool ROWS, int VAR, bool PING>
-__device__ __forceinline__ void fx_sweep(double2 (&d)[PassTileFx<N, ROWS, VAR>::E], const PassArgs &a,
-                                         const LineGeom &g, double2 *sm, double2 *ss, int tl, int l, const double2 *tw,
-                                         unsigned *lsc, int op_pre, int fft1, int op_mid, int fft2)
+template <typename T, bool PING>
+__device__ __forceinline__ void fx_sweep(double2 (&d)[T::E], const PassArgs &a, const LineGeom &g, double s,
+                                         double2 *sm, double2 *ss, int tl, int l, const int4 *tw, unsigned *lsc,
+                                         int op_pre, int fft1, int op_mid, int fft2)
 {
-    using T = PassTileFx<N, ROWS, VAR>;
+    constexpr int E = T::E, TPL = T::TPL, L = T::NP, N = E * TPL;
     using G = FxGrowth<typename T::PL, ilog2c(N)>;
-    constexpr int E = T::E, TPL = T::TPL, L = T::NP;
-    if (op_pre == OP_SCALE || op_pre == OP_SCALE_NIMAG) {
-        const double s = a.scale[g.inst];
-        if (op_pre == OP_SCALE_NIMAG) {
+    if (op_pre == OP_SCALE || op_pre == OP_SCALE_NIMAG || op_pre == OP_NIMAG) {
+        if (op_pre != OP_SCALE) {
             fx_nimag<E, TPL>(d, s, a, g, tl);
         } else {
 #pragma unroll
@@ -673,8 +672,8 @@ __device__ __forceinline__ void fx_sweep(double2 (&d)[PassTileFx<N, ROWS, VAR>::
 #pragma unroll
     for (int e = 0; e < E; ++e) v[0][e] = mk(fx_from(d[e].x, q), fx_from(d[e].y, q));
     if (op_pre == OP_NREAL) fx_nreal<E, TPL>(v[0], q, a, g, tl);
-    sweep_transforms<T, PING>(v, reinterpret_cast<fx2 *>(sm), reinterpret_cast<fx2 *>(ss), tl, l,
-                              reinterpret_cast<const int4 *>(tw), fft1, fft2, [&]() {
+    sweep_transforms<T, PING>(v, reinterpret_cast<fx2 *>(sm), reinterpret_cast<fx2 *>(ss), tl, l, tw, fft1, fft2,
+                              [&]() {
         q += G::DROP;
         if (op_mid == OP_NREAL) {
             fx_nreal<E, TPL>(v[0], q, a, g, tl);
@@ -1047,8 +1046,10 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
                 if (tl == 0 && g[ln].valid) a.partials[(int64_t)(6 + a.axis) * a.lines_cap + g[ln].lg] = sk[ln];
         } else {
             if constexpr (sizeof(R) == 8) {
-                fx_sweep<N, ROWS, VAR, PING>(v[0], a, g[0], sm, PING ? scr : sm, tl, l0, tw, lsc, op_pre, fft1, op_mid,
-                                             fft2);
+                const bool scaled = op_pre == OP_SCALE || op_pre == OP_SCALE_NIMAG;
+                fx_sweep<PassTileFx<N, ROWS, VAR>, PING>(v[0], a, g[0], scaled ? a.scale[g[0].inst] : 1.0, sm,
+                                                         PING ? scr : sm, tl, l0, reinterpret_cast<const int4 *>(tw),
+                                                         lsc, op_pre, fft1, op_mid, fft2);
             } else {
 #pragma unroll
                 for (int ln = 0; ln < LPT; ++ln)
