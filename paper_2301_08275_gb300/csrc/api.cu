@@ -144,7 +144,7 @@ struct gpe_plan {
     // trap tables of one time level (gpe_step_real_trap), allocated on first use
     void *sched[3] = {nullptr, nullptr, nullptr};
     void *sched_last = nullptr;
-    double *dtab = nullptr;                 // dither angles and offsets per step (resident kernel)
+    float *dtab = nullptr;                  // dither angles and offsets per step (resident kernel)
     // complex128 sweeps of 2D and 3D steps run in fixed point, on tables of their own
     bool fxp() const { return prec == GPE_C128 && ndim >= 2; }
 };
@@ -569,6 +569,11 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
         for (int64_t b = 0; b < B; ++b)
             for (int full = 0; full < 2; ++full) gq[2 * b + full] = coupling_fx(gs[b], full ? p->dt : 0.5 * p->dt);
         PLAN_TRY(upload_raw(p, &p->gq, gq.data(), gq.size() * sizeof(FxCoupling)));
+    } else {
+        std::vector<float> gq(2 * B);
+        for (int64_t b = 0; b < B; ++b)
+            for (int full = 0; full < 2; ++full) gq[2 * b + full] = (float)(gs[b] * (full ? p->dt : 0.5 * p->dt));
+        PLAN_TRY(upload_raw(p, &p->gq, gq.data(), gq.size() * sizeof(float)));
     }
 #undef PLAN_TRY
     p->gamma_host = gam;
@@ -784,7 +789,7 @@ static PassArgs make_pass(const gpe_plan *p, int axis, const void *src, void *ds
     a.vsamp = p->ndim >= 2 ? p->vsamp : nullptr;
     a.vsamp_diag = p->vsamp;
     a.g = p->g_dev;
-    a.inv_n = 1.0 / (double)p->N;
+    a.inv_n = (float)(1.0 / (double)p->N);
     // states of up to 64 MiB (1024^2 complex64 is 8 MiB): every sweep is one
     // short wave of CTAs, and the next kernel's launch may start with it
     // (1024^2 complex64 step 27.1 -> 25.5 us); larger states trigger it at
@@ -823,6 +828,15 @@ static void set_nreal(const gpe_plan *p, PassArgs &a, bool full)
     a.vt_o0 = o0 < p->ndim ? vt[o0] : nullptr;
     a.vt_o1 = o1 < p->ndim ? vt[o1] : nullptr;
     a.nl_c = full ? p->dt : 0.5 * p->dt;
+    a.nl_cf = (float)a.nl_c;
+}
+
+// an imaginary-time nonlinear half-step
+static void set_nimag(const gpe_plan *p, PassArgs &a)
+{
+    a.vq_full = 0;
+    a.nl_c = 0.5 * p->dt;
+    a.nl_cf = (float)a.nl_c;
 }
 
 // ------------------------------------------------------------------ tensor maps
@@ -998,6 +1012,8 @@ static cudaError_t plane_steps(gpe_plan *p, void *psi, int64_t nsteps, bool imag
         a.vf[i] = p->prec == GPE_C128 ? p->vq[i] : p->vf[i];
     }
     a.dt = p->dt;
+    a.dtf = (float)p->dt;
+    a.half_dtf = (float)(0.5 * p->dt);
     a.dv = p->dv;
     a.target = target;
     a.dither = !imag && p->prec == GPE_C64 && !p->no_dither;
@@ -1009,9 +1025,10 @@ static cudaError_t plane_steps(gpe_plan *p, void *psi, int64_t nsteps, bool imag
         for (int s = 0; a.dither && s < a.nsteps; ++s) {
             PassArgs k;
             memset(&k, 0, sizeof(k));
-            a.dphi[s] = dither_angle(s0 + s);
-            set_dither(k, a.dphi[s]);
-            for (int q = 0; q < 4; ++q) a.dk[s][q] = (float)k.dk[q];
+            const double phi = dither_angle(s0 + s);
+            set_dither(k, phi);
+            a.dphi[s] = (float)phi;
+            for (int q = 0; q < 4; ++q) a.dk[s][q] = k.dk[q];
         }
         TraceScope ts(p, "plane" + std::to_string(p->n[0]) + "x" + std::to_string(p->n[1]) + (imag ? ":imag" : ":real"));
         const cudaError_t e = p->prec == GPE_C64 ? launch_plane_f32((int)p->n[0], (int)p->n[1], a, p->st)
@@ -1136,7 +1153,7 @@ static gpe_status step_real_dev(gpe_plan *p, void *psi, int64_t nsteps, const do
             GPE_TRY(trap_level(p, p->sched, gamma_t, s + 1, last || p->fxp() ? 0.5 : 1.0));
             use_sched(p, x);
         }
-        x.dphi = phi;
+        x.dphi = (float)phi;
         x.fft2 = last ? 0 : -1;
         GPE_TRY(run(p, x));
         if (p->ndim == 3 && !last) {
@@ -1273,7 +1290,7 @@ static gpe_status step_real_host_slabs_enqueue(gpe_plan *p, unsigned char *host,
             x.fft1 = +1;
             x.op_mid = OP_NREAL;
             set_nreal(p, x, !last);
-            x.dphi = phi;
+            x.dphi = (float)phi;
             x.fft2 = last ? 0 : -1;
             if (last) {
                 GPE_TRY(slab_pass(x, 0, k));
@@ -1683,7 +1700,7 @@ static gpe_status imag_steps(gpe_plan *p, void *psi, int64_t nsteps, double targ
     for (int64_t s = 0; s < nsteps; ++s) {
         PassArgs x = make_pass(p, 0, psi, psi, B);
         x.op_pre = OP_SCALE_NIMAG;
-        x.nl_c = 0.5 * p->dt;
+        set_nimag(p, x);
         x.fft1 = -1;
         GPE_TRY(run(p, x));
         if (p->ndim == 3) {
@@ -1704,7 +1721,7 @@ static gpe_status imag_steps(gpe_plan *p, void *psi, int64_t nsteps, double targ
         PassArgs x2 = make_pass(p, 0, psi, psi, B);
         x2.fft1 = +1;
         x2.op_mid = OP_NIMAG;
-        x2.nl_c = 0.5 * p->dt;
+        set_nimag(p, x2);
         x2.red = RED_NORM;
         GPE_TRY(run(p, x2));
         cudaError_t e = launch_reduce_lines(p->partials, p->lines_cap, 0, 1, B, p->N / p->n[0], p->csum, p->sums,
@@ -1974,12 +1991,18 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
     double gm[3] = {0, 0, 0};
     for (int a = 0; a < p->ndim; ++a) gm[a] = gamma[a];
     GPE_CUDA(cudaMemcpyAsync(p->gamma_dev + 3 * slot, gm, sizeof(gm), cudaMemcpyHostToDevice, p->st));
-    if (p->prec == GPE_C128) {
-        FxCoupling gq[2];
-        for (int full = 0; full < 2; ++full) gq[full] = coupling_fx(g, full ? p->dt : 0.5 * p->dt);
-        GPE_CUDA(cudaMemcpyAsync((FxCoupling *)p->gq + 2 * slot, gq, sizeof(gq), cudaMemcpyHostToDevice, p->st));
-        GPE_CUDA(cudaStreamSynchronize(p->st));        // host staging goes out of scope
+    FxCoupling gx[2];
+    float gf[2];
+    for (int full = 0; full < 2; ++full) {
+        const double c = full ? p->dt : 0.5 * p->dt;
+        gx[full] = coupling_fx(g, c);
+        gf[full] = (float)(g * c);
     }
+    if (p->prec == GPE_C128)
+        GPE_CUDA(cudaMemcpyAsync((FxCoupling *)p->gq + 2 * slot, gx, sizeof(gx), cudaMemcpyHostToDevice, p->st));
+    else
+        GPE_CUDA(cudaMemcpyAsync((float *)p->gq + 2 * slot, gf, sizeof(gf), cudaMemcpyHostToDevice, p->st));
+    GPE_CUDA(cudaStreamSynchronize(p->st));        // host staging goes out of scope
     for (int a = 0; a < p->ndim; ++a) {
         if (!p->trap[a]) continue;
         const int64_t na = p->n[a];
@@ -2052,17 +2075,17 @@ gpe_status plan_prepare_resident(gpe_plan *p)
 {
     if (p->dtab) return GPE_OK;
     DeviceGuard dg(p->device);
-    std::vector<double> h(5 * (size_t)GPE_DITHER_PERIOD);
+    std::vector<float> h(5 * (size_t)GPE_DITHER_PERIOD);
     for (int64_t s = 0; s < GPE_DITHER_PERIOD; ++s) {
         PassArgs k;
         memset(&k, 0, sizeof(k));
         const double phi = dither_angle(s);
         set_dither(k, phi);
-        h[5 * s] = phi;
+        h[5 * s] = (float)phi;
         for (int q = 0; q < 4; ++q) h[5 * s + 1 + q] = k.dk[q];
     }
-    GPE_TRY(dalloc(p, (void **)&p->dtab, sizeof(double) * h.size()));
-    GPE_CUDA(cudaMemcpy(p->dtab, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice));
+    GPE_TRY(dalloc(p, (void **)&p->dtab, sizeof(float) * h.size()));
+    GPE_CUDA(cudaMemcpy(p->dtab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
     return GPE_OK;
 }
 

@@ -62,19 +62,23 @@ struct PassArgs {
     // trap angles in 2^-64 turns (int64; the full step doubles them, vq_full),
     // vi_* the half-step trap exponents V_a c log2(e) to 53 fraction bits
     // (int64), ki_ax exp(-k^2 dt/2) 2^-kiq_e to 62 bits (int64; ki_o0 and ki_o1
-    // stay double), gq the nonlinear coupling ([batch][half, full])
+    // stay double), gq the nonlinear coupling ([batch][half, full]; complex64:
+    // g nl_c as floats)
     const void *gq;
     int vq_full, kiq_e, lg_n;      // lg_n: log2 of the points of an instance
     const double *g;       // per-instance interaction
     double nl_c;           // theta = g * nl_c * |psi|^2
     // per-step phase dither of the complex64 real-time step: the kinetic
     // substep multiplies by exp(-i phi) as well (dk: its offset exp(-i phi) - 1
-    // as a hi, hi, lo, lo float quadruple stored in doubles) and the following
+    // as a hi, hi, lo, lo float quadruple) and the following
     // nonlinear substep by exp(+i phi) (dphi = phi); 0 when off
+    // (all complex64 scalars are rounded on the host: a conversion from double
+    // takes the FP64 pipe for 64 cycles per warp)
     int dither;
-    double dk[4];
-    double dphi;
-    double inv_n;          // 1/N applied with the kinetic substep
+    float dk[4];
+    float dphi;
+    float inv_n;           // 1/N applied with the kinetic substep
+    float nl_cf;           // nl_c
     // programmatic dependent launch: 1 lets the next kernel of the stream
     // start its launch as soon as every CTA of this one has begun (grids that
     // are resident at once: small states), 0 once every CTA has written its
@@ -135,7 +139,7 @@ struct ResidentArgs {
     const void *vh[2], *vf[2]; // trap tables of x and y (half and full steps), or NULL
     double dt;
     int dither;                // 1: the complex64 phase dither of the real-time step
-    const double *dtab;        // [GPE_DITHER_PERIOD][5]: phi, then the offset of exp(-i phi) as hi, hi, lo, lo
+    const float *dtab;         // [GPE_DITHER_PERIOD][5]: phi, then the offset of exp(-i phi) as hi, hi, lo, lo
 };
 cudaError_t launch_resident2d(int n, const ResidentArgs &a, cudaStream_t st);
 bool resident2d_supported(int prec, int ndim, const int64_t *n);
@@ -156,9 +160,10 @@ struct PlaneArgs {
     int64_t count;             // instances
     int nsteps, imag;
     int first, last;           // this launch opens / closes the call's real-time steps
+    float dtf, half_dtf;       // complex64: dt and dt / 2
     double dt, dv, target;     // imaginary time: cell volume and target norm
     int dither;
-    double dphi[PLANE_STEPS];
+    float dphi[PLANE_STEPS];
     float dk[PLANE_STEPS][4];
 };
 cudaError_t launch_plane_f32(int n0, int n1, const PlaneArgs &a, cudaStream_t st);

@@ -220,7 +220,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
     if (op == OP_KREAL) {
         // tables hold exp(-i k_a^2 dt/2) - 1; the 1/N of the inverse transform is exact
         const U *kt = static_cast<const U *>(a.kt_ax);
-        const R invn = (R)a.inv_n;
+        const R invn = a.inv_n;
         const U *k0 = static_cast<const U *>(a.kt_o0);
         const U *k1 = static_cast<const U *>(a.kt_o1);
         if (!k0 && !k1) {
@@ -233,7 +233,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
         U fl = offset_product(k0 ? k0[c0] : U{}, k1 ? k1[c1] : U{});
         if constexpr (sizeof(R) == 4) {
             if (a.dither)
-                fl = offset_product(fl, make_float4((float)a.dk[0], (float)a.dk[1], (float)a.dk[2], (float)a.dk[3]));
+                fl = offset_product(fl, make_float4(a.dk[0], a.dk[1], a.dk[2], a.dk[3]));
         }
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = cscale(uomul(uomul(v[e], kt[tl + TPL * e]), fl), invn);
@@ -254,7 +254,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
         for (int e = 0; e < E; ++e) v[e] = cscale(v[e], s);
         if (op == OP_SCALE) return;
     }
-    const R gc = (R)(a.g[ti] * a.nl_c);
+    const R gc = static_cast<const float *>(a.gq)[2 * ti + a.vq_full];
     if (op == OP_NREAL) {
         // trap tables hold exp(-i V_a c) - 1
         const U *vax = static_cast<const U *>(a.vt_ax);
@@ -265,10 +265,10 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
         // separate paths with and without a sampled potential keep the
         // common one free of its address arithmetic (fewer live registers)
         R th[E];
-        const R dphi = (R)a.dphi;      // undoes the kinetic substep's dither (0 when off)
+        const R dphi = a.dphi;      // undoes the kinetic substep's dither (0 when off)
         if (a.vsamp) {
             const R *vs = static_cast<const R *>(a.vsamp) + off;
-            const R cc = (R)a.nl_c;
+            const R cc = a.nl_cf;
 #pragma unroll
             for (int e = 0; e < E; ++e)
                 th[e] = fma(vs[(int64_t)(tl + TPL * e) * a.estride], cc, gc * cabs2(v[e])) - dphi;
@@ -294,7 +294,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
     if (a.vi_o0) fl *= static_cast<const R *>(a.vi_o0)[(int64_t)ti * a.o0n + c0];
     if (a.vi_o1) fl *= static_cast<const R *>(a.vi_o1)[(int64_t)ti * a.o1n + c1];
     const R *vs = static_cast<const R *>(a.vsamp);
-    const R cc = (R)a.nl_c;
+    const R cc = a.nl_cf;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         R th = gc * cabs2(v[e]);
@@ -814,6 +814,7 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
         }
         __syncthreads();
     }
+    const int64_t es = ROWS ? 1 : a.estride;     // between the points of a line
     int issued[2] = {0, 0};   // boxes sets issued into each buffer (thread 0)
     // Programmatic dependent launch: everything above (twiddles, barriers)
     // touches nothing the previous kernel of the stream writes, so it may
@@ -848,12 +849,22 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
         if (tile < a.ntiles) {
 #pragma unroll
             for (int ln = 0; ln < LPT; ++ln) {
+                if (ROWS && !a.inst_ptr) {
+                    // rows of back-to-back instances follow one another
+                    const int64_t lg = a.line0 + tile * L + l0 + ln;
+                    if (lg < a.lines_total) {
+                        const C *src = static_cast<const C *>(a.src) + lg * N + tl;
+#pragma unroll
+                        for (int e = 0; e < E; ++e) cp_async_point(buf + T::sidx_own(tl, e, l0 + ln), src + TPL * e);
+                    }
+                    continue;
+                }
                 const LineGeom g = line_geom<L>(a, tile, l0 + ln);
                 if (g.valid) {
                     const C *src = inst_src<C>(a, g.inst) + g.off;
 #pragma unroll
                     for (int e = 0; e < E; ++e)
-                        cp_async_point(buf + T::sidx_own(tl, e, l0 + ln), src + (int64_t)(tl + TPL * e) * a.estride);
+                        cp_async_point(buf + T::sidx_own(tl, e, l0 + ln), src + (int64_t)(tl + TPL * e) * es);
                 }
             }
         }
@@ -1096,7 +1107,7 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
                 if (g[ln].valid) {
                     C *dst = inst_dst<C>(a, g[ln].inst) + g[ln].off;
 #pragma unroll
-                    for (int e = 0; e < E; ++e) dst[(int64_t)(tl + TPL * e) * a.estride] = v[ln][e];
+                    for (int e = 0; e < E; ++e) dst[(int64_t)(tl + TPL * e) * es] = v[ln][e];
                 }
             }
         }

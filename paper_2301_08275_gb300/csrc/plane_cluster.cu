@@ -192,7 +192,8 @@ __global__ void __launch_bounds__(PlaneCfg<R, N0, N1>::NT) k_plane(const PlaneAr
             r.vt_o0 = pa.vh[1];
             r.nl_c = 0.5 * pa.dt;
             r.vq_full = 0;
-            r.dphi = 0.0;
+            r.dphi = 0.0f;
+            r.nl_cf = pa.half_dtf;
             row_sweep(r, OP_NREAL, -1, OP_NONE, 0);
             __syncthreads();
             clear();
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(PlaneCfg<R, N0, N1>::NT) k_plane(const PlaneAr
             if (sizeof(R) == 4) {
                 k.dither = pa.dither;
                 if (pa.dither)
-                    for (int q = 0; q < 4; ++q) k.dk[q] = (double)pa.dk[s][q];
+                    for (int q = 0; q < 4; ++q) k.dk[q] = pa.dk[s][q];
             }
             column_sweep(k, OP_KREAL);
             const bool last = pa.last && s == pa.nsteps - 1;
@@ -211,12 +212,15 @@ __global__ void __launch_bounds__(PlaneCfg<R, N0, N1>::NT) k_plane(const PlaneAr
             r.vt_o0 = last ? pa.vh[1] : pa.vf[1];
             r.nl_c = last ? 0.5 * pa.dt : pa.dt;
             r.vq_full = last ? 0 : 1;
-            r.dphi = sizeof(R) == 4 && pa.dither ? pa.dphi[s] : 0.0;
+            r.dphi = sizeof(R) == 4 && pa.dither ? pa.dphi[s] : 0.0f;
+            r.nl_cf = last ? pa.half_dtf : pa.dtf;
             row_sweep(r, OP_NONE, 1, OP_NREAL, last ? 0 : -1);
         }
     } else {
         PassArgs r = pa.rows;
         r.nl_c = 0.5 * pa.dt;
+        r.vq_full = 0;
+        r.nl_cf = pa.half_dtf;
 #pragma unroll 1
         for (int s = 0; s < pa.nsteps; ++s) {
             row_sweep(r, OP_NIMAG, -1, OP_NONE, 0);

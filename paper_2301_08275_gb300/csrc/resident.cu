@@ -93,8 +93,8 @@ __global__ void __launch_bounds__(ResidentCfg<N>::NT, 1) k_resident2d(const Resi
             *sa = ra.rows;
             sa->vt_ax = ra.vh[0];
             sa->vt_o0 = ra.vh[1];
-            sa->nl_c = 0.5 * ra.dt;
-            sa->dphi = 0.0;
+            sa->vq_full = 0;
+            sa->dphi = 0.0f;
         }
         __syncthreads();
         rows(OP_NREAL, -1, OP_NONE, 0);
@@ -115,8 +115,8 @@ __global__ void __launch_bounds__(ResidentCfg<N>::NT, 1) k_resident2d(const Resi
                 *sa = ra.rows;
                 sa->vt_ax = last ? ra.vh[0] : ra.vf[0];
                 sa->vt_o0 = last ? ra.vh[1] : ra.vf[1];
-                sa->nl_c = last ? 0.5 * ra.dt : ra.dt;
-                sa->dphi = ra.dither ? ra.dtab[5 * d] : 0.0;
+                sa->vq_full = last ? 0 : 1;
+                sa->dphi = ra.dither ? ra.dtab[5 * d] : 0.0f;
             }
             __syncthreads();
             rows(OP_NONE, +1, OP_NREAL, last ? 0 : -1);
