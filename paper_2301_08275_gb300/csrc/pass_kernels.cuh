@@ -1135,25 +1135,41 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
 __host__ __device__ constexpr size_t line1d_red_bytes(int nt) { return (sizeof(double) * (size_t)nt + 15) / 16 * 16; }
 
 // Each line is one instance and stays in registers for all nsteps steps of
-// the launch; real time merges consecutive nonlinear half-steps, imaginary
-// time renormalises the line after every step.
+// the launch; real time (complex64; complex128 takes k_line1d_fx) merges
+// consecutive nonlinear half-steps, imaginary time renormalises the line after
+// every step.  Twiddles lie in pass order (in natural order the reads of the
+// later passes were up to 8-way bank conflicts: 64 lines of 4096 points 11.0
+// us per step, now 5.1; one line of 256 points 1.24, now 1.07); a second
+// exchange region saves a barrier per pass where it fits.
+template <typename R, int N, int L> struct Line1DCfg {
+    using T = GTile<R, N, 1, 1, true>;        // one line per thread group, swizzled exchange
+    static constexpr int NT = L * T::TPL;
+    static constexpr size_t buf = sizeof(typename T::C) * N * L;
+    static constexpr size_t base = buf + line1d_red_bytes(NT) + sizeof(typename T::U) * N;
+    static constexpr bool PING = T::PL::P > 1 && base + buf <= 200 * 1024;
+    static constexpr size_t smem = base + (PING ? buf : 0);
+};
 template <typename R, int N, int L>
-__global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1DArgs a)
+__global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DArgs a)
 {
-    using T = Tile<R, N, L, true>;
+    using Cfg = Line1DCfg<R, N, L>;
+    using T = typename Cfg::T;
     using C = typename T::C;
     constexpr int E = T::E, TPL = T::TPL;
+    constexpr bool PING = Cfg::PING;
     using U = typename T::U;
     if (a.stop && *reinterpret_cast<const volatile int *>(a.stop)) return;   // see k_pass
     extern __shared__ __align__(128) unsigned char smraw[];
-    C *sm = reinterpret_cast<C *>(smraw);
-    double *red = reinterpret_cast<double *>(smraw + sizeof(C) * T::SMEM_POINTS);
+    constexpr int NT = Cfg::NT;
+    const int t = threadIdx.x, l = t / TPL, tl = t % TPL;
+    C *const sm = reinterpret_cast<C *>(smraw) + l * N;
+    C *const ss = PING ? sm + L * N : sm;
     // the reduction scratch is rounded up to 16 bytes so that the 16-byte
     // twiddle entries after it stay aligned (tiles of one short line have an
     // odd thread count)
-    U *tw = reinterpret_cast<U *>(smraw + sizeof(C) * T::SMEM_POINTS + line1d_red_bytes(T::NT));
-    const int t = threadIdx.x, l = T::line_of(t), tl = T::tl_of(t);
-    for (int i = t; i < N; i += T::NT) tw[i] = static_cast<const U *>(a.tw)[i];
+    double *red = reinterpret_cast<double *>(smraw + (PING ? 2 : 1) * Cfg::buf);
+    U *tw = reinterpret_cast<U *>(reinterpret_cast<unsigned char *>(red) + line1d_red_bytes(NT));
+    T::load_twiddles(tw, static_cast<const U *>(a.tw), t, NT);
     __syncthreads();
     const int64_t ntiles = (a.batch + L - 1) / L;
 
@@ -1164,7 +1180,8 @@ __global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1D
         // instance storage and its parameter/table slot
         C *psi = a.inst_ptr ? static_cast<C *>(a.inst_ptr[ip]) : static_cast<C *>(a.psi) + ip * N;
         const int64_t ib = a.slot_of ? a.slot_of[ip] : ip;
-        C v[E];
+        C w[1][E];
+        C(&v)[E] = w[0];
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = valid ? psi[tl + TPL * e] : mk((R)0, (R)0);
         const double g = a.g[ib];
@@ -1186,10 +1203,10 @@ __global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1D
                 if (vh) v[e] = uomul(v[e], vh[ib * N + tl + TPL * e]);
 #pragma unroll 1
             for (int64_t st = 0; st < a.nsteps; ++st) {
-                T::template fft<-1>(v, sm, tl, l, tw);
+                T::template fft<-1, PING>(w, sm, ss, tl, 0, tw);
 #pragma unroll
                 for (int e = 0; e < E; ++e) v[e] = cscale(uomul(v[e], kt[tl + TPL * e]), invn);
-                T::template fft<1>(v, sm, tl, l, tw);
+                T::template fft<1, PING>(w, sm, ss, tl, 0, tw);
                 const bool last = (st == a.nsteps - 1);
                 const R gc = last ? gh : gf;
                 const U *vt = last ? (a.vh_last ? static_cast<const U *>(a.vh_last) : vh) : vf;
@@ -1215,10 +1232,10 @@ __global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1D
                     if (vi) f *= vi[ib * N + tl + TPL * e];
                     v[e] = cscale(x, f);
                 }
-                T::template fft<-1>(v, sm, tl, l, tw);
+                T::template fft<-1, PING>(w, sm, ss, tl, 0, tw);
 #pragma unroll
                 for (int e = 0; e < E; ++e) v[e] = cscale(v[e], ki[tl + TPL * e]);
-                T::template fft<1>(v, sm, tl, l, tw);
+                T::template fft<1, PING>(w, sm, ss, tl, 0, tw);
                 double nrm = 0.0;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
@@ -1242,6 +1259,7 @@ __global__ void __launch_bounds__(Tile<R, N, L, true>::NT) k_line1d(const Line1D
 #pragma unroll
             for (int e = 0; e < E; ++e) psi[tl + TPL * e] = v[e];
         }
+        __syncthreads();         // the exchange regions are reused
     }
 }
 
@@ -1431,16 +1449,17 @@ static int sm_count()
 
 template <typename R, int N, int L> static cudaError_t launch_line1d_l(const Line1DArgs &a, cudaStream_t st)
 {
-    using T = Tile<R, N, L, true>;
+    using T = typename Line1DCfg<R, N, L>::T;
+    static_assert(T::layout_consistent(), "shared layout of the exchanges");
     static LaunchCache lc;
-    const size_t smem = sizeof(typename T::C) * T::SMEM_POINTS + line1d_red_bytes(T::NT) + sizeof(typename T::U) * N;
+    const size_t smem = Line1DCfg<R, N, L>::smem;
     int cap = 0;
-    cudaError_t e = prepare(k_line1d<R, N, L>, lc, T::NT, smem, &cap);
+    cudaError_t e = prepare(k_line1d<R, N, L>, lc, Line1DCfg<R, N, L>::NT, smem, &cap);
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (a.batch + L - 1) / L;
     if (ntiles <= 0) return cudaSuccess;
     const int grid = (int)(ntiles < cap ? ntiles : cap);
-    k_line1d<R, N, L><<<grid, T::NT, smem, st>>>(a);
+    k_line1d<R, N, L><<<grid, Line1DCfg<R, N, L>::NT, smem, st>>>(a);
     return cudaGetLastError();
 }
 
