@@ -16,11 +16,14 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgpe.so")
-SOURCES = ["pass_f32_w512_0.cu", "pass_f32_w512_1.cu", "pass_f32_w1024_0.cu", "pass_f32_w1024_1.cu",
-           "pass_f32_w256_0.cu", "pass_f32_w256_1.cu", "pass_f32.cu", "pass_f32_s1.cu", "pass_f32_rows.cu",
-           "pass_f32_rows1.cu", "pass_f64.cu", "pass_f64_s1.cu", "pass_f64_rows.cu", "pass_f64_rows1.cu",
-           "diag_spec.cu", "api.cu", "noalloc.cu", "serve.cu", "peak.cu", "resident.cu", "line_cluster.cu",
-           "plane_cluster.cu", "plane_cluster_f64.cu"]
+SOURCES = ["pass_f32_s1024_0.cu", "pass_f32_s1024_1.cu", "pass_f32_s512_0.cu", "pass_f32_s512_1.cu",
+           "pass_f32_s256_0.cu", "pass_f32_s256_1.cu", "pass_f32_s64.cu", "pass_f32_s2048.cu",
+           "pass_f32_r1024.cu", "pass_f32_r512.cu", "pass_f32_r256.cu", "pass_f32_r64.cu", "pass_f32_r2048.cu",
+           "pass_f64_s1024.cu", "pass_f64_s512.cu", "pass_f64_s256.cu", "pass_f64_s128.cu", "pass_f64_s64.cu",
+           "pass_f64_s2048.cu", "pass_f64_r1024.cu", "pass_f64_r512.cu", "pass_f64_r256.cu",
+           "pass_f64_r128.cu", "pass_f64_r64.cu", "pass_f64_r2048.cu", "line1d_f64.cu", "line1d_f32.cu",
+           "pass_f32.cu", "pass_f64.cu", "plane_cluster_f64.cu", "plane_cluster.cu", "diag_spec.cu", "api.cu",
+           "noalloc.cu", "serve.cu", "peak.cu", "resident.cu", "line_cluster.cu"]
 HEADERS = ["plane_cluster.cu", "fx.cuh", "fft_tile.cuh", "pass_kernels.cuh", "gpe_internal.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]

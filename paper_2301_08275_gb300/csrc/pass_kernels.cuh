@@ -98,7 +98,8 @@ __device__ __forceinline__ void apply_phase(C (&v)[E], const R (&th)[E])
 // 512^3 grid, whose consecutive points are 2 MiB apart, ran at under half the
 // copy bandwidth.  VAR 1: 4096 points / 8 lines, two CTAs per SM.
 // complex128 VAR 0: 2048 points / 4 lines (64-byte pieces), two CTAs per SM;
-// VAR 1: 4096 points / 8 lines.
+// VAR 1: shorter than 512 points, tiles of 512 points (at most 4 lines), for
+// grids of few tiles (256^2: 20.6 -> 16.3 us per step); else 4096 points / 8 lines.
 // Contiguous rows (x).  A split tile holds a fraction of the points and lines
 // with the swizzled shared layout and several CTAs per SM: each lane's points
 // lie in its own row, and fewer rows per warp request with longer pieces of
@@ -118,7 +119,10 @@ template <typename R, int N, bool ROWS, int VAR> __host__ __device__ constexpr i
 {
     constexpr bool c64 = sizeof(R) == 4;
     int maxpts = c64 ? 4096 : 2048, lmax = c64 ? 8 : 4;
-    if (ROWS) {
+    if (!c64 && VAR == 1 && N < 512) {
+        // small tiles: grids too small to give every SM a tile of shape 0
+        maxpts = 512;
+    } else if (ROWS) {
         if (rows_split<R, N, ROWS, VAR>()) {
             // complex64 rows of 256 or 512 points: tiles of 512 points (shape 0:
             // 2 rows of 256, 1 row of 512) or 4 rows (shape 1)
@@ -1407,11 +1411,13 @@ static cudaError_t launch_pass_p(const PassArgs &a, cudaStream_t st, const CUten
     return cudaLaunchKernelEx(&cfg, k_pass<R, N, ROWS, VAR, PROG>, a, tmap ? *tmap : none);
 }
 
-// complex64 lines of 256 to 1024 points (the large grids) get the fixed-program
-// kernels of the sweeps they run; everything else the generic one
+// Lines of at least 64 points (complex128: to 1024) get the fixed-program kernels
+// of the sweeps they run; everything else the generic one, which carries the
+// registers and the code of every program.  Measured, us per complex64 step,
+// generic / fixed: 64^3 21.2 / 17.3, four 128^3 193 / 152.
 template <typename R, int N, bool ROWS> constexpr bool sweep_progs_compiled()
 {
-    return sizeof(R) == 4 && N >= 256 && N <= 1024;
+    return N >= 64 && (sizeof(R) == 4 || N <= 1024);
 }
 template <typename R, int N, bool ROWS, int VAR>
 static cudaError_t launch_pass_t(const PassArgs &a, cudaStream_t st, const CUtensorMap *tmap)
@@ -1503,19 +1509,20 @@ template <typename R, int N> static cudaError_t launch_line1d_t(const Line1DArgs
 
 #define GPE_FOR_EACH_N(X) X(2) X(4) X(8) X(16) X(32) X(64) X(128) X(256) X(512) X(1024) X(2048) X(4096)
 
-// Strided complex64 lines of 256 to 1024 points (radix-32 kernels, the
-// longest to compile) are instantiated in translation units of their own,
-// one per line length and tile shape (pass_f32_w<N>_<VAR>.cu), so that the
-// library builds in parallel.
-template <int N, int VAR> cudaError_t launch_pass_wide_f32(const PassArgs &a, cudaStream_t st, const CUtensorMap *tmap);
-template <typename R, int N, bool ROWS> constexpr bool pass_wide_tu()
-{
-    return sizeof(R) == 4 && !ROWS && N >= 256 && N <= 1024;
-}
+// Lines of at least 64 points are instantiated in translation units of their
+// own, a few lengths each (pass_f32_*.cu, pass_f64_*.cu), so that the library
+// builds in parallel.
+template <typename R, int N, bool ROWS, int VAR>
+cudaError_t launch_pass_tu(const PassArgs &a, cudaStream_t st, const CUtensorMap *tmap);
+#define GPE_PASS_TU(R, N, ROWS, VAR)                                                                               \
+    template <> cudaError_t launch_pass_tu<R, N, ROWS, VAR>(const PassArgs &a, cudaStream_t st, const CUtensorMap *tmap) \
+    {                                                                                                              \
+        return launch_pass_t<R, N, ROWS, VAR>(a, st, tmap);                                                        \
+    }
 template <typename R, int N, bool ROWS, int VAR>
 static cudaError_t launch_pass_n(const PassArgs &a, cudaStream_t st, const CUtensorMap *tmap)
 {
-    if constexpr (pass_wide_tu<R, N, ROWS>()) return launch_pass_wide_f32<N, VAR>(a, st, tmap);
+    if constexpr (N >= 64) return launch_pass_tu<R, N, ROWS, VAR>(a, st, tmap);
     else return launch_pass_t<R, N, ROWS, VAR>(a, st, tmap);
 }
 
