@@ -111,6 +111,7 @@ struct gpe_plan {
     size_t pin_len = 0;
     void *work[4] = {};
     double *hist = nullptr, *spec_out = nullptr;
+    float *dk = nullptr;                    // derivative wavenumbers of x, y, z (complex64 spectra)
     void *host_buf = nullptr;    // device copy for gpe_step_real_host
     // slab pipeline of gpe_step_real_host: a copy stream and one event per slab and direction
     cudaStream_t copy_st = nullptr;
@@ -1880,11 +1881,13 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
     double *slot[4] = {nullptr, nullptr, nullptr, nullptr};
     std::vector<double> tmp(2 * ns);
     // bin the given fields and write shells (scaled) into o0 / o1 (either may be NULL)
-    auto bin_out = [&](void *const *uh, int split, int ncomp, double scale, double *o0, double *o1) -> gpe_status {
+    // (sq: nsq numbers whose sum times `total` is the sum of squares of the fields)
+    auto bin_out = [&](void *const *uh, int split, int ncomp, const double *sq, int nsq, double total, double scale,
+                       double *o0, double *o1) -> gpe_status {
         SpecArgs sb = sa;
         sb.split = split;
         sb.ncomp = ncomp;
-        cudaError_t e = launch_bin(sb, uh, ns, partial, ncomp * nv, p->hist, 0.5 * p->dv / (double)p->N, p->spec_out,
+        cudaError_t e = launch_bin(sb, uh, ns, sq, nsq, total, p->hist, 0.5 * p->dv / (double)p->N, p->spec_out,
                                    p->st);
         if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
         GPE_CUDA(cudaMemcpyAsync(tmp.data(), p->spec_out, sizeof(double) * 2 * ns, cudaMemcpyDeviceToHost, p->st));
@@ -1895,20 +1898,75 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
                 for (int64_t s2 = 0; s2 < nshells; ++s2) o[k][s2] = s2 < ns ? scale * tmp[k * ns + s2] : 0.0;
         return GPE_OK;
     };
-    // derivative fields -> u (part 0) or w (part 1) -> their transforms, in work[1..ndim]
+    // derivative fields -> u (part 0) or w (part 1) -> their transforms, in
+    // work[1..ndim], and the sums of squares of each component
+    //
+    // complex64 grids of 2D and 3D whose sweeps have compiled programs: the
+    // factor i k is a substep of the inverse transform's first sweep and the
+    // velocity one of the forward transform's, with the squares per row (a
+    // separate kernel each read and wrote the field once more: 50 of 185 us of
+    // a 1024^2 spectrum)
+    bool fused = p->prec == GPE_C64 && p->ndim >= 2 && !p->generic_passes;
+    for (int a = 0; a < p->ndim; ++a) fused = fused && p->n[a] >= 64;
+    const int64_t lines = p->N / p->n[0], sqcap = lines > REDUCE_CHUNK ? p->lines_cap : lines;
+    if (fused && !p->dk) {
+        std::vector<float> dk;
+        for (int a = 0; a < p->ndim; ++a)
+            for (int64_t j = 0; j < p->n[a]; ++j)
+                dk.push_back(2 * j == p->n[a] ? 0.0f : (float)(p->kf[a] * (double)(j < p->n[a] / 2 ? j : j - p->n[a])));
+        GPE_TRY(dalloc(p, (void **)&p->dk, dk.size() * sizeof(float)));
+        GPE_CUDA(cudaMemcpy(p->dk, dk.data(), dk.size() * sizeof(float), cudaMemcpyHostToDevice));
+    }
     auto gradient_parts = [&](const void *pb, int part) -> gpe_status {
         SpecArgs sv = sa;
         sv.part = part;
+        const float *dk = p->dk;
         for (int a = 0; a < p->ndim; ++a) {
-            cudaError_t e = launch_deriv(sa, p->work[0], p->work[1 + a], a, p->st);
+            void *w = p->work[1 + a];
+            if (fused) {
+                for (int ax = 0; ax < p->ndim; ++ax) {
+                    PassArgs t = make_pass(p, ax, ax == 0 ? p->work[0] : w, w, 1);
+                    t.fft1 = +1;
+                    if (ax == 0) {
+                        t.op_pre = OP_DERIV;
+                        (a == 0 ? t.dk_ax : a == 1 ? t.dk_o0 : t.dk_o1) = dk;
+                    }
+                    GPE_TRY(run(p, t));
+                }
+                dk += p->n[a];
+                for (int ax = 0; ax < p->ndim; ++ax) {
+                    PassArgs t = make_pass(p, ax, w, w, 1);
+                    t.fft1 = -1;
+                    if (ax == 0) {
+                        t.op_pre = OP_VEL;
+                        t.red = RED_NORM;
+                        t.partials = p->partials + a * sqcap;
+                        t.vel_psi = pb;
+                        t.vel_part = part;
+                    }
+                    GPE_TRY(run(p, t));
+                }
+            } else {
+                cudaError_t e = launch_deriv(sa, p->work[0], w, a, p->st);
+                if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
+                GPE_TRY(fft_nd(p, w, w, +1));
+                e = launch_velocity(sv, pb, w, partial + (size_t)a * nv, p->st);
+                if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
+                GPE_TRY(fft_nd(p, w, w, -1));
+            }
+        }
+        // every block of the binning kernel adds the sums up: not more than a few thousand
+        if (fused && lines > REDUCE_CHUNK) {
+            cudaError_t e = launch_reduce_lines(p->partials, sqcap, 0, p->ndim, 1, lines, p->csum, p->sums, p->st);
             if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
-            GPE_TRY(fft_nd(p, p->work[1 + a], p->work[1 + a], +1));
-            e = launch_velocity(sv, pb, p->work[1 + a], partial + (size_t)a * nv, p->st);
-            if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
-            GPE_TRY(fft_nd(p, p->work[1 + a], p->work[1 + a], -1));
         }
         return GPE_OK;
     };
+    const bool reduced = fused && lines > REDUCE_CHUNK;
+    const double *sq = reduced ? p->sums : fused ? p->partials : partial;
+    // Parseval: the fields are transformed over all axes, the rows' squares over x
+    const double sqtotal = fused ? (double)(p->N / p->n[0]) : (double)p->N;
+    const int nsq = p->ndim * (reduced ? 1 : fused ? (int)lines : nv);
     void *uh[3] = {p->work[1], p->ndim > 1 ? p->work[2] : nullptr, p->ndim > 2 ? p->work[3] : nullptr};
     for (int64_t b = 0; b < p->batch; ++b) {
         int kslot = 0;
@@ -1925,15 +1983,15 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
             sn.part = 2;
             cudaError_t e = launch_velocity(sn, pb, nullptr, partial, p->st);
             if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
-            GPE_TRY(bin_out(ph, 0, 1, 2.0, slot[3], nullptr));
+            GPE_TRY(bin_out(ph, 0, 1, partial, nv, (double)p->N, 2.0, slot[3], nullptr));
         }
         if (slot[0] || slot[1]) {
             GPE_TRY(gradient_parts(pb, 0));
-            GPE_TRY(bin_out(uh, 1, p->ndim, 1.0, slot[0], slot[1]));
+            GPE_TRY(bin_out(uh, 1, p->ndim, sq, nsq, sqtotal, 1.0, slot[0], slot[1]));
         }
         if (slot[2]) {
             GPE_TRY(gradient_parts(pb, 1));
-            GPE_TRY(bin_out(uh, 0, p->ndim, 1.0, slot[2], nullptr));
+            GPE_TRY(bin_out(uh, 0, p->ndim, sq, nsq, sqtotal, 1.0, slot[2], nullptr));
         }
     }
     return GPE_OK;

@@ -205,14 +205,17 @@ __global__ void k_deriv(const SpecArgs s, const typename CT<R>::C *__restrict__ 
     }
 }
 
-// sum of one double per thread of a 256-thread block, in a fixed order; thread 0 has it
+// sum of one double per thread of a block, in a fixed order; thread 0 has it
 __device__ __forceinline__ double block_sum(double s, double *sh)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
-    return ((sh[0] + sh[1]) + (sh[2] + sh[3])) + ((sh[4] + sh[5]) + (sh[6] + sh[7]));
+    double r = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
+    return r;
 }
 
 // w <- u = Im(conj(psi) * w / N) / |psi| (part 0) or Re(...) / |psi| (part 1: the
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(256) k_velocity(const SpecArgs s, const typena
         const R rho = p.x * p.x + p.y * p.y;
         if (s.part == 2) return sqrt(rho);
         const C d = w[i];
-        R u = (R)0;
+        R u = (R)0;      // as velocity_of (pass_kernels.cuh)
         if (rho >= (R)1e-30) u = (s.part ? (p.x * d.x + p.y * d.y) : (p.x * d.y - p.y * d.x)) * invn / sqrt(rho);
         return u;
     };
@@ -260,7 +263,7 @@ __global__ void __launch_bounds__(256) k_velocity(const SpecArgs s, const typena
 // over the k grid.  Shell sums are accumulated in 64-bit fixed point so that
 // they do not depend on the order in which threads and blocks add (integer
 // addition is associative).  The scale is the power of two that maps the
-// field's total, N sum u^2 (Parseval, from k_velocity's partial sums), below
+// field's total (Parseval, from the sums of squares in real space), below
 // 2^61; rounding costs at most total * 2^-62 per point, of either sign.
 //
 // FP64 arithmetic bounded this kernel (about 100 FP64 operations a point with
@@ -346,25 +349,31 @@ __device__ __forceinline__ double field_scale(double total, int prec)
     return ldexp(1.0, -h);
 }
 
+//
+// Modes +-m of every axis share their shell and their q up to signs: a thread
+// takes all of them (4 points in 2D, 8 in 3D) and divides, converts and adds
+// once.  Warps take runs of 32 consecutive m_x >= 0 of a row of (m_y, m_z) >= 0.
+constexpr int BIN_THREADS = 512;
 template <typename R>
-__global__ void __launch_bounds__(256) k_bin(const SpecArgs s, const typename CT<R>::C *__restrict__ u0,
-                                             const typename CT<R>::C *__restrict__ u1,
-                                             const typename CT<R>::C *__restrict__ u2, int nshells,
-                                             const double *__restrict__ partial, int npartial,
-                                             unsigned long long *__restrict__ hist, double *__restrict__ scale_out)
+__global__ void __launch_bounds__(BIN_THREADS) k_bin(const SpecArgs s, const typename CT<R>::C *__restrict__ u0,
+                                                     const typename CT<R>::C *__restrict__ u1,
+                                                     const typename CT<R>::C *__restrict__ u2, int nshells,
+                                                     const double *__restrict__ partial, int npartial, double total,
+                                                     unsigned long long *__restrict__ hist,
+                                                     double *__restrict__ scale_out)
 {
     using C = typename CT<R>::C;
     using W = Wide<R>;
     using T = typename W::T;
     extern __shared__ unsigned long long shq[];   // [2][nshells]
-    __shared__ double shd[8], shs;
+    __shared__ double shd[BIN_THREADS / 32], shs;
     const int nsum = (s.split ? 2 : 1) * nshells;
-    for (int i = threadIdx.x; i < nsum; i += 256) shq[i] = 0ull;
+    for (int i = threadIdx.x; i < nsum; i += BIN_THREADS) shq[i] = 0ull;
     double t = 0.0;
-    for (int i = threadIdx.x; i < npartial; i += 256) t += partial[i];
+    for (int i = threadIdx.x; i < npartial; i += BIN_THREADS) t += partial[i];
     t = block_sum(t, shd);
     if (threadIdx.x == 0) {
-        shs = field_scale(t * (double)s.N, s.prec);
+        shs = field_scale(t * total, s.prec);
         // a field that is not finite has no spectrum
         if (blockIdx.x == 0) *scale_out = isfinite(t) ? shs : __longlong_as_double(0x7ff8000000000000ll);
     }
@@ -373,27 +382,31 @@ __global__ void __launch_bounds__(256) k_bin(const SpecArgs s, const typename CT
     const C *const u[3] = {u0, u1, u2};
     const int lane = threadIdx.x & 31;
     const T lr[3] = {W::make(s.lratio[0]), W::make(s.lratio[1]), W::make(s.lratio[2])};
+    const int n[3] = {1 << s.lg[0], 1 << s.lg[1], 1 << s.lg[2]};
+    const int h0 = n[0] / 2 + 1, h1 = n[1] / 2 + 1, h2 = n[2] / 2 + 1;      // modes 0 .. n/2 (one for an absent axis)
+    const int chunks = (h0 + 31) / 32;
+    const int64_t units = (int64_t)chunks * h1 * h2;
+    const int nc = s.split ? s.ndim : s.ncomp;
     // whole warps run every iteration (the shuffles below)
-    const int64_t step = (int64_t)gridDim.x * 256;
-    for (int64_t i0 = blockIdx.x * (int64_t)256 + (threadIdx.x & ~31); i0 < s.N; i0 += step) {
-        const int64_t i = i0 + lane;
-        const bool on = i < s.N;
+    for (int64_t w = blockIdx.x * (int64_t)(BIN_THREADS / 32) + (threadIdx.x >> 5); w < units;
+         w += (int64_t)gridDim.x * (BIN_THREADS / 32)) {
+        const int row = (int)(w / chunks);
+        int m[3];
+        m[0] = (int)(w - (int64_t)row * chunks) * 32 + lane;
+        m[2] = row / h1;
+        m[1] = row - m[2] * h1;
+        const bool on = m[0] < h0;
         long long ei = 0, ec = 0;
         int shell = -1;
         if (on) {
-            int m[3] = {0, 0, 0};
-            for (int a = 0; a < s.ndim; ++a) {
-                const int j = axis_index(i, s, a), na = 1 << s.lg[a];
-                m[a] = j < na / 2 ? j : j - na;
-            }
             T q[3], q2;
             if (s.cubic) {
                 const int k2 = m[0] * m[0] + m[1] * m[1] + m[2] * m[2];
                 // floor(sqrt(k2) + 1/2) = n  <=>  n^2 - n < k2 <= n^2 + n (or n = 0 = k2)
-                int n = (int)(sqrtf((float)k2) + 0.5f);
-                if (n > 0 && k2 <= n * n - n) --n;
-                if (k2 > n * n + n) ++n;
-                shell = n;
+                int r = (int)(sqrtf((float)k2) + 0.5f);
+                if (r > 0 && k2 <= r * r - r) --r;
+                if (k2 > r * r + r) ++r;
+                shell = r;
                 q2 = W::whole((R)k2);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) q[a] = W::whole((R)m[a]);
@@ -415,28 +428,52 @@ __global__ void __launch_bounds__(256) k_bin(const SpecArgs s, const typename CT
                     shell = (int)floor(sqrt(d2) + 0.5);
                 }
             }
-            R re[3] = {(R)0, (R)0, (R)0}, im[3] = {(R)0, (R)0, (R)0};
-            const int nc = s.split ? s.ndim : s.ncomp;
-            for (int a = 0; a < nc; ++a) {
-                const C v = u[a][i];
-                re[a] = v.x * sc;
-                im[a] = v.y * sc;
-            }
-            if (!s.split || (m[0] | m[1] | m[2]) == 0) {
-                T e = W::whole((R)0);
+            const bool parts = s.split && (m[0] | m[1] | m[2]) != 0;
+            T si = W::whole((R)0), scp = W::whole((R)0);
+            // sign of every axis; modes 0 and n/2 (the Nyquist mode, -n/2) have one
+            const int k0 = m[0] == 0 || 2 * m[0] == n[0] ? 1 : 2, k1 = m[1] == 0 || 2 * m[1] == n[1] ? 1 : 2,
+                      k2s = m[2] == 0 || 2 * m[2] == n[2] ? 1 : 2;
+            for (int c2 = 0; c2 < k2s; ++c2)
+                for (int c1 = 0; c1 < k1; ++c1)
+                    for (int c0 = 0; c0 < k0; ++c0) {
+                        const int64_t i = (int64_t)(c0 ? n[0] - m[0] : m[0]) +
+                                          ((int64_t)(c1 ? n[1] - m[1] : m[1]) << s.lg[0]) +
+                                          ((int64_t)(c2 ? n[2] - m[2] : m[2]) << (s.lg[0] + s.lg[1]));
+                        const R sg[3] = {c0 || 2 * m[0] == n[0] ? -sc : sc, c1 || 2 * m[1] == n[1] ? -sc : sc,
+                                         c2 || 2 * m[2] == n[2] ? -sc : sc};
+                        R re[3] = {(R)0, (R)0, (R)0}, im[3] = {(R)0, (R)0, (R)0};
+                        for (int a = 0; a < nc; ++a) {
+                            const C v = u[a][i];
+                            // q_a carries its sign through the component (all products below are even in it)
+                            re[a] = v.x * (parts ? sg[a] : sc);
+                            im[a] = v.y * (parts ? sg[a] : sc);
+                        }
+                        if (!parts) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) e = W::add(e, W::add(W::sq(W::whole(re[a])), W::sq(W::whole(im[a]))));
-                ei = W::fixed(e);
+                            for (int a = 0; a < 3; ++a)
+                                si = W::add(si, W::add(W::sq(W::whole(re[a])), W::sq(W::whole(im[a]))));
+                            continue;
+                        }
+                        auto cross = [&](const R *v, int a, int b) {
+                            return W::add(W::mul(q[a], v[b]), W::neg(W::mul(q[b], v[a])));
+                        };
+                        auto dot = [&](const R *v) {
+                            T d = W::add(W::mul(q[0], v[0]), W::mul(q[1], v[1]));
+                            if (s.ndim > 2) d = W::add(d, W::mul(q[2], v[2]));
+                            return d;
+                        };
+                        si = W::add(si, W::add(W::sq(cross(re, 0, 1)), W::sq(cross(im, 0, 1))));
+                        if (s.ndim > 2) {
+                            si = W::add(si, W::add(W::sq(cross(re, 0, 2)), W::sq(cross(im, 0, 2))));
+                            si = W::add(si, W::add(W::sq(cross(re, 1, 2)), W::sq(cross(im, 1, 2))));
+                        }
+                        scp = W::add(scp, W::add(W::sq(dot(re)), W::sq(dot(im))));
+                    }
+            if (parts) {
+                ei = W::fixed(W::div(si, q2));
+                ec = W::fixed(W::div(scp, q2));
             } else {
-                auto cross = [&](const R *v, int a, int b) { return W::add(W::mul(q[a], v[b]), W::neg(W::mul(q[b], v[a]))); };
-                auto dot = [&](const R *v) { return W::add(W::add(W::mul(q[0], v[0]), W::mul(q[1], v[1])), W::mul(q[2], v[2])); };
-                T in = W::add(W::sq(cross(re, 0, 1)), W::sq(cross(im, 0, 1)));
-                if (s.ndim > 2) {
-                    in = W::add(in, W::add(W::sq(cross(re, 0, 2)), W::sq(cross(im, 0, 2))));
-                    in = W::add(in, W::add(W::sq(cross(re, 1, 2)), W::sq(cross(im, 1, 2))));
-                }
-                ei = W::fixed(W::div(in, q2));
-                ec = W::fixed(W::div(W::add(W::sq(dot(re)), W::sq(dot(im))), q2));
+                ei = W::fixed(si);
             }
         }
         // sums over runs of lanes with one shell; the first lane of a run adds them
@@ -459,7 +496,7 @@ __global__ void __launch_bounds__(256) k_bin(const SpecArgs s, const typename CT
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nsum; i += 256)
+    for (int i = threadIdx.x; i < nsum; i += BIN_THREADS)
         if (shq[i]) atomicAdd(&hist[i], shq[i]);
 }
 // shells out of the histogram (second slot only when split)
@@ -482,7 +519,7 @@ static int grid_for(int64_t N)
 int velocity_blocks(const SpecArgs &s)
 {
     const int64_t b = (s.N + 255) / 256;
-    return (int)(b < 1 ? 1 : b > 152 * 8 ? 152 * 8 : b);
+    return (int)(b < 1 ? 1 : b > 152 * 4 ? 152 * 4 : b);
 }
 
 cudaError_t launch_deriv(const SpecArgs &s, const void *src, void *dst, int axis, cudaStream_t st)
@@ -551,28 +588,30 @@ cudaError_t launch_trap_level(int prec, void *const *tab, int ndim, const int64_
 }
 
 // histogram and shells of the fields uh; work: 2 nshells + 1 doubles (histogram
-// and scale), partial: npartial sums of squares from launch_velocity
+// and scale); total times the sum of the npartial numbers at partial is the sum of
+// squares of the fields
 cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, const double *partial, int npartial,
-                       double *work, double half_dv_over_n, double *out, cudaStream_t st)
+                       double total, double *work, double half_dv_over_n, double *out, cudaStream_t st)
 {
     unsigned long long *hist = reinterpret_cast<unsigned long long *>(work);
     double *scale = work + 2 * nshells;
     const size_t smem = sizeof(unsigned long long) * (s.split ? 2 : 1) * (size_t)nshells;
-    // blocks of at least two iterations, as many as fit beside one another
-    const int64_t want = (s.N + 511) / 512, fit = smem > 64 * 1024 ? 2 : smem > 32 * 1024 ? 3 : 6;
-    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(want, 152 * fit));
+    // two blocks per SM: each sums the partials (FP64) before it starts
+    int64_t units = (((int64_t)1 << s.lg[0]) / 2 + 32) / 32;
+    for (int a = 1; a < 3; ++a) units *= ((int64_t)1 << s.lg[a]) / 2 + 1;
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((units + BIN_THREADS / 32 - 1) / (BIN_THREADS / 32), 152 * 2));
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * 2 * (size_t)nshells, st);
     if (e != cudaSuccess) return e;
     if (s.prec == 0) {
         e = cudaFuncSetAttribute(k_bin<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_bin<float><<<nb, 256, smem, st>>>(s, (const float2 *)uh[0], (const float2 *)uh[1], (const float2 *)uh[2],
-                                            (int)nshells, partial, npartial, hist, scale);
+        k_bin<float><<<nb, BIN_THREADS, smem, st>>>(s, (const float2 *)uh[0], (const float2 *)uh[1], (const float2 *)uh[2],
+                                            (int)nshells, partial, npartial, total, hist, scale);
     } else {
         e = cudaFuncSetAttribute(k_bin<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_bin<double><<<nb, 256, smem, st>>>(s, (const double2 *)uh[0], (const double2 *)uh[1], (const double2 *)uh[2],
-                                             (int)nshells, partial, npartial, hist, scale);
+        k_bin<double><<<nb, BIN_THREADS, smem, st>>>(s, (const double2 *)uh[0], (const double2 *)uh[1], (const double2 *)uh[2],
+                                             (int)nshells, partial, npartial, total, hist, scale);
     }
     k_hist_out<<<(unsigned)((2 * nshells + 127) / 128), 128, 0, st>>>(hist, (int)nshells, s.split, scale,
                                                                      half_dv_over_n, out);

@@ -15,6 +15,8 @@ enum PointOp : int {
     OP_KIMAG = 4,        // psi *= prod_a exp(-k_a^2 dt/2)/n_a            (imaginary-time kinetic substep)
     OP_SCALE_NIMAG = 5,  // psi *= s[instance], then OP_NIMAG            (deferred renormalisation)
     OP_SCALE = 6,        // psi *= s[instance]
+    OP_DERIV = 7,        // psi *= i k_a, one axis a (complex64 spectra)
+    OP_VEL = 8,          // d -> Im(conj(psi) d / N) / |psi| (vel_part 0) or Re(...) / |psi| (1), see k_velocity
 };
 
 // reductions a pass can produce, one value per line per quantity
@@ -64,6 +66,11 @@ struct PassArgs {
     // (int64), ki_ax exp(-k^2 dt/2) 2^-kiq_e to 62 bits (int64; ki_o0 and ki_o1
     // stay double), gq the nonlinear coupling ([batch][half, full]; complex64:
     // g nl_c as floats)
+    // OP_DERIV: wavenumbers of the derivative's axis (floats, Nyquist mode zero)
+    // in the pointer of that axis; OP_VEL: psi and which part
+    const float *dk_ax, *dk_o0, *dk_o1;
+    const void *vel_psi;
+    int vel_part;
     const void *gq;
     int vq_full, kiq_e, lg_n;      // lg_n: log2 of the points of an instance
     const double *g;       // per-instance interaction
@@ -257,6 +264,6 @@ cudaError_t launch_deriv(const SpecArgs &s, const void *src, void *dst, int axis
 int velocity_blocks(const SpecArgs &s);     // partial sums that launch_velocity writes
 cudaError_t launch_velocity(const SpecArgs &s, const void *psi, void *w, double *partial, cudaStream_t st);
 cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, const double *partial, int npartial,
-                       double *work, double half_dv_over_n, double *out, cudaStream_t st);
+                       double total, double *work, double half_dv_over_n, double *out, cudaStream_t st);
 
 }  // namespace gpe

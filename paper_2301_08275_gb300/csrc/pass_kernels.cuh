@@ -210,6 +210,16 @@ __device__ __forceinline__ double2 offset_product(double2 a, double2 b)
     return make_double2(a.x + b.x + (a.x * b.x - a.y * b.y), a.y + b.y + (a.x * b.y + a.y * b.x));
 }
 
+// Component of the velocity (part 0: Im) or of the gradient of |psi| (part 1: Re)
+// from psi and a derivative d not yet divided by N; zero where |psi|^2 < 1e-30.
+template <typename R, typename C> __device__ __forceinline__ R velocity_of(C p, C d, int part, R invn)
+{
+    const R rho = p.x * p.x + p.y * p.y;
+    R u = (R)0;
+    if (rho >= (R)1e-30) u = (part ? (p.x * d.x + p.y * d.y) : (p.x * d.y - p.y * d.x)) * invn / sqrt(rho);
+    return u;
+}
+
 // pointwise substep on the E points (indices tl + TPL*e on this axis) of one line
 // inst: position of the instance in this launch (renormalisation factor);
 // ti: its parameter/table slot
@@ -251,6 +261,24 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = cscale(v[e], fl * ki[tl + TPL * e]);
         return;
+    }
+    if constexpr (sizeof(R) == 4) {
+        if (op == OP_DERIV) {
+            const float kl = a.dk_o0 ? a.dk_o0[c0] : a.dk_o1 ? a.dk_o1[c1] : 0.0f;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const float k = a.dk_ax ? a.dk_ax[tl + TPL * e] : kl;
+                v[e] = mk(-k * v[e].y, k * v[e].x);
+            }
+            return;
+        }
+        if (op == OP_VEL) {                // rows
+            const C *psi = static_cast<const C *>(a.vel_psi) + off;
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                v[e] = mk(velocity_of<R>(psi[tl + TPL * e], v[e], a.vel_part, a.inv_n), 0.0f);
+            return;
+        }
     }
     if (op == OP_SCALE || op == OP_SCALE_NIMAG) {
         const R s = (R)a.scale[inst];
@@ -758,9 +786,11 @@ __host__ __device__ constexpr SweepProg sweep_prog(int p)
            : p == 7 ? SweepProg{OP_NONE, 1, OP_NIMAG, 0, OP_NONE, RED_NORM}     // I, decay, norm
            : p == 8 ? SweepProg{OP_NREAL, -1, OP_NONE, 0, OP_NONE, RED_NONE}    // first half-step, F
            : p == 9 ? SweepProg{OP_NONE, 1, OP_NREAL, 0, OP_NONE, RED_NONE}     // I, last half-step
+           : p == 10 ? SweepProg{OP_DERIV, 1, OP_NONE, 0, OP_NONE, RED_NONE}    // derivative, I (spectra)
+           : p == 11 ? SweepProg{OP_VEL, -1, OP_NONE, 0, OP_NONE, RED_NORM}     // velocity, F, its squares
                     : SweepProg{-1, -1, -1, -1, -1, -1};
 }
-constexpr int NUM_SWEEP_PROGS = 9;
+constexpr int NUM_SWEEP_PROGS = 11;
 inline int sweep_prog_of(const PassArgs &a)
 {
     if (a.generic) return 0;
@@ -781,6 +811,12 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
     const int op_pre = PROG ? PP.op_pre : a.op_pre, op_mid = PROG ? PP.op_mid : a.op_mid;
     const int op_post = PROG ? PP.op_post : a.op_post, rmode = PROG ? PP.red : a.red;
     const int fft1 = PROG ? PP.fft1 : a.fft1, fft2 = PROG ? PP.fft2 : a.fft2;
+    if (PROG == 0) {
+        // the spectra's substeps come in their own programs only
+        __builtin_assume(op_pre < OP_DERIV);
+        __builtin_assume(op_mid < OP_DERIV);
+        __builtin_assume(op_post < OP_DERIV);
+    }
     constexpr int LPT = lines_per_thread<R>();
     constexpr int L = pick_lines<R, N, ROWS, VAR>();
     using T = PassTile<R, N, ROWS, VAR>;
@@ -1430,6 +1466,11 @@ static cudaError_t launch_pass_t(const PassArgs &a, cudaStream_t st, const CUten
             if (p == 7) return launch_pass_p<R, N, ROWS, VAR, 7>(a, st, tmap);
             if (p == 8) return launch_pass_p<R, N, ROWS, VAR, 8>(a, st, tmap);
             if (p == 9) return launch_pass_p<R, N, ROWS, VAR, 9>(a, st, tmap);
+            if constexpr (sizeof(R) == 4) {
+                if (p == 3) return launch_pass_p<R, N, ROWS, VAR, 3>(a, st, tmap);
+                if (p == 10) return launch_pass_p<R, N, ROWS, VAR, 10>(a, st, tmap);
+                if (p == 11) return launch_pass_p<R, N, ROWS, VAR, 11>(a, st, tmap);
+            }
         } else {
             if (p == 1) return launch_pass_p<R, N, ROWS, VAR, 1>(a, st, tmap);
             if (p == 2) return launch_pass_p<R, N, ROWS, VAR, 2>(a, st, tmap);

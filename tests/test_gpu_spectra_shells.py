@@ -45,3 +45,27 @@ def test_spectra_match_oracle(gpe, orc, n, length, prec, scale):
         got = got[: len(want)]
         total = max(np.linalg.norm(want), 1e-3 * np.linalg.norm(ref[0]) + 1e-3 * np.linalg.norm(ref[1]))
         assert np.linalg.norm(got - want) <= tol * total
+
+
+@pytest.mark.parametrize("n,length", [((64, 128), (9.0, 9.0)), ((256, 64), (10.0, 4.0)), ((64, 128, 64), (5.0, 5.0, 5.0))],
+                         ids=lambda v: "x".join(str(x) for x in v))
+def test_fused_derivative_and_velocity_sweeps(gpe, orc, n, length):
+    """Complex64 grids of at least 64 points per axis form i k psi and the velocity
+    inside the transforms' sweeps; the separate kernels (generic passes) give the
+    same spectra, to the rounding of single values (1e-6 of the total)."""
+    import torch
+    sp = gi.Spec(n=n, lo=(0.0,) * len(n), length=length, g=1.0, dt=1e-3, gamma=(0.0,) * len(n))
+    psi = gi.random_field(sp, seed=5).astype(np.complex64)
+    psi[..., :3] = 0.0                                  # points without density have no velocity
+    kinds = gpe.GPE_SPEC_INC | gpe.GPE_SPEC_COMP | gpe.GPE_SPEC_QP
+    outs = []
+    for generic in (0, 1):
+        p = gpe.Plan(n, sp.lo, length, g=1.0, dt=1e-3, prec=gpe.GPE_C64)
+        p.set_option(gpe.GPE_OPT_GENERIC_PASSES, generic)
+        outs.append(p.spectrum(torch.from_numpy(psi).cuda(), kinds)[:, 0])
+        p.close()
+    P = orc.Problem(**sp.kwargs())
+    ref = list(P.spectrum(psi.astype(np.complex128))) + [P.spectrum_qp_num(psi.astype(np.complex128))[0]]
+    for a, b, r in zip(outs[0], outs[1], ref):
+        assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(b)
+        assert np.linalg.norm(a[: len(r)] - r) <= 1e-5 * np.linalg.norm(r)
