@@ -77,14 +77,25 @@ __device__ __forceinline__ float2 phase_offset(float th)
 // choice is made per element, so a point's result does not depend on which
 // lines share its warp (tile shapes and kernels with other thread layouts
 // give the same bits); a warp whose angles are all small takes one branch.
+// The choice costs one branch per thread: a thread with any larger angle goes
+// through its elements a second time (a branch per element was 4 of the 134
+// instructions per point of a 512-point row sweep).
 template <typename C, typename R, int E>
 __device__ __forceinline__ void apply_phase(C (&v)[E], const R (&th)[E])
 {
+    R most = (R)0;
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        auto w = phase_offset_small(th[e]);
-        if (fabs(th[e]) > (R)0.0625) w = phase_offset(th[e]);
-        v[e] = cmadd1(v[e], w);
+    for (int e = 0; e < E; ++e) most = max(most, fabs(th[e]));
+    if (!(most > (R)0.0625)) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = cmadd1(v[e], phase_offset_small(th[e]));
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            auto w = phase_offset_small(th[e]);
+            if (fabs(th[e]) > (R)0.0625) w = phase_offset(th[e]);
+            v[e] = cmadd1(v[e], w);
+        }
     }
 }
 
@@ -410,7 +421,7 @@ struct LineGeom {
     int inst, ti, c0, c1;
     bool valid;
 };
-template <int L>
+template <int L, int ROWN = 0>      // ROWN: points per line of a row sweep (line starts follow one another)
 __device__ __forceinline__ LineGeom line_geom(const PassArgs &a, int64_t tile, int l)
 {
     LineGeom g;
@@ -421,7 +432,8 @@ __device__ __forceinline__ LineGeom line_geom(const PassArgs &a, int64_t tile, i
     g.li = g.lg & ((int64_t(1) << a.lg_lpi) - 1);
     g.c0 = int(g.li & (a.o0n - 1));
     g.c1 = int(g.li >> a.lg_o0);
-    g.off = (g.li & ((int64_t(1) << a.lg_A) - 1)) + (g.li >> a.lg_A) * a.Sb;
+    if (ROWN) g.off = g.li * ROWN;
+    else g.off = (g.li & ((int64_t(1) << a.lg_A) - 1)) + (g.li >> a.lg_A) * a.Sb;
     return g;
 }
 // base pointers of an instance (inst_ptr indirection or back-to-back storage)
@@ -935,18 +947,15 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
         }
         LineGeom g[LPT];
 #pragma unroll
-        for (int ln = 0; ln < LPT; ++ln) g[ln] = line_geom<L>(a, tile, l0 + ln);
+        for (int ln = 0; ln < LPT; ++ln) g[ln] = line_geom<L, ROWS ? N : 0>(a, tile, l0 + ln);
         C v[LPT][E];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             if (tma) T::ld_plain(sm, tl, e, l0, v);    // the copy engine's tile is unswizzled
             else T::ld(sm, tl, e, l0, v);
         }
-#pragma unroll
-        for (int ln = 0; ln < LPT; ++ln)
-            if (!g[ln].valid)
-#pragma unroll
-                for (int e = 0; e < E; ++e) v[ln][e] = mk((R)0, (R)0);
+        // (lines beyond the last hold what the buffer held: they are computed and
+        // never stored, and no line's result depends on another's)
 
         if (rmode == RED_DIAG_X || rmode == RED_DIAG_XM) {
             // real-space moments of rho = |psi|^2 along each row, then kx^2 |F_x psi|^2
@@ -1145,7 +1154,8 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
 #pragma unroll
             for (int ln = 0; ln < LPT; ++ln) {
                 if (g[ln].valid) {
-                    C *dst = inst_dst<C>(a, g[ln].inst) + g[ln].off;
+                    C *dst = ROWS && !a.inst_ptr ? static_cast<C *>(a.dst) + g[ln].lg * N
+                                                 : inst_dst<C>(a, g[ln].inst) + g[ln].off;
 #pragma unroll
                     for (int e = 0; e < E; ++e) dst[(int64_t)(tl + TPL * e) * es] = v[ln][e];
                 }
