@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
+#include <type_traits>
 
 #include "fx.cuh"
 
@@ -571,9 +572,9 @@ template <typename R, int N, int L, int LPT, bool SW = false, int EPT = 0, bool 
     // in a pass that a later barrier closed.  A transform's input registers
     // must not depend on pending reads of ss or sb by other threads beyond
     // these rules (the tile's own load from sb is closed by the barrier of pass 1).
-    template <int DIR, int p, bool PING = false>
-    __device__ __forceinline__ static void pass(C (&v)[LPT][E], C *sb, C *ss, int tl, int l0,
-                                                const U *__restrict__ tw)
+    // tw: the pass-ordered table, or a RegTwiddles
+    template <int DIR, int p, bool PING = false, typename TW>
+    __device__ __forceinline__ static void pass(C (&v)[LPT][E], C *sb, C *ss, int tl, int l0, const TW &tw)
     {
         constexpr int r = PL::radix(p);
         constexpr int Ns = PL::ns(p);
@@ -599,10 +600,11 @@ template <typename R, int N, int L, int LPT, bool SW = false, int EPT = 0, bool 
 #pragma unroll
                 for (int m = 0; m < r; ++m) x[ln][m] = v[ln][q + m * B];
             if constexpr (Ns > 1) {
-                const U *twk = tw + tw_off(p) + k;
 #pragma unroll
                 for (int m = 1; m < r; ++m) {
-                    const U w = twk[(m - 1) * Ns];
+                    U w;
+                    if constexpr (std::is_pointer<TW>::value) w = (tw + tw_off(p) + k)[(m - 1) * Ns];
+                    else w = tw.template get<p>(q, m, k);
 #pragma unroll
                     for (int ln = 0; ln < LPT; ++ln) x[ln][m] = umul<(DIR > 0), PL::TWSH>(x[ln][m], w);
                 }
@@ -630,8 +632,8 @@ template <typename R, int N, int L, int LPT, bool SW = false, int EPT = 0, bool 
         }
     }
 
-    template <int DIR, bool PING = false, int p = 0>
-    __device__ __forceinline__ static void fft(C (&v)[LPT][E], C *sb, C *ss, int tl, int l0, const U *tw)
+    template <int DIR, bool PING = false, int p = 0, typename TW>
+    __device__ __forceinline__ static void fft(C (&v)[LPT][E], C *sb, C *ss, int tl, int l0, const TW &tw)
     {
         if constexpr (p < PL::P) {
             pass<DIR, p, PING>(v, sb, ss, tl, l0, tw);
@@ -653,14 +655,42 @@ template <typename R, int N, int L, int LPT, bool SW = false, int EPT = 0, bool 
     }
 };
 
+// A thread's own twiddles of the passes from FIRST on, read from the table once
+// and kept in registers: they depend on its position only, not on the tile.
+// Reading them in every transform is 4 of 9 shared-memory wavefronts per point
+// and pass of rows (each lane its own 16 bytes), where the exchange takes 4 in
+// all.  For tiles of one butterfly per thread and pass.
+template <typename T, int FIRST> struct RegTwiddles {
+    using U = typename T::U;
+    static_assert(T::E == T::PL::radix(T::PL::P - 1) && T::E == T::PL::radix(FIRST), "one butterfly per pass");
+    static constexpr int R = T::E;
+    U w[T::PL::P - FIRST][R - 1];
+    const U *tws;
+    template <int p = FIRST> __device__ __forceinline__ void load(const U *tw, int tl)
+    {
+        tws = tw;
+        if constexpr (p < T::PL::P) {
+#pragma unroll
+            for (int m = 1; m < R; ++m)
+                w[p - FIRST][m - 1] = tw[T::tw_off(p) + (tl & (T::PL::ns(p) - 1)) + (m - 1) * T::PL::ns(p)];
+            load<p + 1>(tw, tl);
+        }
+    }
+    template <int p> __device__ __forceinline__ U get(int, int m, int k) const
+    {
+        if constexpr (p >= FIRST) return w[p - FIRST][m - 1];
+        else return (tws + T::tw_off(p) + k)[(m - 1) * T::PL::ns(p)];
+    }
+};
+
 // Two transforms with a pointwise step between them, f1, f2 in {-1 forward,
 // +1 inverse, 0 none}: one copy of the forward transform in a loop, the
 // inverse as conj(F(conj(v))).  Every kernel of the library that runs the
 // 2D/3D sweeps goes through here, so all of them round alike.
-template <typename T, bool PING, typename Mid>
+template <typename T, bool PING, typename TW, typename Mid>
 __device__ __forceinline__ void sweep_transforms(typename T::C (&v)[T::LPT_][T::E], typename T::C *sb,
-                                                 typename T::C *ss, int tl, int l0, const typename T::U *tw, int f1,
-                                                 int f2, Mid &&mid)
+                                                 typename T::C *ss, int tl, int l0, const TW &tw, int f1, int f2,
+                                                 Mid &&mid)
 {
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {

@@ -605,10 +605,23 @@ template <typename R, int N, bool ROWS, int VAR> __host__ __device__ constexpr s
 // CTAs per SM the registers are budgeted for: 4 per SM for split rows (1024 /
 // threads per CTA, at most 16), else 2 (1 for CTAs of more than 512 threads),
 // never more than fit in the SM's shared memory
-template <typename R, int N, bool ROWS, int VAR> __host__ __device__ constexpr int pass_min_blocks()
+// Program 12: the steady row sweep of 512-point complex64 rows without a trap,
+// twiddles in registers.  That sweep was bound by the shared-memory pipe (81 % of
+// its wavefront rate, 14 of 36 wavefronts per 32 points for twiddles); 124
+// registers instead of 68.  Measured, us per sweep, table / registers: 512^3
+// 665 / 627, 512 x 256^2 175 / 166, 32 instances of 512^2 49.3 / 47.3.  With trap
+// factors the occupancy is worth more (128 instances of 512^2 221 / 260, 512 x
+// 64^2 20.5 / 22.5; 512^3 836 / 800), and so it is for 256-point rows (109 / 113
+// at 256^3).
+template <typename R, int N, bool ROWS, int PROG> __host__ __device__ constexpr bool pass_reg_twiddles()
+{
+    return ROWS && sizeof(R) == 4 && N == 512 && PROG == 12;
+}
+template <typename R, int N, bool ROWS, int VAR, int PROG = 0> __host__ __device__ constexpr int pass_min_blocks()
 {
     constexpr int nt = PassTile<R, N, ROWS, VAR>::NT;
-    constexpr int want = 1024 / nt > 16 ? 16 : 1024 / nt;
+    constexpr int threads = pass_reg_twiddles<R, N, ROWS, PROG>() ? 512 : 1024;
+    constexpr int want = threads / nt > 16 ? 16 : threads / nt;
     // (strided tiles of 32 points per thread keep 2: capping their registers
     // for a third CTA, 170, made the 512^3 y sweep slower, 0.347 -> 0.475 ms)
     constexpr int b = rows_split<R, N, ROWS, VAR>() && want > 2 ? want : (nt > 512 ? 1 : 2);
@@ -799,6 +812,7 @@ __host__ __device__ constexpr SweepProg sweep_prog(int p)
            : p == 8 ? SweepProg{OP_NREAL, -1, OP_NONE, 0, OP_NONE, RED_NONE}    // first half-step, F
            : p == 9 ? SweepProg{OP_NONE, 1, OP_NREAL, 0, OP_NONE, RED_NONE}     // I, last half-step
            : p == 10 ? SweepProg{OP_DERIV, 1, OP_NONE, 0, OP_NONE, RED_NONE}    // derivative, I (spectra)
+           : p == 12 ? SweepProg{OP_NONE, 1, OP_NREAL, -1, OP_NONE, RED_NONE}   // program 4 (see pass_reg_twiddles)
            : p == 11 ? SweepProg{OP_VEL, -1, OP_NONE, 0, OP_NONE, RED_NORM}     // velocity, F, its squares
                     : SweepProg{-1, -1, -1, -1, -1, -1};
 }
@@ -816,7 +830,7 @@ inline int sweep_prog_of(const PassArgs &a)
 }
 
 template <typename R, int N, bool ROWS, int VAR, int PROG>
-__global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_blocks<R, N, ROWS, VAR>()))
+__global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_blocks<R, N, ROWS, VAR, PROG>()))
     k_pass(const PassArgs a, const __grid_constant__ CUtensorMap tmap)
 {
     constexpr SweepProg PP = sweep_prog(PROG);
@@ -923,6 +937,14 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
         cp_async_commit();
     };
 
+    constexpr bool RTW = pass_reg_twiddles<R, N, ROWS, PROG>();
+    typename std::conditional<RTW, RegTwiddles<T, (RTW ? 1 : 0)>, const U *>::type twr;
+    if constexpr (RTW) {
+        __syncthreads();
+        twr.load(tw, tl);
+    } else {
+        twr = tw;
+    }
     int64_t tile = blockIdx.x;
     stage(tile, buf0, 0);
     stage(tile + gridDim.x, buf1, 1);
@@ -1114,7 +1136,7 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
 #pragma unroll
                 for (int ln = 0; ln < LPT; ++ln)
                     point_op<R, E, TPL>(op_pre, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
-                sweep_transforms<T, PING>(v, sm, PING ? scr : sm, tl, l0, tw, fft1, fft2, [&]() {
+                sweep_transforms<T, PING>(v, sm, PING ? scr : sm, tl, l0, twr, fft1, fft2, [&]() {
 #pragma unroll
                     for (int ln = 0; ln < LPT; ++ln)
                         point_op<R, E, TPL>(op_mid, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
@@ -1198,6 +1220,9 @@ template <typename R, int N, int L> struct Line1DCfg {
     static constexpr size_t base = buf + line1d_red_bytes(NT) + sizeof(typename T::U) * N;
     static constexpr bool PING = T::PL::P > 1 && base + buf <= 200 * 1024;
     static constexpr size_t smem = base + (PING ? buf : 0);
+    // one long line per CTA: registers to spare for the twiddles of the last passes
+    static constexpr bool RTW = sizeof(R) == 4 && L == 1 && N >= 512 && N <= 4096;
+    static constexpr int FIRST = T::PL::P - 2 > 1 ? T::PL::P - 2 : 1;
 };
 template <typename R, int N, int L>
 __global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DArgs a)
@@ -1221,6 +1246,9 @@ __global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DA
     U *tw = reinterpret_cast<U *>(reinterpret_cast<unsigned char *>(red) + line1d_red_bytes(NT));
     T::load_twiddles(tw, static_cast<const U *>(a.tw), t, NT);
     __syncthreads();
+    typename std::conditional<Cfg::RTW, RegTwiddles<T, (Cfg::RTW ? Cfg::FIRST : 0)>, const U *>::type twr;
+    if constexpr (Cfg::RTW) twr.load(tw, tl);
+    else twr = tw;
     const int64_t ntiles = (a.batch + L - 1) / L;
 
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -1253,10 +1281,10 @@ __global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DA
                 if (vh) v[e] = uomul(v[e], vh[ib * N + tl + TPL * e]);
 #pragma unroll 1
             for (int64_t st = 0; st < a.nsteps; ++st) {
-                T::template fft<-1, PING>(w, sm, ss, tl, 0, tw);
+                T::template fft<-1, PING>(w, sm, ss, tl, 0, twr);
 #pragma unroll
                 for (int e = 0; e < E; ++e) v[e] = cscale(uomul(v[e], kt[tl + TPL * e]), invn);
-                T::template fft<1, PING>(w, sm, ss, tl, 0, tw);
+                T::template fft<1, PING>(w, sm, ss, tl, 0, twr);
                 const bool last = (st == a.nsteps - 1);
                 const R gc = last ? gh : gf;
                 const U *vt = last ? (a.vh_last ? static_cast<const U *>(a.vh_last) : vh) : vf;
@@ -1282,10 +1310,10 @@ __global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DA
                     if (vi) f *= vi[ib * N + tl + TPL * e];
                     v[e] = cscale(x, f);
                 }
-                T::template fft<-1, PING>(w, sm, ss, tl, 0, tw);
+                T::template fft<-1, PING>(w, sm, ss, tl, 0, twr);
 #pragma unroll
                 for (int e = 0; e < E; ++e) v[e] = cscale(v[e], ki[tl + TPL * e]);
-                T::template fft<1, PING>(w, sm, ss, tl, 0, tw);
+                T::template fft<1, PING>(w, sm, ss, tl, 0, twr);
                 double nrm = 0.0;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
@@ -1471,6 +1499,9 @@ static cudaError_t launch_pass_t(const PassArgs &a, cudaStream_t st, const CUten
     if constexpr (sweep_progs_compiled<R, N, ROWS>()) {
         const int p = sweep_prog_of(a);
         if constexpr (ROWS) {
+            if constexpr (sizeof(R) == 4 && N == 512) {
+                if (p == 4 && !a.vt_ax && !a.vt_o0 && !a.vt_o1) return launch_pass_p<R, N, ROWS, VAR, 12>(a, st, tmap);
+            }
             if (p == 4) return launch_pass_p<R, N, ROWS, VAR, 4>(a, st, tmap);
             if (p == 5) return launch_pass_p<R, N, ROWS, VAR, 5>(a, st, tmap);
             if (p == 7) return launch_pass_p<R, N, ROWS, VAR, 7>(a, st, tmap);
