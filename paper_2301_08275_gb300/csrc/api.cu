@@ -100,6 +100,7 @@ struct gpe_plan {
     double *g_dev = nullptr, *gamma_dev = nullptr, *scale = nullptr, *partials = nullptr;
     double *sums = nullptr, *out6 = nullptr, *out4 = nullptr;
     double *csum = nullptr;                  // chunk sums of the line reductions
+    unsigned *red_count = nullptr;           // CTAs of a line reduction that are done
     // imaginary-time convergence on the device: [0] stop word (int), [8] steps done (int64_t)
     unsigned char *istate = nullptr;
     double *eprev = nullptr;                 // [batch] energies of the last check
@@ -557,7 +558,8 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
     {
         int64_t nch = 1;
         for (int a = 0; a < d->ndim; ++a) nch = std::max(nch, reduce_chunks(p->N / p->n[a]));
-        PLAN_TRY(dalloc(p, (void **)&p->csum, sizeof(double) * NQ * B * nch));
+        PLAN_TRY(dalloc(p, (void **)&p->csum, sizeof(double) * (NQ * B * nch + 1)));
+        p->red_count = reinterpret_cast<unsigned *>(p->csum + NQ * B * nch);
     }
     PLAN_TRY(dalloc(p, (void **)&p->istate, 16));
     PLAN_TRY(dalloc(p, (void **)&p->eprev, sizeof(double) * B));
@@ -587,7 +589,8 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
     }
     if (cudaMemcpy(p->g_dev, gs.data(), sizeof(double) * B, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(p->gamma_dev, gam.data(), sizeof(double) * 3 * B, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess) {
+        cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(p->red_count, 0, sizeof(unsigned)) != cudaSuccess) {
         destroy(p);
         return fail(GPE_ECUDA, "uploading plan parameters failed");
     }
@@ -1353,10 +1356,10 @@ static gpe_status diag_dev(gpe_plan *p, const void *psi, bool kinetic = true)
         GPE_TRY(run(p, k));
     }
     const int *stop = p->cur_stop;
-    cudaError_t e = launch_reduce_lines(p->partials, p->lines_cap, 0, 7, B, p->N / p->n[0], p->csum, p->sums, p->st,
+    cudaError_t e = launch_reduce_lines(p->partials, p->lines_cap, 0, 7, B, p->N / p->n[0], p->csum, p->sums, p->red_count, p->st,
                                         0.0, 0.0, nullptr, nullptr, stop);
     for (int a = 1; a < p->ndim && e == cudaSuccess && kinetic; ++a)
-        e = launch_reduce_lines(p->partials, p->lines_cap, 6 + a, 1, B, p->N / p->n[a], p->csum, p->sums, p->st,
+        e = launch_reduce_lines(p->partials, p->lines_cap, 6 + a, 1, B, p->N / p->n[a], p->csum, p->sums, p->red_count, p->st,
                                 0.0, 0.0, nullptr, nullptr, stop);
     if (e == cudaSuccess)
         e = launch_finish_diag(p->sums, B, p->ndim, p->n, p->dv, p->g_dev, p->out6, p->out4, p->st, stop);
@@ -1726,7 +1729,7 @@ static gpe_status imag_steps(gpe_plan *p, void *psi, int64_t nsteps, double targ
         x2.red = RED_NORM;
         GPE_TRY(run(p, x2));
         cudaError_t e = launch_reduce_lines(p->partials, p->lines_cap, 0, 1, B, p->N / p->n[0], p->csum, p->sums,
-                                            p->st, p->dv, target, p->scale, p->err, p->cur_stop);
+                                            p->red_count, p->st, p->dv, target, p->scale, p->err, p->cur_stop);
         if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("renormalisation: ") + cudaGetErrorString(e));
     }
     // apply the last renormalisation
@@ -1957,7 +1960,8 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
         }
         // every block of the binning kernel adds the sums up: not more than a few thousand
         if (fused && lines > REDUCE_CHUNK) {
-            cudaError_t e = launch_reduce_lines(p->partials, sqcap, 0, p->ndim, 1, lines, p->csum, p->sums, p->st);
+            cudaError_t e = launch_reduce_lines(p->partials, sqcap, 0, p->ndim, 1, lines, p->csum, p->sums, p->red_count,
+                                                p->st);
             if (e != cudaSuccess) return fail(GPE_ECUDA, cudaGetErrorString(e));
         }
         return GPE_OK;

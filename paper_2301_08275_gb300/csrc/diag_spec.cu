@@ -18,11 +18,37 @@ namespace gpe {
 // per lane, shuffles).  FP64 additions are slow on this GPU (one warp
 // instruction per 64 cycles per SM sub-partition): spreading them over many
 // SMs is what makes the sum fast (65536 lines: 24 us in one CTA before).
-__global__ void __launch_bounds__(256) k_reduce_chunks(const double *__restrict__ partials, int64_t cap, int q0,
-                                                       int64_t lpi, int64_t nch, double *__restrict__ csum,
-                                                       const int *stop)
+// One launch: the last CTA to finish its chunk adds the chunk sums (an instance
+// of one chunk has none to add).  With scale set, the sum of quantity 0 (the norm)
+// also gives the imaginary-time renormalisation factor s_b = sqrt(target / (sum
+// rho dV)).  Launched dependent on the sweep before it and with the next sweep
+// dependent on it, as the sweeps are on one another: as two ordinary launches
+// it was 22 of the 346 us of a 256^3 complex64 imaginary step (ncu: 10 us of
+// work) and half of the difference between real and imaginary steps of small grids.
+__device__ __forceinline__ void reduce_finish(double s, int64_t b, int q, double *sums, double dv, double target,
+                                              double *scale, int *err)
+{
+    sums[b * NQ + q] = s;
+    if (scale && q == 0) {
+        const double nrm = s * dv;
+        if (!(nrm > 0.0) || !isfinite(nrm)) {
+            atomicOr(err, (int)ERR_NUMERIC);
+            scale[b] = 1.0;
+        } else {
+            scale[b] = sqrt(target / nrm);
+        }
+    }
+}
+__global__ void __launch_bounds__(256) k_reduce_lines(const double *__restrict__ partials, int64_t cap, int q0, int nq,
+                                                      int64_t lpi, int64_t nch, int64_t batch, double *csum,
+                                                      double *__restrict__ sums, double dv, double target,
+                                                      double *__restrict__ scale, int *err, unsigned *counter,
+                                                      const int *stop)
 {
     __shared__ double sh[8];
+    __shared__ bool last;
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" :::);
     if (stop && *reinterpret_cast<const volatile int *>(stop)) return;
     const int64_t c = blockIdx.x, b = blockIdx.z;
     const int q = q0 + blockIdx.y, t = threadIdx.x;
@@ -43,40 +69,31 @@ __global__ void __launch_bounds__(256) k_reduce_chunks(const double *__restrict_
     __syncthreads();
     if (t == 0) {
         const double r = ((sh[0] + sh[1]) + (sh[2] + sh[3])) + ((sh[4] + sh[5]) + (sh[6] + sh[7]));
-        csum[(b * NQ + q) * nch + c] = r;
-    }
-}
-
-// One warp per (instance, quantity): sums of the chunk sums.  With scale set,
-// the sum of quantity 0 (the norm) also gives the imaginary-time
-// renormalisation factor s_b = sqrt(target / (sum rho dV)).
-__global__ void __launch_bounds__(128) k_reduce_final(const double *__restrict__ csum, int q0, int nq, int64_t batch,
-                                                      int64_t nch, double *__restrict__ sums, double dv, double target,
-                                                      double *__restrict__ scale, int *err, const int *stop)
-{
-    if (stop && *reinterpret_cast<const volatile int *>(stop)) return;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= batch * nq) return;      // uniform per warp
-    const int64_t b = w / nq;
-    const int q = q0 + (int)(w % nq);
-    const double *p = csum + (b * NQ + q) * nch;
-    double s = 0.0;
-    for (int64_t j = lane; j < nch; j += 32) s += p[j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-        sums[b * NQ + q] = s;
-        if (scale && q == 0) {
-            const double nrm = s * dv;
-            if (!(nrm > 0.0) || !isfinite(nrm)) {
-                atomicOr(err, (int)ERR_NUMERIC);
-                scale[b] = 1.0;
-            } else {
-                scale[b] = sqrt(target / nrm);
-            }
+        last = false;
+        if (nch == 1) {
+            reduce_finish(r, b, q, sums, dv, target, scale, err);
+        } else {
+            csum[(b * NQ + q) * nch + c] = r;
+            __threadfence();
+            last = atomicAdd(counter, 1u) == gridDim.x * gridDim.y * gridDim.z - 1;
         }
     }
+    __syncthreads();
+    if (!last) return;
+    // every chunk sum is written: one warp per (instance, quantity)
+    __threadfence();
+    const int lane = t & 31;
+    for (int64_t w = t >> 5; w < batch * nq; w += 8) {
+        const int64_t wb = w / nq;
+        const int wq = q0 + (int)(w % nq);
+        const double *pc = csum + (wb * NQ + wq) * nch;
+        double x = 0.0;
+        for (int64_t k = lane; k < nch; k += 32) x += __ldcg(pc + k);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) reduce_finish(x, wb, wq, sums, dv, target, scale, err);
+    }
+    if (t == 0) *counter = 0;        // for the next launch on this stream
 }
 
 // norm, E_kin, E_pot, E_int, E, mu and sigma_x, sigma_y, sigma_z, r_rms from the
@@ -114,17 +131,22 @@ __global__ void k_finish_diag(const double *__restrict__ sums, int64_t batch, in
 int64_t reduce_chunks(int64_t lines_per_inst) { return (lines_per_inst + REDUCE_CHUNK - 1) / REDUCE_CHUNK; }
 
 cudaError_t launch_reduce_lines(const double *partials, int64_t lines_cap, int nq_first, int nq, int64_t batch,
-                                int64_t lines_per_inst, double *csum, double *sums, cudaStream_t st, double dv,
-                                double target, double *scale, int *err, const int *stop)
+                                int64_t lines_per_inst, double *csum, double *sums, unsigned *counter, cudaStream_t st,
+                                double dv, double target, double *scale, int *err, const int *stop)
 {
     if (batch <= 0 || nq <= 0) return cudaSuccess;
     const int64_t nch = reduce_chunks(lines_per_inst);
-    dim3 grid((unsigned)nch, (unsigned)nq, (unsigned)batch);
-    k_reduce_chunks<<<grid, 256, 0, st>>>(partials, lines_cap, nq_first, lines_per_inst, nch, csum, stop);
-    const int64_t warps = batch * nq;
-    k_reduce_final<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(csum, nq_first, nq, batch, nch, sums, dv, target,
-                                                              scale, err, stop);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nch, (unsigned)nq, (unsigned)batch);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_reduce_lines, partials, lines_cap, nq_first, nq, lines_per_inst, nch, batch, csum,
+                              sums, dv, target, scale, err, counter, stop);
 }
 
 __global__ void k_imag_init(const double *__restrict__ out6, double *__restrict__ eprev, int64_t batch, int *stop,

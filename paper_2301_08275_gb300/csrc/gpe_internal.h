@@ -223,13 +223,14 @@ cudaError_t launch_trap_level(int prec, void *const *tab, int ndim, const int64_
 // sums[b*NQ + q], q in [nq_first, nq_first + nq): per-instance sums of the
 // per-line partials, in a fixed order (chunks of REDUCE_CHUNK lines, then the
 // chunk sums); csum is scratch of batch * NQ * reduce_chunks(lines_per_inst)
-// doubles.  With scale set, the q = 0 sum also gives the renormalisation
+// doubles, counter a word that is zero before the first call on a stream.  With
+// scale set, the q = 0 sum also gives the renormalisation
 // factor scale[b] = sqrt(target / (sum * dv)) (err |= ERR_NUMERIC and
 // scale[b] = 1 for a zero or non-finite norm).
 constexpr int64_t REDUCE_CHUNK = 4096;
 int64_t reduce_chunks(int64_t lines_per_inst);
 cudaError_t launch_reduce_lines(const double *partials, int64_t lines_cap, int nq_first, int nq, int64_t batch,
-                                int64_t lines_per_inst, double *csum, double *sums, cudaStream_t st,
+                                int64_t lines_per_inst, double *csum, double *sums, unsigned *counter, cudaStream_t st,
                                 double dv = 0.0, double target = 0.0, double *scale = nullptr, int *err = nullptr,
                                 const int *stop = nullptr);
 cudaError_t launch_finish_diag(const double *sums, int64_t batch, int ndim, const int64_t *n, double dv,

@@ -214,9 +214,10 @@ extern "C" gpe_status gpe_norm_energy_noalloc(const gpe_plan_desc *d, const void
     double *out6 = reinterpret_cast<double *>(base + kOutOff);
     double *out4 = out6 + 6;
     double *csum = reinterpret_cast<double *>(base + kCsumOff);
-    NA_CUDA(launch_reduce_lines(partials, kMaxLines, 0, 7, 1, N / n[0], csum, sums, st));
+    unsigned *counter = reinterpret_cast<unsigned *>(base + kSumsOff + 192);     // cleared above
+    NA_CUDA(launch_reduce_lines(partials, kMaxLines, 0, 7, 1, N / n[0], csum, sums, counter, st));
     for (int a = 1; a < d->ndim; ++a)
-        NA_CUDA(launch_reduce_lines(partials, kMaxLines, 6 + a, 1, 1, N / n[a], csum, sums, st));
+        NA_CUDA(launch_reduce_lines(partials, kMaxLines, 6 + a, 1, 1, N / n[a], csum, sums, counter, st));
     NA_CUDA(launch_finish_diag(sums, 1, d->ndim, n, dv, reinterpret_cast<const double *>(base + kParamOff), out6, out4,
                                st));
     NA_CUDA(cudaMemcpyAsync(out_host, out6, 6 * sizeof(double), cudaMemcpyDeviceToHost, st));
