@@ -235,9 +235,12 @@ template <typename R, typename C> __device__ __forceinline__ R velocity_of(C p, 
 // inst: position of the instance in this launch (renormalisation factor);
 // ti: its parameter/table slot
 // off: offset of the line's first point within its instance (sampled potential)
+// vreg: the thread's trap factors of the sweep's own axis, held in registers
+// (NULL: read from the table)
 template <typename R, int E, int TPL>
 __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], const PassArgs &a, int inst,
-                                         int ti, int c0, int c1, int tl, int64_t off)
+                                         int ti, int c0, int c1, int tl, int64_t off,
+                                         const typename UT<R>::U *vreg = nullptr)
 {
     using C = typename CT<R>::C;
     if (op == OP_NONE) return;
@@ -324,7 +327,8 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             C x = v[e];
-            if (vax) x = uomul(x, vax[(int64_t)ti * a.nax + tl + TPL * e]);
+            if (vreg) x = uomul(x, vreg[e]);
+            else if (vax) x = uomul(x, vax[(int64_t)ti * a.nax + tl + TPL * e]);
             if (v0) x = uomul(x, f0);
             if (v1) x = uomul(x, f1);
             v[e] = x;
@@ -617,10 +621,22 @@ template <typename R, int N, bool ROWS, int PROG> __host__ __device__ constexpr 
 {
     return ROWS && sizeof(R) == 4 && N == 512 && PROG == 12;
 }
+// Program 13: the same sweep with a trap, rows of 256 or 512 points; each thread
+// holds its trap factors along x (they change with the instance only) and a CTA
+// takes consecutive rows, so that they are read once per instance.  From the
+// table they are 16 bytes per point, as much as the state's reads and writes, and another 4
+// shared-memory/L1 wavefronts per 32 points.  Measured, us per sweep, table /
+// registers: 512^3 838 / 748, 128 instances of 512^2 219 / 192, 256^3 109 / 103,
+// 512 x 64^2 20.7 / 20.5.  Rows of 1024 points spill (17.2 / 18.1 at 1024^2),
+// rows of 128 gain nothing (34.0 / 35.0 at two 128^3).
+template <typename R, int N, bool ROWS, int PROG> __host__ __device__ constexpr bool pass_reg_trap()
+{
+    return ROWS && sizeof(R) == 4 && PROG == 13;
+}
 template <typename R, int N, bool ROWS, int VAR, int PROG = 0> __host__ __device__ constexpr int pass_min_blocks()
 {
     constexpr int nt = PassTile<R, N, ROWS, VAR>::NT;
-    constexpr int threads = pass_reg_twiddles<R, N, ROWS, PROG>() ? 512 : 1024;
+    constexpr int threads = pass_reg_twiddles<R, N, ROWS, PROG>() ? 512 : pass_reg_trap<R, N, ROWS, PROG>() ? 640 : 1024;
     constexpr int want = threads / nt > 16 ? 16 : threads / nt;
     // (strided tiles of 32 points per thread keep 2: capping their registers
     // for a third CTA, 170, made the 512^3 y sweep slower, 0.347 -> 0.475 ms)
@@ -812,6 +828,7 @@ __host__ __device__ constexpr SweepProg sweep_prog(int p)
            : p == 8 ? SweepProg{OP_NREAL, -1, OP_NONE, 0, OP_NONE, RED_NONE}    // first half-step, F
            : p == 9 ? SweepProg{OP_NONE, 1, OP_NREAL, 0, OP_NONE, RED_NONE}     // I, last half-step
            : p == 10 ? SweepProg{OP_DERIV, 1, OP_NONE, 0, OP_NONE, RED_NONE}    // derivative, I (spectra)
+           : p == 13 ? SweepProg{OP_NONE, 1, OP_NREAL, -1, OP_NONE, RED_NONE}   // program 4 (see pass_reg_trap)
            : p == 12 ? SweepProg{OP_NONE, 1, OP_NREAL, -1, OP_NONE, RED_NONE}   // program 4 (see pass_reg_twiddles)
            : p == 11 ? SweepProg{OP_VEL, -1, OP_NONE, 0, OP_NONE, RED_NORM}     // velocity, F, its squares
                     : SweepProg{-1, -1, -1, -1, -1, -1};
@@ -945,12 +962,20 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
     } else {
         twr = tw;
     }
-    int64_t tile = blockIdx.x;
-    stage(tile, buf0, 0);
-    stage(tile + gridDim.x, buf1, 1);
+    // tiles of this CTA: every gridDim.x-th one, or a run of consecutive ones
+    constexpr bool VREG = pass_reg_trap<R, N, ROWS, PROG>();
+    static_assert(!VREG || LPT == 1, "one table slot per thread and tile");
+    const int64_t chunk = VREG ? (a.ntiles + gridDim.x - 1) / gridDim.x : 1;
+    const int64_t step = VREG ? 1 : gridDim.x;
+    int64_t tile = VREG ? blockIdx.x * chunk : blockIdx.x;
+    const int64_t tend = VREG && tile + chunk < a.ntiles ? tile + chunk : a.ntiles;
+    U vreg[VREG ? E : 1];
+    int vti = -1;
+    stage(tile < tend ? tile : a.ntiles, buf0, 0);
+    stage(tile + step < tend ? tile + step : a.ntiles, buf1, 1);
     int it = 0;
     bool aborted = false;
-    for (; tile < a.ntiles; ++it, tile += gridDim.x) {
+    for (; tile < tend; ++it, tile += step) {
         C *sm = (it & 1) ? buf1 : buf0;
         if constexpr (sizeof(R) == 8) {
             if (t < 2 * L) lsc[t] = 0;       // published by the barrier that follows
@@ -1136,10 +1161,19 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
 #pragma unroll
                 for (int ln = 0; ln < LPT; ++ln)
                     point_op<R, E, TPL>(op_pre, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
+                if constexpr (VREG) {
+                    if (g[0].ti != vti) {
+                        vti = g[0].ti;
+                        const U *vax = static_cast<const U *>(a.vt_ax) + (int64_t)vti * N;
+#pragma unroll
+                        for (int e = 0; e < E; ++e) vreg[e] = vax[tl + TPL * e];
+                    }
+                }
                 sweep_transforms<T, PING>(v, sm, PING ? scr : sm, tl, l0, twr, fft1, fft2, [&]() {
 #pragma unroll
                     for (int ln = 0; ln < LPT; ++ln)
-                        point_op<R, E, TPL>(op_mid, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off);
+                        point_op<R, E, TPL>(op_mid, v[ln], a, g[ln].inst, g[ln].ti, g[ln].c0, g[ln].c1, tl, g[ln].off,
+                                            VREG ? vreg : nullptr);
                 });
 #pragma unroll
                 for (int ln = 0; ln < LPT; ++ln)
@@ -1185,7 +1219,7 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
         }
         if (tma) fence_async_shared();   // this thread's accesses to the buffer precede the next copy into it
         __syncthreads();         // every thread is done with this buffer
-        stage(tile + 2 * (int64_t)gridDim.x, sm, it & 1);
+        stage(tile + 2 * step < tend ? tile + 2 * step : a.ntiles, sm, it & 1);
     }
     // this CTA's tiles are written: the next kernel may start its launch (its
     // CTAs still wait for this whole grid before they read the state)
@@ -1501,6 +1535,9 @@ static cudaError_t launch_pass_t(const PassArgs &a, cudaStream_t st, const CUten
         if constexpr (ROWS) {
             if constexpr (sizeof(R) == 4 && N == 512) {
                 if (p == 4 && !a.vt_ax && !a.vt_o0 && !a.vt_o1) return launch_pass_p<R, N, ROWS, VAR, 12>(a, st, tmap);
+            }
+            if constexpr (sizeof(R) == 4 && (N == 256 || N == 512)) {
+                if (p == 4 && a.vt_ax) return launch_pass_p<R, N, ROWS, VAR, 13>(a, st, tmap);
             }
             if (p == 4) return launch_pass_p<R, N, ROWS, VAR, 4>(a, st, tmap);
             if (p == 5) return launch_pass_p<R, N, ROWS, VAR, 5>(a, st, tmap);
