@@ -17,7 +17,6 @@ from __future__ import annotations
 import argparse
 import hashlib
 import json
-import math
 import os
 import subprocess
 import sys
@@ -45,10 +44,7 @@ WORKLOADS = {
 }
 METRIC = "TSSP grid-point updates/s vs HBM roofline"
 UNIT = "grid-point updates/s"
-KERNEL_SOURCES = ["fft_tile.cuh", "pass_kernels.cuh", "pass_f32.cu", "pass_f32_s1.cu", "pass_f32_rows.cu",
-                  "pass_f32_rows1.cu", "pass_f32_w256_0.cu", "pass_f32_w256_1.cu", "pass_f32_w512_0.cu",
-                  "pass_f32_w512_1.cu", "pass_f32_w1024_0.cu", "pass_f32_w1024_1.cu", "pass_f64.cu",
-                  "pass_f64_s1.cu", "pass_f64_rows.cu", "pass_f64_rows1.cu"]
+KERNEL_SOURCES = ["fft_tile.cuh", "fx.cuh", "pass_kernels.cuh"]   # every sweep is an instance of these
 
 
 def initial_state(key, spec, seed=0):
@@ -188,45 +184,21 @@ def cpu_sample(key, spec, max_seconds=25.0, steps=None, max_steps=None):
     return rec, psi, done
 
 
-def pass_flops_per_point(kind):
-    """Algorithmic FLOPs per grid point of one sweep, from its trace kind such
-    as 'y1024:F-KR-I': 5 log2(n) per n-point complex transform (the usual
-    radix-2 count) and 6 per pointwise complex multiplication substep."""
-    head, prog = kind.split(":", 1)
-    if head.startswith("line1d"):
-        # the on-chip 1D kernel: every step two transforms and two pointwise substeps
-        n = int(head[len("line1d"):])
-        return 2.0 * 5.0 * math.log2(n) + 2.0 * 6.0
-    n = int("".join(ch for ch in head if ch.isdigit()))
-    toks = prog.split("-")
-    ffts = sum(1 for t in toks if t in ("F", "I"))
-    pointwise = sum(1 for t in toks if t not in ("F", "I"))
-    return 5.0 * math.log2(n) * ffts + 6.0 * pointwise
-
-
-def alu_roofline(gpe, stream, kind, avg_ms, npoints, kernels):
-    """Roofline of a complex128 sweep: FP64 arithmetic against the measured
-    FP64 FMA rate of this GPU (complex128 sweeps are bound by it, not HBM)."""
-    peak = gpe.gpe_measure_fp64_peak(stream.cuda_stream) / 1e12
-    flops = pass_flops_per_point(kind) * npoints
-    achieved = flops / (avg_ms / 1e3) / 1e12
-    out = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-           "traffic": None, "kernel": kind, "kernel_avg_ms": avg_ms, "flops_per_launch": flops,
-           "peak_source": "measured: gpe_measure_fp64_peak (independent FP64 FMA chains on every SM)",
-           "flops_model": "5 log2(n) per n-point transform + 6 per pointwise complex multiply, per point",
-           "kernels": kernels}
-    if kind == "line1d256:real":
-        # one 256-point line is a latency problem, not a throughput one: its
-        # cluster of 16 CTAs (one warp each) issues one FP64 warp instruction
-        # per 64 cycles per SM sub-partition (measured), and a step is 62 such
-        # instructions in a chain plus two all-to-all exchanges (0.31 us each,
-        # measured for 16 CTAs)
-        steps = npoints / 256
-        model_us = 62 * 64 / 2.07e3 + 2 * 0.31
-        out["latency_model"] = {"us_per_step_model": model_us, "us_per_step": 1e3 * avg_ms / steps,
-                                "frac": model_us / (1e3 * avg_ms / steps),
-                                "model": "62 dependent FP64 warp instructions x 64 cycles at 2.07 GHz + two "
-                                         "cluster exchanges of 0.31 us (one line over a cluster of 16 CTAs)"}
+def hbm_roofline(kind, avg_ms, state_bytes, kernels, traffic=None):
+    """Roofline of a sweep: it reads and writes every point once (a 1D launch
+    does so once for all its steps)."""
+    peak, src = measured_peaks()
+    nbytes = 2.0 * state_bytes
+    achieved = nbytes / (avg_ms / 1e3) / 1e9
+    out = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+           "traffic": traffic, "kernel": kind, "kernel_avg_ms": avg_ms, "bytes_per_launch": nbytes,
+           "peak_source": src, "kernels": kernels}
+    if kind.startswith("line1d"):
+        out["on_chip"] = "one launch runs every step of the call with the lines on chip: bound by latency"
+    elif state_bytes < 100e6:
+        out["l2_resident"] = ("the %.0f MiB state stays in L2 between launches: HBM bytes do not bind "
+                              "these launches (each CTA runs one or two tiles; latency bound)"
+                              % (state_bytes / 2 ** 20))
     return out
 
 
@@ -350,8 +322,7 @@ def cufft_reference(spec, psi, steps=10):
 def config_record(key, steps=None):
     """One of the smaller configurations at its full length on an autotuned
     plan: updates/s from CUDA events, the per-kernel split from a traced
-    repeat, and the roofline of the dominant kernel (HBM for complex64,
-    FP64 arithmetic for complex128).  Turbulence runs read their spectra every
+    repeat, and the HBM roofline of the dominant kernel.  Turbulence runs read their spectra every
     200 steps inside the timed region, as the full workload does."""
     import torch
     import paper_2301_08275_gb300 as gpe
@@ -391,18 +362,7 @@ def config_record(key, steps=None):
     kind, (cnt, tot) = max(tr.items(), key=lambda kv: kv[1][1])
     kernels = {k: {"launches": c, "avg_ms": t / c} for k, (c, t) in tr.items()}
     state_bytes = spec.N * (8 if prec == gpe.GPE_C64 else 16)
-    if prec == gpe.GPE_C128:
-        # a 1D launch runs every step of the call: its flops per launch scale with them
-        per_launch = spec.N * (min(steps, 200) / cnt if kind.startswith("line1d") else 1)
-        roof = alu_roofline(gpe, stream, kind, tot / cnt, per_launch, kernels)
-    else:
-        peak, src = measured_peaks()
-        ach = 2.0 * state_bytes / (tot / cnt / 1e3) / 1e9
-        roof = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak, "kernel": kind,
-                "kernel_avg_ms": tot / cnt, "peak_source": src, "kernels": kernels}
-        if state_bytes < 100e6:
-            roof["l2_resident"] = "the %.0f MiB state stays in L2 between launches (latency bound)" % (
-                state_bytes / 2 ** 20)
+    roof = hbm_roofline(kind, tot / cnt, state_bytes, kernels)
     plan.close()
     return {"workload": wl["name"], "value": spec.N * steps / (ms / 1e3), "unit": UNIT, "steps": steps,
             "ms_per_step": ms / steps, "us_per_step": 1e3 * ms / steps, "dtype": wl["prec"], "tiles": tiles,
@@ -476,25 +436,10 @@ def run_ours(args, key, wl):
     dom = max(tr.items(), key=lambda kv: kv[1][1])
     kind, (cnt, tot) = dom
     avg_ms = tot / cnt
-    bytes_per_launch = 2.0 * spec.N * (8 if prec == gpe.GPE_C64 else 16)
     kernels = {k: {"launches": c, "avg_ms": t / c, "share": t / sum(x[1] for x in tr.values())}
                for k, (c, t) in tr.items()}
     state_bytes = spec.N * (8 if prec == gpe.GPE_C64 else 16)
-    if prec == gpe.GPE_C128:
-        # a 1D launch runs every step of its call: its flops per launch scale with them
-        per_launch = spec.N * (args.steps / cnt if kind.startswith("line1d") else 1)
-        roofline = alu_roofline(gpe, stream, kind, avg_ms, per_launch, kernels)
-    else:
-        peak, peak_src = measured_peaks()
-        achieved = bytes_per_launch / (avg_ms / 1e3) / 1e9
-        traffic = read_traffic(kind, key)
-        roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                    "traffic": traffic, "kernel": kind, "kernel_avg_ms": avg_ms,
-                    "bytes_per_launch": bytes_per_launch, "peak_source": peak_src, "kernels": kernels}
-        if state_bytes < 100e6:
-            roofline["l2_resident"] = ("the %.0f MiB state stays in L2 between launches: HBM bytes do not bind "
-                                       "these launches (each CTA runs one or two tiles; latency bound)"
-                                       % (state_bytes / 2 ** 20))
+    roofline = hbm_roofline(kind, avg_ms, state_bytes, kernels, read_traffic(kind, key))
 
     # end to end through the host-buffer entry point: every step copies the
     # state in from pinned host memory and the result back

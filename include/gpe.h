@@ -295,8 +295,7 @@ gpe_status gpe_norm_energy_noalloc(const gpe_plan_desc *desc, const void *psi_de
                                    double *out_host);
 
 /* Measured double-precision FMA throughput of the current device (a
- * measurement aid for the roofline of complex128 runs, which are bound by
- * FP64 arithmetic rather than HBM; no counterpart in the paper).  Launches a
+ * measurement aid; no counterpart in the paper).  Launches a
  * kernel of independent FMA chains on every SM on cuda_stream, synchronises
  * it, and writes the best of three timed launches to *flops_per_s (2 flops
  * per FMA).  GPE_EINVAL for a NULL pointer, GPE_ECUDA on a launch error. */

@@ -299,7 +299,9 @@ __global__ void __launch_bounds__(256) k_velocity(const SpecArgs s, const typena
 //  * neighbouring lanes of one shell add through shuffles, the first of them
 //    adds to the block's histogram, and the blocks add theirs to one in global
 //    memory (no per-block copies to sum afterwards).
-// Spectra of a 1024^2 complex64 field, the whole call: 458 -> 219 us.
+// Spectra of a 1024^2 complex64 field, the whole call: 458 -> 219 us with
+// this binning, 153 us with each mode binned beside its mirror image and the
+// derivative and the velocity taken inside the transforms (OP_DERIV, OP_VEL).
 struct Pf {
     float h, l;
 };

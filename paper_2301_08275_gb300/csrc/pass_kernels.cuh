@@ -1245,8 +1245,9 @@ __host__ __device__ constexpr size_t line1d_red_bytes(int nt) { return (sizeof(d
 // consecutive nonlinear half-steps, imaginary time renormalises the line after
 // every step.  Twiddles lie in pass order (in natural order the reads of the
 // later passes were up to 8-way bank conflicts: 64 lines of 4096 points 11.0
-// us per step, now 5.1; one line of 256 points 1.24, now 1.07); a second
-// exchange region saves a barrier per pass where it fits.
+// us per step, now 5.2, and 4.6 with the twiddles of the last two passes in
+// registers; one line of 256 points 1.24, now 1.07); a second exchange region
+// saves a barrier per pass where it fits.
 template <typename R, int N, int L> struct Line1DCfg {
     using T = GTile<R, N, 1, 1, true>;        // one line per thread group, swizzled exchange
     static constexpr int NT = L * T::TPL;

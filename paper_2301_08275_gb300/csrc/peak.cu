@@ -1,11 +1,11 @@
-// peak.cu - measured arithmetic peak of this GPU for the roofline of the
-// complex128 workloads (a measurement aid; the paper has no counterpart).
+// peak.cu - measured double-precision peak of this GPU (a measurement aid; the
+// paper has no counterpart).
 //
 // gpe_measure_fp64_peak launches a kernel of independent double-precision
 // fused multiply-add chains (eight per thread, no memory traffic inside the
 // timed loop) on every SM and returns the achieved FLOP/s (2 per FMA), timed
-// with CUDA events on the given stream.  The complex128 sweeps of the library
-// are bound by this rate, not by HBM.
+// with CUDA events on the given stream.  This
+// rate is why complex128 sweeps compute in 64-bit fixed point (fx.cuh).
 #include <cuda_runtime.h>
 
 #include "../../include/gpe.h"

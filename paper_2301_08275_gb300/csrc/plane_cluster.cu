@@ -14,7 +14,7 @@
 // The lines run the same transforms, tables and pointwise code as the streaming
 // sweeps (pass_kernels.cuh), so real-time steps give the same bits.
 // Measured, us per step on chip / as sweeps, one instance: 64^2 complex64 real
-// 5.5 / 12.4, imaginary 4.7 / 22.7; 128^2 complex64 6.6 / 13.5 and 6.2 / 24.8;
+// 4.9 / 11.7, imaginary 4.7 / 22.7; 128^2 complex64 6.6 / 13.5 and 6.2 / 24.8;
 // 64^2 complex128 8.7 / 17.4 and 13 / 31; 128^2 complex128 14 / 19 and 20 / 33.
 // 8 instances of 128^2 complex128: 20.6 / 22 and 29 / 39 (PLANE_MAX_POINTS).
 //
