@@ -621,13 +621,14 @@ template <typename R, int N, bool ROWS, int PROG> __host__ __device__ constexpr 
 {
     return ROWS && sizeof(R) == 4 && N == 512 && PROG == 12;
 }
-// Program 13: the same sweep with a trap, rows of 256 or 512 points; each thread
+// Program 13: the same sweep with a trap, rows of 64, 256 or 512 points; each thread
 // holds its trap factors along x (they change with the instance only) and a CTA
 // takes consecutive rows, so that they are read once per instance.  From the
 // table they are 16 bytes per point, as much as the state's reads and writes, and another 4
 // shared-memory/L1 wavefronts per 32 points.  Measured, us per sweep, table /
 // registers: 512^3 838 / 748, 128 instances of 512^2 219 / 192, 256^3 109 / 103,
-// 512 x 64^2 20.7 / 20.5.  Rows of 1024 points spill (17.2 / 18.1 at 1024^2),
+// 64^3 9.9 / 8.4, 16 of them 29.9 / 27.6 (64 x 256^2, as many points, 27.3 /
+// 28.2), 512 x 64^2 20.7 / 20.5.  Rows of 1024 points spill (17.2 / 18.1 at 1024^2),
 // rows of 128 gain nothing (34.0 / 35.0 at two 128^3).
 template <typename R, int N, bool ROWS, int PROG> __host__ __device__ constexpr bool pass_reg_trap()
 {
@@ -1537,7 +1538,7 @@ static cudaError_t launch_pass_t(const PassArgs &a, cudaStream_t st, const CUten
             if constexpr (sizeof(R) == 4 && N == 512) {
                 if (p == 4 && !a.vt_ax && !a.vt_o0 && !a.vt_o1) return launch_pass_p<R, N, ROWS, VAR, 12>(a, st, tmap);
             }
-            if constexpr (sizeof(R) == 4 && (N == 256 || N == 512)) {
+            if constexpr (sizeof(R) == 4 && (N == 64 || N == 256 || N == 512)) {
                 if (p == 4 && a.vt_ax) return launch_pass_p<R, N, ROWS, VAR, 13>(a, st, tmap);
             }
             if (p == 4) return launch_pass_p<R, N, ROWS, VAR, 4>(a, st, tmap);

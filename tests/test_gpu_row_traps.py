@@ -1,5 +1,5 @@
 """Row sweeps of complex64 that hold an instance's trap factors in registers
-(rows of 256 and 512 points): runs of consecutive rows that begin and end inside
+(rows of 64, 256 and 512 points): runs of consecutive rows that begin and end inside
 an instance or cross several, ragged last tiles, instances with their own trap.
 """
 import numpy as np
@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,batch", [((2, 512), 1), ((4, 512), 701), ((64, 512), 67), ((512, 4), 1), ((2, 256), 1203),
-                                     ((256, 256), 5), ((2, 4, 256), 301), ((4, 8, 512), 97)],
+                                     ((256, 256), 5), ((2, 4, 256), 301), ((4, 8, 512), 97), ((2, 64), 2051),
+                                     ((64, 64, 64), 3)],
                          ids=lambda v: "x".join(map(str, v)) if isinstance(v, tuple) else str(v))
 def test_instances_with_their_own_traps_match_the_oracle(orc, n, batch):
     """Same bound as the batches of shorter rows: 2e-5 after 5 steps."""
