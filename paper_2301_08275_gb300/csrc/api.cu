@@ -330,8 +330,12 @@ static int64_t turns_fx(double th)
     t -= rint(t);                                      // [-1/2, 1/2]
     return (int64_t)((uint64_t)(int64_t)ldexp(t, 63) << 1);
 }
-// an exponent V c (natural) in powers of two, to 53 fraction bits; beyond 2^+-200 the factor stays there
-static int64_t exponent_fx(double th) { return llrint(ldexp(std::max(-200.0, std::min(200.0, th * M_LOG2E)), 53)); }
+// an exponent V c (natural) in powers of two, to 53 fraction bits; beyond 2^+-FX_EXP_MAX the factor stays there
+static int64_t exponent_fx(double th)
+{
+    const double m = (double)FX_EXP_MAX;
+    return llrint(ldexp(std::max(-m, std::min(m, th * M_LOG2E)), 53));
+}
 
 // half-step trap angles and exponents of one instance on axis a, or of a sampled 1D potential
 static void trap_fx(const gpe_plan *p, int a, double gamma, int64_t *vq, int64_t *viq)
@@ -489,10 +493,12 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
             for (int64_t t = 0; t < na; ++t) kmax = std::max(kmax, ki[t] * (double)na);
             int ex = 0;
             if (kmax > 1.0) frexp(kmax, &ex);
+            // a factor out of the range of doubles: an exponent that makes the line NaN (fx_sweep)
+            if (!isfinite(kmax)) ex = 4096;
             p->kix_e[a] = ex;
             for (int64_t t = 0; t < na; ++t) {
                 ux[t] = fx_pack(one + llrint(ldexp(kt[2 * t], 62)), llrint(ldexp(kt[2 * t + 1], 62)));
-                kx[t] = (int64_t)ldexp(ki[t] * (double)na, 62 - ex);
+                kx[t] = isfinite(kmax) ? (int64_t)ldexp(ki[t] * (double)na, 62 - ex) : 0;
             }
             for (int64_t b = 0; nv && b < B; ++b) trap_fx(p, a, gam[3 * b + a], vq + b * na, viq + b * na);
             memcpy(tab.data() + 2 * na, ux.data(), na * sizeof(int4));

@@ -335,6 +335,9 @@ __device__ __forceinline__ fx2 fx_rotate(fx2 v, long long t)
     if (t + (1ll << 58) >= 0 && t <= (1ll << 58)) return fx_madd1(v, fx_small_offset(t));
     return fx_rotate_any(v, t);
 }
+// largest exponent of two that one term of an imaginary-time factor may have
+// (three of them add up, see fx_nimag, and fx_exp2m takes less than 1024)
+constexpr int FX_EXP_MAX = 340;
 // 2^-a for a held to 53 fraction bits (|a| < 1024), as a double: the nearest
 // whole number to the exponent, exp of the rest from its Maclaurin series to
 // the 14th term (z = 2 rest in [-1, 1], variable z / 4, 60 fraction bits; the

@@ -694,7 +694,11 @@ __device__ __forceinline__ void fx_nreal(fx2 (&v)[E], int q, const PassArgs &a, 
 }
 
 // nonlinear substep (imaginary time) on the line's doubles: the exponents of
-// interaction and trap are added to 53 fraction bits; s scales the values first
+// interaction and trap are added to 53 fraction bits; s scales the values first.
+// Three terms (the sweep's own axis, the other axes together, interaction with a
+// sampled potential), each held within +-FX_EXP_MAX: their sum stays below 2^10,
+// and a state whose norm is a double (its factors are then above 2^-256 where
+// it is, in each of a step's two half-steps) meets no limit.
 template <int E, int TPL>
 __device__ __forceinline__ void fx_nimag(double2 (&d)[E], double s, const PassArgs &a, const LineGeom &g, int tl)
 {
@@ -704,15 +708,18 @@ __device__ __forceinline__ void fx_nimag(double2 (&d)[E], double s, const PassAr
     long long line = 0;
     if (v0) line += v0[(int64_t)g.ti * a.o0n + g.c0];
     if (v1) line += v1[(int64_t)g.ti * a.o1n + g.c1];
+    constexpr long long most = (long long)FX_EXP_MAX << 53;
+    line = line > most ? most : line < -most ? -most : line;
     const double cl = a.nl_c * 1.4426950408889634074;
     const double gc = a.g[g.ti] * cl * (s * s);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         double x = gc * (d[e].x * d[e].x + d[e].y * d[e].y);
         if (vs) x += cl * vs[g.off + (int64_t)(tl + TPL * e) * a.estride];
-        // beyond 2^+-300 the factor is what it is there
+        // beyond 2^+-FX_EXP_MAX the factor is what it is there (high word of 340.0)
+        static_assert(FX_EXP_MAX == 340, "the constant below");
         const int hx = __double2hiint(x);
-        if ((hx & 0x7fffffff) > 0x4072c000) x = hx < 0 ? -300.0 : 300.0;
+        if ((hx & 0x7fffffff) >= 0x40754000) x = hx < 0 ? -(double)FX_EXP_MAX : (double)FX_EXP_MAX;
         long long ex = fx_from(x, -53) + line;
         if (vax) ex += vax[(int64_t)g.ti * a.nax + tl + TPL * e];
         const double f = s * fx_exp2m(ex);
