@@ -604,6 +604,12 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
         destroy(p);
         return fail(GPE_ECUDA, "uploading plan parameters failed");
     }
+    // the copies and the memset above went through the default stream and may be
+    // in flight still: a plan stream created non-blocking does not wait for them
+    if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+        destroy(p);
+        return fail(GPE_ECUDA, "uploading plan parameters failed");
+    }
     p->pin_len = (size_t)B * 6 + 64;
     if (cudaMallocHost((void **)&p->pin, sizeof(double) * p->pin_len) != cudaSuccess) {
         p->pin = nullptr;
@@ -1927,8 +1933,10 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
         for (int a = 0; a < p->ndim; ++a)
             for (int64_t j = 0; j < p->n[a]; ++j)
                 dk.push_back(2 * j == p->n[a] ? 0.0f : (float)(p->kf[a] * (double)(j < p->n[a] / 2 ? j : j - p->n[a])));
-        GPE_TRY(dalloc(p, (void **)&p->dk, dk.size() * sizeof(float)));
-        GPE_CUDA(cudaMemcpy(p->dk, dk.data(), dk.size() * sizeof(float), cudaMemcpyHostToDevice));
+        float *dev = nullptr;
+        GPE_TRY(dalloc(p, (void **)&dev, dk.size() * sizeof(float)));
+        GPE_CUDA(cudaMemcpyAsync(dev, dk.data(), dk.size() * sizeof(float), cudaMemcpyHostToDevice, p->st));
+        p->dk = dev;
     }
     auto gradient_parts = [&](const void *pb, int part) -> gpe_status {
         SpecArgs sv = sa;
@@ -2156,8 +2164,11 @@ gpe_status plan_prepare_resident(gpe_plan *p)
         h[5 * s] = (float)phi;
         for (int q = 0; q < 4; ++q) h[5 * s + 1 + q] = k.dk[q];
     }
-    GPE_TRY(dalloc(p, (void **)&p->dtab, sizeof(float) * h.size()));
-    GPE_CUDA(cudaMemcpy(p->dtab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
+    float *dev = nullptr;
+    GPE_TRY(dalloc(p, (void **)&dev, sizeof(float) * h.size()));
+    GPE_CUDA(cudaMemcpyAsync(dev, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice, p->st));
+    GPE_CUDA(cudaStreamSynchronize(p->st));    // a captured graph runs on another stream
+    p->dtab = dev;
     return GPE_OK;
 }
 

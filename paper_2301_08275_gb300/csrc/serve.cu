@@ -192,7 +192,9 @@ extern "C" gpe_status gpe_batch_create(const gpe_plan_desc *descs, int count, vo
         if (s == GPE_OK) {
             std::vector<int> slots(n);
             for (int j = 0; j < n; ++j) slots[j] = j;
-            if (cudaMemcpy(g.d_slots, slots.data(), sizeof(int) * n, cudaMemcpyHostToDevice) != cudaSuccess)
+            // (waited for: a captured graph reads them on another stream)
+            if (cudaMemcpyAsync(g.d_slots, slots.data(), sizeof(int) * n, cudaMemcpyHostToDevice, g.st) != cudaSuccess ||
+                cudaStreamSynchronize(g.st) != cudaSuccess)
                 s = sfail(GPE_ECUDA, "uploading slots failed");
         }
         b->groups.push_back(g);
@@ -223,7 +225,8 @@ static gpe_status batch_upload_ptrs(gpe_batch *b, void *const *psi)
     for (auto &g : b->groups) {
         std::vector<void *> h(g.members.size());
         for (size_t j = 0; j < h.size(); ++j) h[j] = psi[g.members[j]];
-        S_CUDA(cudaMemcpy(g.d_ptrs, h.data(), sizeof(void *) * h.size(), cudaMemcpyHostToDevice));
+        // on the caller's stream, which every group's work and every graph follows
+        S_CUDA(cudaMemcpyAsync(g.d_ptrs, h.data(), sizeof(void *) * h.size(), cudaMemcpyHostToDevice, b->st));
     }
     b->last_ptrs = cur;
     return GPE_OK;

@@ -1,0 +1,120 @@
+"""What the library's host code asks of the CUDA runtime, and in which order, against
+a stand-in for the runtime (fake_cudart.cpp; no GPU, no kernel runs)."""
+import ctypes
+import os
+import re
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+STREAM = 0x1000                      # a stream of the caller's: only its number counts
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+
+class Fake:
+    def __init__(self, lib):
+        self.lib = lib
+        lib.fake_log.restype = ctypes.c_char_p
+        lib.fake_live_bytes.restype = ctypes.c_size_t
+
+    def log(self):
+        return self.lib.fake_log().decode().splitlines()
+
+
+@pytest.fixture(scope="module")
+def loaded(tmp_path_factory):
+    import paper_2301_08275_gb300 as gpe
+    from paper_2301_08275_gb300 import buildlib
+    gpe.build()
+    path = str(tmp_path_factory.mktemp("fake") / "libgpe_fake.so")
+    objs = [os.path.join(buildlib.BUILD, s.replace(".cu", ".o")) for s in buildlib.SOURCES]
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-I" + os.path.join(CUDA, "include"),
+                    os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-o", path, "-lpthread"], check=True)
+    real = gpe.LIB_PATH, gpe._lib
+    gpe.LIB_PATH, gpe._lib = path, None
+    try:
+        yield gpe, Fake(gpe.lib())
+    finally:
+        gpe.LIB_PATH, gpe._lib = real
+        os.unlink(path)
+
+
+@pytest.fixture
+def gpe(loaded):
+    return loaded[0]
+
+
+@pytest.fixture
+def fake(loaded):
+    loaded[1].lib.fake_reset()
+    return loaded[1]
+
+
+def desc(gpe, n, prec=0, gamma=1.0, batch=1, V=None):
+    d = len(n)
+    return gpe.make_desc(n, (-6.0,) * d, (12.0,) * d, g=10.0, dt=1e-3, gamma=None if V is not None else (gamma,) * d,
+                         prec=prec, batch=batch, V=V)
+
+
+class Made:
+    """A plan on STREAM and a state for it."""
+
+    def __init__(self, gpe, n, prec=0, gamma=1.0, batch=1, V=None):
+        self.gpe = gpe
+        self.d, self.keep = desc(gpe, n, prec, gamma, batch, V)
+        self.batch = batch
+        self.h = gpe.gpe_plan_create(self.d, STREAM)
+        # (16 bytes aligned)
+        self.buf = np.zeros(2 * int(np.prod(n)) * batch + 2, dtype=np.float64)
+        self.psi = (self.buf.ctypes.data + 15) // 16 * 16
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        self.gpe.gpe_plan_destroy(self.h)
+
+
+def unordered(log):
+    """Lines of work on a stream of its own while work of the default stream (whose
+    calls may return before it is done, and which such a stream does not wait for)
+    has not been waited for."""
+    pending, out = False, []
+    for line in log:
+        what, _, rest = line.partition(" ")
+        s = rest.split(" ")[0]
+        if line in ("wait 0", "wait all"):
+            pending = False
+        elif what in ("copy", "set") and s == "0":
+            pending = True
+        elif what in ("copy", "set", "kernel") and pending:
+            out.append(line)
+    return out
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+@pytest.mark.parametrize("n", [(4096,), (64, 64), (128, 256), (128, 128, 64)], ids=lambda n: "x".join(map(str, n)))
+def test_uploads_are_complete_before_the_plan_stream_runs(gpe, fake, n, prec):
+    with Made(gpe, n, prec) as p:
+        gpe.gpe_step_real(p.h, p.psi, 2)
+        gpe.gpe_step_imag(p.h, p.psi, 2, 1.0, 0.0, 1, 1)
+        gpe.gpe_norm_energy(p.h, p.psi, 1)
+        gpe.gpe_spectrum(p.h, p.psi, 15, 1)
+    assert any(line.startswith("kernel") for line in fake.log())
+    assert unordered(fake.log()) == []
+
+
+@pytest.mark.parametrize("graph", [0, 1])
+def test_batch_uploads_are_complete_before_the_groups_run(gpe, fake, graph):
+    ns = [(64, 64), (64, 64), (256, 128), (128, 128, 64)]
+    made = [desc(gpe, n) for n in ns]
+    bufs = [np.zeros(2 * int(np.prod(n)) + 2) for n in ns]
+    ptrs = [(b.ctypes.data + 15) // 16 * 16 for b in bufs]
+    b = gpe.gpe_batch_create([m[0] for m in made], STREAM)
+    gpe.gpe_batch_step_real(b, ptrs, 2, graph)
+    gpe.gpe_batch_step_real(b, ptrs[1::-1] + ptrs[2:], 2, graph)
+    gpe.gpe_batch_norm_energy(b, ptrs)
+    gpe.gpe_batch_destroy(b)
+    assert unordered(fake.log()) == []
