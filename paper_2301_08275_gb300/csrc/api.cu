@@ -1883,18 +1883,16 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
     }
     sa.N = p->N;
     const size_t field = (size_t)p->N * p->csize;
-    if (!p->work[0]) {
-        for (int w = 0; w <= p->ndim; ++w) GPE_TRY(dalloc(p, &p->work[w], field));
-    }
+    // (each on its own: an earlier call may have failed between them)
+    for (int w = 0; w <= p->ndim; ++w)
+        if (!p->work[w]) GPE_TRY(dalloc(p, &p->work[w], field));
     for (int a = 0; a < 3; ++a) sa.lg[a] = ilog2_64(p->n[a]);
     sa.cubic = 1;
     for (int a = 0; a < p->ndim; ++a) sa.cubic = sa.cubic && sa.lratio[a] == 1.0;
     const int nv = velocity_blocks(sa);
-    if (!p->hist) {
-        // histogram and scale, then the partial sums of every component
-        GPE_TRY(dalloc(p, (void **)&p->hist, sizeof(double) * (2 * (size_t)ns + 1 + 3 * (size_t)nv)));
-        GPE_TRY(dalloc(p, (void **)&p->spec_out, sizeof(double) * 2 * (size_t)ns));
-    }
+    // histogram and scale, then the partial sums of every component
+    if (!p->hist) GPE_TRY(dalloc(p, (void **)&p->hist, sizeof(double) * (2 * (size_t)ns + 1 + 3 * (size_t)nv)));
+    if (!p->spec_out) GPE_TRY(dalloc(p, (void **)&p->spec_out, sizeof(double) * 2 * (size_t)ns));
     double *const partial = p->hist + 2 * ns + 1;
     // output slot of each kind: requested kinds in bit order
     double *slot[4] = {nullptr, nullptr, nullptr, nullptr};

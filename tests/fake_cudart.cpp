@@ -4,7 +4,7 @@
 // about is a line of the log:
 //   kernel S NAME | copy S | set S      work on stream S (0: the default stream)
 //   wait S                              the host waits for stream S (device: "wait all")
-//   resolve NAME                        a kernel's attributes are set or its occupancy asked for
+//   resolve NAME [VALUE]                an attribute of a kernel is set or its occupancy asked for
 //   alloc BYTES | begin | end           device allocation; stream capture
 #include <cuda_runtime_api.h>
 
@@ -128,9 +128,9 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void
     add("kernel " + sid(c->stream) + " " + name(f));
     return cudaSuccess;
 }
-cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int)
+cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute, int v)
 {
-    add("resolve " + name(f));
+    add("resolve " + name(f) + " " + std::to_string(v));
     return cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *, int, size_t, unsigned)

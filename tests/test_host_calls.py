@@ -118,3 +118,28 @@ def test_batch_uploads_are_complete_before_the_groups_run(gpe, fake, graph):
     gpe.gpe_batch_norm_energy(b, ptrs)
     gpe.gpe_batch_destroy(b)
     assert unordered(fake.log()) == []
+
+
+SPEC_PLANS = [((64, 128), 0), ((64, 128), 1), ((32, 64), 0), ((64, 64, 128), 0), ((512,), 1)]
+
+
+@pytest.mark.parametrize("n,prec", SPEC_PLANS, ids=lambda v: str(v))
+def test_spectra_after_a_failed_allocation(gpe, fake, n, prec):
+    """Whichever of a first spectrum's allocations fails, a later call makes the rest:
+    as many bytes live on the device as after a first call that met no failure."""
+    sizes = []
+    for k in range(12):
+        with Made(gpe, n, prec) as p:
+            start = fake.lib.fake_live_bytes()
+            fake.lib.fake_fail_alloc(k)
+            if k:
+                try:
+                    gpe.gpe_spectrum(p.h, p.psi, 15, 1)
+                except gpe.GpeError as e:
+                    assert e.status in (3, 4)
+                else:
+                    break
+            fake.lib.fake_fail_alloc(0)
+            gpe.gpe_spectrum(p.h, p.psi, 15, 1)
+            sizes.append(fake.lib.fake_live_bytes() - start)
+    assert len(sizes) > 4 and len(set(sizes)) == 1
