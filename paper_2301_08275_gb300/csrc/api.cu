@@ -1868,7 +1868,7 @@ extern "C" gpe_status gpe_spectrum(gpe_plan *p, const void *psi, unsigned kinds,
                                 "GPE_SPEC_QP and GPE_SPEC_NUM");
     const int64_t ns = nshells_of(p);
     if (nshells < ns) return fail(GPE_EINVAL, "nshells smaller than gpe_spectrum_nshells()");
-    if (ns > 6144) return fail(GPE_EUNSUPPORTED, "too many spectral shells");
+    if (ns > MAX_SHELLS) return fail(GPE_EUNSUPPORTED, "too many spectral shells");
     DeviceGuard dg(p->device);
     SpecArgs sa;
     memset(&sa, 0, sizeof(sa));

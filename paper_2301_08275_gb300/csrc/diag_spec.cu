@@ -624,15 +624,18 @@ cudaError_t launch_bin(const SpecArgs &s, void *const *uh, int64_t nshells, cons
     int64_t units = (((int64_t)1 << s.lg[0]) / 2 + 32) / 32;
     for (int a = 1; a < 3; ++a) units *= ((int64_t)1 << s.lg[a]) / 2 + 1;
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((units + BIN_THREADS / 32 - 1) / (BIN_THREADS / 32), 152 * 2));
+    // the attribute belongs to the process: always the largest size, so that no call
+    // takes room from another thread's launch
+    constexpr int most = (int)(2 * MAX_SHELLS * sizeof(unsigned long long));
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * 2 * (size_t)nshells, st);
     if (e != cudaSuccess) return e;
     if (s.prec == 0) {
-        e = cudaFuncSetAttribute(k_bin<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_bin<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
         k_bin<float><<<nb, BIN_THREADS, smem, st>>>(s, (const float2 *)uh[0], (const float2 *)uh[1], (const float2 *)uh[2],
                                             (int)nshells, partial, npartial, total, hist, scale);
     } else {
-        e = cudaFuncSetAttribute(k_bin<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_bin<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
         k_bin<double><<<nb, BIN_THREADS, smem, st>>>(s, (const double2 *)uh[0], (const double2 *)uh[1], (const double2 *)uh[2],
                                              (int)nshells, partial, npartial, total, hist, scale);

@@ -248,6 +248,8 @@ cudaError_t launch_imag_init(const double *out6, double *eprev, int64_t batch, i
 cudaError_t launch_imag_check(const double *out6, double *eprev, int64_t batch, double etol, int64_t chunk, int *stop,
                               int64_t *done, const int *err, cudaStream_t st);
 
+constexpr int64_t MAX_SHELLS = 6144;      // shells of a spectrum (two histograms of them in shared memory: 96 KiB)
+
 struct SpecArgs {
     int prec;
     int ndim;

@@ -143,3 +143,14 @@ def test_spectra_after_a_failed_allocation(gpe, fake, n, prec):
             gpe.gpe_spectrum(p.h, p.psi, 15, 1)
             sizes.append(fake.lib.fake_live_bytes() - start)
     assert len(sizes) > 4 and len(set(sizes)) == 1
+
+
+def test_spectra_of_two_threads_ask_for_one_shared_memory_size(gpe, fake):
+    """The size a kernel may take is the process's, not the call's: a call that set
+    a smaller one could take it from another thread's launch."""
+    for n in ((64, 64), (128, 64)):
+        with Made(gpe, n) as p:
+            for kinds in (3, 4):
+                gpe.gpe_spectrum(p.h, p.psi, kinds, 1)
+    got = {line for line in fake.log() if line.startswith("resolve") and "k_bin" in line}
+    assert len(got) == 1
