@@ -1389,8 +1389,8 @@ __global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DA
 // of the launch (transform, kinetic factor and inverse together keep it), and
 // the line is converted twice per launch.  L lines per CTA, interleaved in
 // shared memory.  Measured, us per step of 1 / 400 lines (FP64 before): 32
-// points 2.4 / 5.0 (17.2 / 17.3), 256 points 2.8 / 6.2 (22.6 / 99), 1024 points
-// 5.4 / 13 (30 / 118), 4096 points 23 / 54 (128 / 386).
+// points 2.7 / 2.9 (17.2 / 17.3), 256 points 3.1 / 4.3 (22.6 / 99), 1024 points
+// 5.8 / 13.5 (30 / 118), 4096 points 18 / 54 (128 / 386).
 template <int N, int L, int EPT> struct Line1DFx {
     using T = GTile<fx, N, L, 1, (L < 8), (N >= 16 ? EPT : 0)>;
     using G = FxGrowth<typename T::PL, ilog2c(N)>;
@@ -1610,14 +1610,18 @@ template <int N, int L, int EPT> static cudaError_t launch_line1d_fx_l(const Lin
     k_line1d_fx<N, L, EPT><<<(int)(ntiles < cap ? ntiles : cap), F::T::NT, F::smem, st>>>(a);
     return cudaGetLastError();
 }
-// Lines that do not fill the SMs: one per CTA and 4 points per thread (shorter
-// chains); otherwise 8 points per thread, with several lines in a CTA when
-// they are short.
+// Points per thread by the line's length alone, so that a line's result does not
+// depend on how many others there are: 4 (radix-4 passes, the shorter chain) up
+// to 1024 points, 8 beyond.  Measured, us per step of 1 / 303 / 1000 lines with 4
+// and with 8: 256 points 3.1 / 3.2 / 7.5 and 6.0 / 6.5 / 8.2, 1024 points
+// 5.8 / 9.3 / 30.6 and 7.6 / 9.9 / 33.5, 2048 points 11.4 / 22.6 / 78 and
+// 10.7 / 17.3 / 58, 4096 points 23 / 46 / 160 and 18 / 36 / 127.
+// Short lines share a CTA once there are more than the SMs take one by one.
 template <int N> static cudaError_t launch_line1d_fx(const Line1DArgs &a, cudaStream_t st)
 {
-    constexpr int L = N >= 256 ? 1 : N >= 64 ? 4 : 8;
-    if (a.batch < 2 * sm_count()) return launch_line1d_fx_l<N, 1, 4>(a, st);
-    return launch_line1d_fx_l<N, L, 0>(a, st);
+    constexpr int L = N >= 256 ? 1 : N >= 64 ? 4 : 8, EPT = N <= 1024 ? 4 : 0;
+    if (L == 1 || a.batch < 2 * sm_count()) return launch_line1d_fx_l<N, 1, EPT>(a, st);
+    return launch_line1d_fx_l<N, L, EPT>(a, st);
 }
 
 // Fewer instances than SMs: one line per CTA, so that no warp spends the SM's

@@ -1,0 +1,45 @@
+"""A line or an instance gives the same bits alone and in company: the number of
+instances of a plan chooses kernels, CTAs and tiles, never a line's arithmetic."""
+import numpy as np
+import pytest
+
+import gpe_inputs as gi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpe():
+    import torch
+    import paper_2301_08275_gb300 as g
+    g.build()
+    g.lib()
+    assert torch.cuda.is_available()
+    return g
+
+
+@pytest.mark.parametrize("imag", [False, True], ids=["real", "imag"])
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+@pytest.mark.parametrize("n", [8, 32, 64, 128, 256, 512, 1024, 2048, 4096])
+def test_lines_alone_and_in_company(gpe, n, prec, imag):
+    """Below and above two lines per SM, one CTA per line (complex128 real time has a
+    cluster kernel for up to 32 lines, switched off here: it factors differently)."""
+    import torch
+    sp = gi.Spec(n=(n,), lo=(-6.0,), length=(12.0,), g=20.0, dt=1e-3, gamma=(1.0,))
+    few = np.stack([gi.random_field(sp, seed=b, smooth=0.05) for b in range(3)])
+    dt = torch.complex128 if prec else torch.complex64
+    out = []
+    for batch in (3, 700):
+        p = gpe.Plan(sp.n, sp.lo, sp.length, g=sp.g, dt=sp.dt, gamma=sp.gamma[:1], prec=prec, batch=batch,
+                     g_each=[sp.g + b % 3 for b in range(batch)])
+        p.set_option(gpe.GPE_OPT_LINE_CLUSTER, 0)
+        x = torch.from_numpy(few[np.arange(batch) % 3]).cuda().to(dt)
+        if imag:
+            p.step_imag(x, 5, 1.0, 0.0, 5)
+        else:
+            p.step_real(x, 5)
+        torch.cuda.synchronize()
+        out.append(x.cpu().numpy())
+        p.close()
+    for b in (0, 1, 2, 303, 304, 698, 699):
+        assert np.array_equal(out[1][b], out[0][b % 3]), b
