@@ -174,8 +174,7 @@ gpe_status gpe_spectrum(gpe_plan *plan, const void *psi_dev, unsigned kinds, dou
 /* Plan options (implementation choices, no counterpart in the paper).  2D grids
  * of 64 or 128 points per axis are stepped on chip by one cluster per instance;
  * setting any of the options 1 to 7 on such a plan selects the sweeps that the
- * option is about (real-time results are the same bits).  Every
- * option takes 0 or 1; results are bit-identical for every setting (each
+ * option is about.  Every option takes 0 or 1; results are bit-identical for every setting (each
  * line's arithmetic does not depend on them, with the one exception noted at
  * GPE_OPT_GENERIC_PASSES), only the speed changes.
  *   GPE_OPT_TMA_STAGING  1 (default): tiles of the y and z sweeps are fetched

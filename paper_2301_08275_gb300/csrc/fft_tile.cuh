@@ -74,6 +74,10 @@ template <typename C> __device__ __forceinline__ C cmulc(C a, C b)
 }
 template <typename C, typename R> __device__ __forceinline__ C cscale(C a, R s) { return mk(a.x * s, a.y * s); }
 template <typename C> __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x) { return a.x * a.x + a.y * a.y; }
+// the same, rounded alike wherever it is inlined (cabs2 leaves to the compiler
+// which product it fuses into the sum): for what several kernels have to agree on
+__device__ __forceinline__ float norm2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
+__device__ __forceinline__ double norm2(double2 a) { return fma(a.x, a.x, a.y * a.y); }
 
 // Table entry of a unit factor: float -> (hi.x, hi.y, lo.x, lo.y), double -> value.
 template <typename R> struct UT;

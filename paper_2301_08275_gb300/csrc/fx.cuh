@@ -23,7 +23,7 @@
 //
 // Measured time of a 1024^2 complex128 real-time step: 451 us in FP64, 83 us
 // in fixed point; of a 128^2 imaginary-time step as sweeps 66 and 33 us (4 in
-// place of 8 points per thread among it), 24 us on chip (plane_cluster.cu).
+// place of 8 points per thread among it), 20 us on chip (plane_cluster.cu).
 //
 // Products: a 64-bit value is split as a = ah 2^32 + al with a SIGNED low half
 // (limbs), so every partial product is one signed IMAD.WIDE.  al * wl (at most

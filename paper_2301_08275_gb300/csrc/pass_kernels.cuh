@@ -344,7 +344,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
     const R cc = a.nl_cf;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        R th = gc * cabs2(v[e]);
+        R th = gc * norm2(v[e]);
         if (vs) th = fma(vs[off + (int64_t)(tl + TPL * e) * a.estride], cc, th);
         R f = fl * exp_r(-th);
         if (iax) f *= iax[(int64_t)ti * a.nax + tl + TPL * e];
@@ -714,8 +714,8 @@ __device__ __forceinline__ void fx_nimag(double2 (&d)[E], double s, const PassAr
     const double gc = a.g[g.ti] * cl * (s * s);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-        double x = gc * (d[e].x * d[e].x + d[e].y * d[e].y);
-        if (vs) x += cl * vs[g.off + (int64_t)(tl + TPL * e) * a.estride];
+        double x = gc * norm2(d[e]);
+        if (vs) x = fma(cl, vs[g.off + (int64_t)(tl + TPL * e) * a.estride], x);
         // beyond 2^+-FX_EXP_MAX the factor is what it is there (high word of 340.0)
         static_assert(FX_EXP_MAX == 340, "the constant below");
         const int hx = __double2hiint(x);
@@ -1195,7 +1195,7 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
                         nh[ln] = 0.0f;
                         nl[ln] = 0.0f;
 #pragma unroll
-                        for (int e = 0; e < E; ++e) df_acc(nh[ln], nl[ln], cabs2(v[ln][e]));
+                        for (int e = 0; e < E; ++e) df_acc(nh[ln], nl[ln], norm2(v[ln][e]));
                     }
                     group_sum_df<L, TPL, LPT>(nh, nl, reinterpret_cast<float2 *>(red), l0, tl);
 #pragma unroll
@@ -1207,7 +1207,7 @@ __global__ void __launch_bounds__(PassTile<R, N, ROWS, VAR>::NT, (pass_min_block
                     for (int ln = 0; ln < LPT; ++ln) {
                         sn[ln] = 0.0;
 #pragma unroll
-                        for (int e = 0; e < E; ++e) sn[ln] += (double)cabs2(v[ln][e]);
+                        for (int e = 0; e < E; ++e) sn[ln] += (double)norm2(v[ln][e]);
                     }
                     group_sum<L, TPL, LPT>(sn, red, l0, tl);
 #pragma unroll

@@ -12,15 +12,17 @@
 // buffer held has been read before the barrier that precedes its next writes).
 //
 // The lines run the same transforms, tables and pointwise code as the streaming
-// sweeps (pass_kernels.cuh), so real-time steps give the same bits.
+// sweeps (pass_kernels.cuh), so their results are the same bits.
 // Measured, us per step on chip / as sweeps, one instance: 64^2 complex64 real
-// 4.9 / 11.7, imaginary 4.7 / 22.7; 128^2 complex64 6.6 / 13.5 and 6.2 / 24.8;
-// 64^2 complex128 8.7 / 17.4 and 13 / 31; 128^2 complex128 14 / 19 and 20 / 33.
-// 8 instances of 128^2 complex128: 20.6 / 22 and 29 / 39 (PLANE_MAX_POINTS).
+// 4.7 / 11.7, imaginary 5.3 / 22.7; 128^2 complex64 6.1 / 13.5 and 6.5 / 24.8;
+// 64^2 complex128 9.0 / 17.4 and 14 / 31; 128^2 complex128 14 / 19 and 20 / 33.
+// 8 instances of 128^2 complex128: 20.5 / 22 and 29 / 39 (PLANE_MAX_POINTS).
 //
-// In imaginary time the norm is summed over the cluster (in another order than the
-// streaming reduction: the last places can differ), and the renormalisation,
-// the last row sweep of a step and the first of the next stay in registers.
+// In imaginary time the norm is summed over the cluster in the order of the
+// streaming reduction (rows as group_sum and group_sum_df add them, then
+// k_reduce_lines' warps of 32 rows), so these steps give the same bits too; the
+// renormalisation, the last row sweep of a step and the first of the next stay
+// in registers.
 #include "pass_kernels.cuh"
 
 namespace gpe {
@@ -73,8 +75,9 @@ template <typename R, int N0, int N1> struct PlaneCfg {
     static constexpr int NT = Rows::NT;
     static_assert(NT == Cols::NT, "one thread layout for both sweeps");
     static constexpr int POINTS = N0 * N1 / CS;
-    static constexpr size_t smem = 2 * sizeof(C) * POINTS + 16 * (size_t)(N0 + N1) + 16 * sizeof(double) * 2 +
-                                   32 * sizeof(double) + 2 * sizeof(unsigned) * (L0 > L1 ? L0 : L1);
+    static_assert(NT >= N1 && N1 <= 128, "the rows' norms are added by one thread each, four warps at most");
+    static constexpr size_t smem = 2 * sizeof(C) * POINTS + 16 * (size_t)(N0 + N1) + 2 * sizeof(double) * N1 +
+                                   sizeof(double) * NT + 2 * sizeof(unsigned) * (L0 > L1 ? L0 : L1);
 };
 
 template <typename R, int N0, int N1, bool IMAG>
@@ -92,9 +95,9 @@ __global__ void __launch_bounds__(PlaneCfg<R, N0, N1>::NT) k_plane(const PlaneAr
     C *const bufb = bufa + Cfg::POINTS;                      // columns: point y of column l at y L1 + l
     U *const tw0 = reinterpret_cast<U *>(bufb + Cfg::POINTS);
     U *const tw1 = tw0 + N0;
-    double *const nrm = reinterpret_cast<double *>(tw1 + N1);    // [2][16] norms of the CTAs
-    double *const red = nrm + 32;                            // [32] warp sums
-    unsigned *const lsc = reinterpret_cast<unsigned *>(red + 32);
+    double *const nrm = reinterpret_cast<double *>(tw1 + N1);    // [2][N1] norms of the rows
+    double *const red = nrm + 2 * N1;                        // [NT] of the sums
+    unsigned *const lsc = reinterpret_cast<unsigned *>(red + NT);
     const int t = threadIdx.x, lr = t % L0, tr = t / L0, lc = t % L1, tc = t / L1;
     if (pa.rows.stop && *reinterpret_cast<const volatile int *>(pa.rows.stop)) return;   // uniform over the grid
     Rows::load_twiddles(tw0, static_cast<const U *>(pa.rows.tw), t, NT);
@@ -136,9 +139,10 @@ __global__ void __launch_bounds__(PlaneCfg<R, N0, N1>::NT) k_plane(const PlaneAr
         if (sizeof(R) == 8)
             for (int i = t; i < 2 * (L0 > L1 ? L0 : L1); i += NT) lsc[i] = 0;
     };
-    auto row_sweep = [&](const PassArgs &a, int op_pre, int fft1, int op_mid, int fft2) {
+    // (scale: of complex128 values before OP_NIMAG, as OP_SCALE_NIMAG has it)
+    auto row_sweep = [&](const PassArgs &a, int op_pre, int fft1, int op_mid, int fft2, double scale = 1.0) {
         if constexpr (sizeof(R) == 8) {
-            fx_sweep<Rows, false>(v, a, gr, 1.0, bufa, bufa, tr, lr, tw0, lsc, op_pre, fft1, op_mid, fft2);
+            fx_sweep<Rows, false>(v, a, gr, scale, bufa, bufa, tr, lr, tw0, lsc, op_pre, fft1, op_mid, fft2);
         } else {
             C w[1][E];
 #pragma unroll
@@ -221,54 +225,65 @@ __global__ void __launch_bounds__(PlaneCfg<R, N0, N1>::NT) k_plane(const PlaneAr
         r.nl_c = 0.5 * pa.dt;
         r.vq_full = 0;
         r.nl_cf = pa.half_dtf;
+        double sc = 1.0;             // renormalisation factor that v still lacks
+        auto rescale = [&]() {
+#pragma unroll
+            for (int e = 0; e < E; ++e) v[e] = cscale(v[e], (R)sc);
+        };
 #pragma unroll 1
         for (int s = 0; s < pa.nsteps; ++s) {
-            row_sweep(r, OP_NIMAG, -1, OP_NONE, 0);
+            if constexpr (sizeof(R) == 4) rescale();
+            row_sweep(r, OP_NIMAG, -1, OP_NONE, 0, sc);
             exchange_to_columns();
             column_sweep(pa.cols, OP_KIMAG);
             row_sweep(r, OP_NONE, 1, OP_NIMAG, 0);
-            // norm: thread, warp, CTA, cluster, each in a fixed order
-            double n = 0.0;
+            // every row's norm, to every CTA.  In complex64 the threads of a row's
+            // first warp have its sum, in complex128 all of them.
+            constexpr int SND = sizeof(R) == 8 ? CS : 32 / L0 < T0 ? 32 / L0 : T0;
+            static_assert(SND <= T0 && CS % SND == 0, "senders of a row");
+            double sn[1] = {0.0};
             if constexpr (sizeof(R) == 4) {
-                float nh = 0.0f, nl = 0.0f;
+                float nh[1] = {0.0f}, nl[1] = {0.0f};
 #pragma unroll
-                for (int e = 0; e < E; ++e) df_acc(nh, nl, cabs2(v[e]));
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const float oh = __shfl_xor_sync(0xffffffffu, nh, o), ol = __shfl_xor_sync(0xffffffffu, nl, o);
-                    df_add(nh, nl, oh, ol);
-                }
-                n = (double)nh + (double)nl;
+                for (int e = 0; e < E; ++e) df_acc(nh[0], nl[0], norm2(v[e]));
+                group_sum_df<L0, T0, 1>(nh, nl, reinterpret_cast<float2 *>(red), lr, tr);
+                sn[0] = (double)nh[0] + (double)nl[0];
             } else {
 #pragma unroll
-                for (int e = 0; e < E; ++e) n += cabs2(v[e]);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+                for (int e = 0; e < E; ++e) sn[0] += norm2(v[e]);
+                group_sum<L0, T0, 1>(sn, red, lr, tr);
+                clear();
             }
-            if ((t & 31) == 0) red[t >> 5] = n;
-            __syncthreads();
-            clear();
-            double *const slot = nrm + 16 * (s & 1);
-            if (t < CS) {
-                double m = 0.0;
-                for (int w = 0; w < NT / 32; ++w) m += red[w];
-                pl_store(pl_map(smem_addr(slot + c), (unsigned)t), m);
+            double *const slot = nrm + N1 * (s & 1);
+            if (tr < SND) {
+                const unsigned at = smem_addr(slot + gr.c0);
+#pragma unroll
+                for (int k = 0; k < CS; k += SND) pl_store(pl_map(at, (unsigned)(tr + k)), sn[0]);
             }
             pl_sync();
-            double tot = (t & 31) < CS ? slot[t & 31] : 0.0;
+            // FP64 additions keep a sub-partition for 64 cycles each: a warp per 32
+            // rows, then one warp for their sums and the factor
+            if (t < N1) {
+                double x = slot[t];
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-            tot = __shfl_sync(0xffffffffu, tot, 0) * pa.dv;
-            double sc = 1.0;
-            if (!(tot > 0.0) || !isfinite(tot)) {
-                if (t == 0 && c == 0) atomicOr(pa.rows.err, (int)ERR_NUMERIC);
-            } else {
-                sc = sqrt(pa.target / tot);
+                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                if ((t & 31) == 0) red[t >> 5] = x;
             }
-            const R f = (R)sc;
-#pragma unroll
-            for (int e = 0; e < E; ++e) v[e] = cscale(v[e], f);
+            __syncthreads();
+            if (t == 0) {
+                const double tot = (N1 == 128 ? (red[0] + red[1]) + (red[2] + red[3]) : red[0] + red[1]) * pa.dv;
+                double f = 1.0;
+                if (!(tot > 0.0) || !isfinite(tot)) {
+                    if (c == 0) atomicOr(pa.rows.err, (int)ERR_NUMERIC);
+                } else {
+                    f = sqrt(pa.target / tot);
+                }
+                red[N1 / 32] = f;
+            }
+            __syncthreads();
+            sc = red[N1 / 32];
         }
+        rescale();
     }
 #pragma unroll
     for (int e = 0; e < E; ++e) psi[gr.off + tr + T0 * e] = v[e];

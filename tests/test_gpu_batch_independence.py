@@ -43,3 +43,40 @@ def test_lines_alone_and_in_company(gpe, n, prec, imag):
         p.close()
     for b in (0, 1, 2, 303, 304, 698, 699):
         assert np.array_equal(out[1][b], out[0][b % 3]), b
+
+
+def imag(gpe, sp, psi, prec, batch, steps, option=None, V=None):
+    import torch
+    p = gpe.Plan(sp.n, sp.lo, sp.length, g=sp.g, dt=sp.dt, gamma=None if V is not None else sp.gamma[:2], prec=prec,
+                 batch=batch, g_each=[sp.g + b % 3 for b in range(batch)], V=V)
+    if option is not None:
+        p.set_option(option, 0)
+    x = torch.from_numpy(psi[np.arange(batch) % 3]).cuda().to(torch.complex128 if prec else torch.complex64)
+    p.trace()
+    p.step_imag(x, steps, 1.0, 0.0, steps)
+    torch.cuda.synchronize()
+    kinds = p.trace_read()
+    p.close()
+    return x.cpu().numpy(), {k.split(":")[0] for k in kinds if not k.endswith("diag")}
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+@pytest.mark.parametrize("sampled", [False, True], ids=["trap", "sampled"])
+@pytest.mark.parametrize("n", [(64, 64), (64, 128), (128, 64), (128, 128)], ids=lambda n: "x".join(map(str, n)))
+def test_imaginary_time_on_chip_and_as_sweeps(gpe, n, sampled, prec):
+    """2D grids of 64 or 128 points per axis are stepped on chip up to 2^17 points in
+    all, as sweeps beyond and with an option of the sweeps: the same bits."""
+    sp = gi.Spec(n=n, lo=(-6.0, -5.0), length=(12.0, 10.0), g=50.0, dt=1e-3, gamma=(0.0, 0.0) if sampled else (1.0, 1.4))
+    V = gi.anharmonic(sp, gamma=(1.0, 1.5), lam=0.1) if sampled else None
+    psi = np.stack([gi.random_field(sp, seed=b, smooth=0.03) for b in range(3)])
+    most = (1 << 17) // (n[0] * n[1])
+    a, ka = imag(gpe, sp, psi, prec, 3, 12, V=V)
+    b, kb = imag(gpe, sp, psi, prec, 3, 12, gpe.GPE_OPT_TILE_X, V=V)
+    at, kat = imag(gpe, sp, psi, prec, most, 12, V=V)
+    over, kover = imag(gpe, sp, psi, prec, most + 1, 12, V=V)
+    plane = {"plane%dx%d" % n}
+    assert ka == kat == plane and kb == kover == {"x%d" % n[0], "y%d" % n[1]}
+    assert np.array_equal(a, b)
+    for i in range(most + 1):
+        assert np.array_equal(over[i], a[i % 3]), i
+        assert i == most or np.array_equal(at[i], a[i % 3]), i
