@@ -244,8 +244,9 @@ gpe_status gpe_plan_get_option(const gpe_plan *plan, int option, int64_t *value)
  * `reps` samples per candidate taken round-robin across the candidates (a
  * sample is one step, or several on grids whose step is shorter than about
  * 2 ms), and keeps the candidate with the fastest sample.  Choices are remembered per
- * grid, precision and instance count for the life of the process, so later
- * plans of the same shape tune without timing.  Needs two state-sized device
+ * device, grid, precision, instance count and kind of potential (which axes have a trap,
+ * sampled or not) for the life of the process, so later plans of the same kind
+ * tune without timing.  Needs two state-sized device
  * scratch arrays for the duration of the call; synchronises the plan stream.
  * 1D plans have nothing to tune (GPE_OK). */
 #define GPE_TUNE_NO_TMA 1

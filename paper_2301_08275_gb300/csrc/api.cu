@@ -1447,14 +1447,16 @@ struct TuneVal {
     bool tma[3];
 };
 std::mutex g_tune_mu;
-std::map<std::string, TuneVal> g_tune;   // choices per grid/precision/instances/flags, process-wide
+std::map<std::string, TuneVal> g_tune;   // choices per tune_key, process-wide
 }  // namespace
 
+// (which axes are trapped and whether a potential is sampled choose the row kernel)
 static std::string tune_key(const gpe_plan *p, int64_t batch, int flags)
 {
-    char buf[160];
-    snprintf(buf, sizeof(buf), "%d/%d/%lldx%lldx%lld/%lld/%d", p->prec, p->ndim, (long long)p->n[0],
-             (long long)p->n[1], (long long)p->n[2], (long long)batch, flags);
+    char buf[192];
+    snprintf(buf, sizeof(buf), "%d/%d/%d/%lldx%lldx%lld/%lld/%d/%d%d%d%d%d", p->device, p->prec, p->ndim,
+             (long long)p->n[0], (long long)p->n[1], (long long)p->n[2], (long long)batch, flags, p->trap[0], p->trap[1],
+             p->trap[2], p->vsamp != nullptr, p->generic_passes);
     return buf;
 }
 

@@ -154,3 +154,26 @@ def test_spectra_of_two_threads_ask_for_one_shared_memory_size(gpe, fake):
                 gpe.gpe_spectrum(p.h, p.psi, kinds, 1)
     got = {line for line in fake.log() if line.startswith("resolve") and "k_bin" in line}
     assert len(got) == 1
+
+
+def timed(gpe, fake, p):
+    """Sweeps that gpe_plan_autotune launches."""
+    fake.lib.fake_reset()
+    gpe.gpe_plan_autotune(p.h, p.psi, 1, 0)
+    return sum(line.startswith("kernel") and "k_pass" in line for line in fake.log())
+
+
+def test_tuner_remembers_by_the_kind_of_potential(gpe, fake):
+    """Row sweeps with a trap, without one and with a sampled potential are different
+    kernels: a choice made for one is not the others'."""
+    n = (512, 32)
+    V = np.zeros((32, 512))
+    kinds = [dict(gamma=1.0), dict(gamma=0.0), dict(V=V)]
+    for kw in kinds:
+        with Made(gpe, n, **kw) as p:
+            assert timed(gpe, fake, p) > 0
+    for kw in kinds:
+        with Made(gpe, n, **kw) as p:
+            assert timed(gpe, fake, p) == 0
+            gpe.gpe_plan_set_option(p.h, gpe.GPE_OPT_GENERIC_PASSES, 1)
+            assert timed(gpe, fake, p) > 0
