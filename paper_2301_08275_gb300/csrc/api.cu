@@ -1495,7 +1495,6 @@ extern "C" gpe_status gpe_plan_autotune(gpe_plan *p, const void *psi, int reps, 
     if (reps < 1 || reps > 1000) return fail(GPE_EINVAL, "reps must be in [1, 1000]");
     if (flags & ~GPE_TUNE_NO_TMA) return fail(GPE_EINVAL, "unknown autotune flag");
     if (p->ndim == 1) return GPE_OK;
-    if (plane_applies(p)) return GPE_OK;       // stepped on chip: no sweeps to choose
     if (p->cur_count > 0) return fail(GPE_EINVAL, "plan is in use by a batch launch");
     DeviceGuard dg(p->device);
     if (!dg.ok) return fail(GPE_ECUDA, "cannot select the plan's device");

@@ -177,3 +177,12 @@ def test_tuner_remembers_by_the_kind_of_potential(gpe, fake):
             assert timed(gpe, fake, p) == 0
             gpe.gpe_plan_set_option(p.h, gpe.GPE_OPT_GENERIC_PASSES, 1)
             assert timed(gpe, fake, p) > 0
+
+
+@pytest.mark.parametrize("clusters", [8, 0])
+def test_tuner_times_the_sweeps_of_planes_stepped_on_chip(gpe, fake, clusters):
+    """Trap schedules and diagnostics of such a plan are sweeps, and so are all its
+    steps where no cluster of that size can be placed."""
+    fake.lib.fake_clusters(clusters)
+    with Made(gpe, (128, 64 if clusters else 128)) as p:
+        assert timed(gpe, fake, p) > 0
