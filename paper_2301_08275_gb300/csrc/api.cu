@@ -141,6 +141,7 @@ struct gpe_plan {
     int tx_extra = 0;                       // GPE_OPT_TEST_STALL_COPIES
     bool generic_passes = false;            // GPE_OPT_GENERIC_PASSES
     bool sweeps_chosen = false;             // an option asked for particular sweeps
+    bool resolving = false;                 // plan_prepare: steps resolve their kernels and launch none
     bool line_cluster = true;               // GPE_OPT_LINE_CLUSTER
     bool no_dither = false;                 // GPE_OPT_NO_DITHER
     // trap tables of one time level (gpe_step_real_trap), allocated on first use
@@ -907,6 +908,11 @@ static gpe_status run(gpe_plan *p, const PassArgs &a_in)
     PassArgs a = a_in;
     a.err = p->err;
     a.generic = p->generic_passes ? 1 : 0;
+    if (p->resolving) {
+        a.ntiles = 0;
+        const cudaError_t e = launch_pass(p->prec, a.axis == 0, a, p->st, nullptr, p->tile_var[a.axis]);
+        return e == cudaSuccess ? GPE_OK : fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
+    }
     const CUtensorMap *tm = nullptr;
     // strided sweeps over one array of back-to-back instances, with whole
     // tiles of consecutive x lines, take the copy-engine staging
@@ -1021,7 +1027,7 @@ static cudaError_t plane_steps(gpe_plan *p, void *psi, int64_t nsteps, bool imag
 {
     PlaneArgs a;
     memset(&a, 0, sizeof(a));
-    a.count = active_count(p);
+    a.count = p->resolving ? 0 : active_count(p);
     a.rows = make_pass(p, 0, psi, psi, a.count);
     a.cols = make_pass(p, 1, psi, psi, a.count);
     set_nreal(p, a.rows, true);
@@ -1105,7 +1111,7 @@ static gpe_status step_real_dev(gpe_plan *p, void *psi, int64_t nsteps, const do
             l.psi = psi;
             l.batch = B;
             l.n = (int)p->n[0];
-            l.nsteps = std::min(chunk, nsteps - done);
+            l.nsteps = p->resolving ? 0 : std::min(chunk, nsteps - done);
             l.imag = 0;
             l.tw = p->tw[0];
             l.kt = p->kt[0];
@@ -1691,7 +1697,7 @@ static gpe_status imag_steps(gpe_plan *p, void *psi, int64_t nsteps, double targ
         l.psi = psi;
         l.batch = B;
         l.n = (int)p->n[0];
-        l.nsteps = nsteps;
+        l.nsteps = p->resolving ? 0 : nsteps;
         l.imag = 1;
         l.tw = p->tw[0];
         l.kt = p->ki[0];
@@ -1745,6 +1751,7 @@ static gpe_status imag_steps(gpe_plan *p, void *psi, int64_t nsteps, double targ
         set_nimag(p, x2);
         x2.red = RED_NORM;
         GPE_TRY(run(p, x2));
+        if (p->resolving) continue;
         cudaError_t e = launch_reduce_lines(p->partials, p->lines_cap, 0, 1, B, p->N / p->n[0], p->csum, p->sums,
                                             p->red_count, p->st, p->dv, target, p->scale, p->err, p->cur_stop);
         if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("renormalisation: ") + cudaGetErrorString(e));
@@ -2026,37 +2033,29 @@ int64_t plan_capacity(const gpe_plan *p) { return p->batch; }
 int64_t plan_points(const gpe_plan *p) { return p->N; }
 size_t plan_point_bytes(const gpe_plan *p) { return p->csize; }
 
-// Resolve every kernel the plan will launch (function attributes, occupancy)
-// with zero-work launches, so that later launches can be captured in graphs.
-gpe_status plan_prepare(gpe_plan *p)
+// Resolve the kernels that the plan's real-time (imag: imaginary-time) steps and
+// diagnostics launch (function attributes, occupancy), so that later launches can
+// be captured in graphs: the steps' own code, with no work in any launch, for
+// one instance and for all of them (the number chooses kernels too).
+gpe_status plan_prepare(gpe_plan *p, int imag)
 {
     DeviceGuard dg(p->device);
-    for (int a = 0; a < p->ndim; ++a) {
+    p->resolving = true;
+    gpe_status s = GPE_OK;
+    for (int a = 0; a < p->ndim && s == GPE_OK; ++a) {
         PassArgs t = make_pass(p, a, nullptr, nullptr, 0);
-        t.ntiles = 0;
-        cudaError_t e = launch_pass(p->prec, a == 0, t, p->st);
-        if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
+        t.red = a ? RED_DIAG_K : RED_DIAG_X;
+        s = run(p, t);
     }
-    if (plane_shape(p->ndim, p->n)) {
-        PlaneArgs a;
-        memset(&a, 0, sizeof(a));
-        for (a.imag = 0; a.imag < 2; ++a.imag) {
-            const cudaError_t e = p->prec == GPE_C64 ? launch_plane_f32((int)p->n[0], (int)p->n[1], a, p->st)
-                                                     : launch_plane_f64((int)p->n[0], (int)p->n[1], a, p->st);
-            if (e != cudaSuccess && e != cudaErrorNotSupported)
-                return fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
-            if (e != cudaSuccess) cudaGetLastError();
-        }
+    for (int64_t count = 1; s == GPE_OK; count = p->batch) {
+        p->cur_count = count;
+        // 3 steps: first, steady and last sweeps
+        s = imag ? imag_steps(p, nullptr, 1, 1.0) : step_real_dev(p, nullptr, 3);
+        if (count == p->batch) break;
     }
-    if (p->ndim == 1) {
-        Line1DArgs l;
-        memset(&l, 0, sizeof(l));
-        l.n = (int)p->n[0];
-        l.batch = 0;
-        cudaError_t e = launch_line1d(p->prec, l, p->st);
-        if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
-    }
-    return GPE_OK;
+    p->cur_count = 0;
+    p->resolving = false;
+    return s;
 }
 
 // Give slot `slot` of a plan new interaction and trap parameters: host FP64
@@ -2168,6 +2167,10 @@ gpe_status plan_prepare_resident(gpe_plan *p)
     GPE_CUDA(cudaMemcpyAsync(dev, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice, p->st));
     GPE_CUDA(cudaStreamSynchronize(p->st));    // a captured graph runs on another stream
     p->dtab = dev;
+    ResidentArgs r;
+    memset(&r, 0, sizeof(r));
+    cudaError_t e = launch_resident2d((int)p->n[0], r, p->st);     // resolves the kernel
+    if (e != cudaSuccess) return fail(GPE_ECUDA, std::string("prepare: ") + cudaGetErrorString(e));
     return GPE_OK;
 }
 

@@ -184,7 +184,7 @@ struct Line1DArgs {
     void *psi;
     int64_t batch;
     int n;
-    int64_t nsteps;
+    int64_t nsteps;         // 0: the kernel is resolved and not launched
     int imag;               // 0 real time, 1 imaginary time with per-step renormalisation
     const void *tw;
     const void *kt;         // offsets exp(-i k^2 dt/2) - 1 (real time) or exp(-k^2 dt/2)/n (imag)

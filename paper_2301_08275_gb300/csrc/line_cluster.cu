@@ -284,6 +284,7 @@ template <int CS> cudaError_t launch_cl(const Line1DArgs &a, cudaStream_t st)
         }
         if (g_cl.ok[dev][slot] < 0) return cudaErrorNotSupported;
     }
+    if (a.nsteps <= 0) return cudaSuccess;
     return cudaLaunchKernelEx(&cfg, k_line1d_cluster<CS>, a);
 }
 
@@ -291,8 +292,7 @@ template <int CS> cudaError_t launch_cl(const Line1DArgs &a, cudaStream_t st)
 
 bool line1d_cluster_applies(const Line1DArgs &a)
 {
-    return !a.imag && (a.n == 64 || a.n == 128 || a.n == 256) && a.batch >= 1 && a.batch <= LINE_CLUSTER_MAX_BATCH &&
-           a.nsteps >= 1;
+    return !a.imag && (a.n == 64 || a.n == 128 || a.n == 256) && a.batch >= 1 && a.batch <= LINE_CLUSTER_MAX_BATCH;
 }
 
 cudaError_t launch_line1d_cluster(const Line1DArgs &a, cudaStream_t st)

@@ -1591,7 +1591,7 @@ template <typename R, int N, int L> static cudaError_t launch_line1d_l(const Lin
     cudaError_t e = prepare(k_line1d<R, N, L>, lc, Line1DCfg<R, N, L>::NT, smem, &cap);
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (a.batch + L - 1) / L;
-    if (ntiles <= 0) return cudaSuccess;
+    if (ntiles <= 0 || a.nsteps <= 0) return cudaSuccess;
     const int grid = (int)(ntiles < cap ? ntiles : cap);
     k_line1d<R, N, L><<<grid, Line1DCfg<R, N, L>::NT, smem, st>>>(a);
     return cudaGetLastError();
@@ -1606,7 +1606,7 @@ template <int N, int L, int EPT> static cudaError_t launch_line1d_fx_l(const Lin
     cudaError_t e = prepare(k_line1d_fx<N, L, EPT>, lc, F::T::NT, F::smem, &cap);
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (a.batch + L - 1) / L;
-    if (ntiles <= 0) return cudaSuccess;
+    if (ntiles <= 0 || a.nsteps <= 0) return cudaSuccess;
     k_line1d_fx<N, L, EPT><<<(int)(ntiles < cap ? ntiles : cap), F::T::NT, F::smem, st>>>(a);
     return cudaGetLastError();
 }

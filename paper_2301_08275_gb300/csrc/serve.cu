@@ -34,7 +34,7 @@ int64_t plan_capacity(const gpe_plan *p);
 int64_t plan_points(const gpe_plan *p);
 size_t plan_point_bytes(const gpe_plan *p);
 gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamma);
-gpe_status plan_prepare(gpe_plan *p);
+gpe_status plan_prepare(gpe_plan *p, int imag);
 gpe_status plan_run(gpe_plan *p, int mode, void *const *dptrs, const int *dslots, int64_t count, int64_t nsteps,
                     double target, double *out6_host);
 gpe_status plan_run_async(gpe_plan *p, int mode, void *const *dptrs, const int *dslots, int64_t count, int64_t nsteps,
@@ -185,7 +185,7 @@ extern "C" gpe_status gpe_batch_create(const gpe_plan_desc *descs, int count, vo
             if (g.resident) s = plan_prepare_resident(g.plan);
             else s = gpe_plan_autotune(g.plan, nullptr, 3, GPE_TUNE_NO_TMA);
         }
-        if (s == GPE_OK) s = plan_prepare(g.plan);
+        if (s == GPE_OK) s = plan_prepare(g.plan, 0);
         if (s == GPE_OK && (cudaMalloc((void **)&g.d_ptrs, sizeof(void *) * n) != cudaSuccess ||
                             cudaMalloc((void **)&g.d_slots, sizeof(int) * n) != cudaSuccess))
             s = sfail(GPE_ENOMEM, "batch pointer arrays");
@@ -430,7 +430,7 @@ static void admit(gpe_server *s)
             d.gamma_each = gm.data();
             if (cudaStreamCreateWithFlags(&g->st, cudaStreamNonBlocking) != cudaSuccess) st = GPE_ECUDA;
             if (st == GPE_OK) st = gpe_plan_create(&d, g->st, &g->plan);
-            if (st == GPE_OK) st = plan_prepare(g->plan);
+            if (st == GPE_OK) st = plan_prepare(g->plan, g->imag);
             if (st == GPE_OK && (cudaMalloc((void **)&g->d_ptrs, sizeof(void *) * d.batch) != cudaSuccess ||
                                  cudaMalloc((void **)&g->d_slots, sizeof(int) * d.batch) != cudaSuccess))
                 st = GPE_ENOMEM;

@@ -2,7 +2,7 @@
 a stand-in for the runtime (fake_cudart.cpp; no GPU, no kernel runs)."""
 import ctypes
 import os
-import re
+import shutil
 import subprocess
 
 import numpy as np
@@ -30,7 +30,8 @@ def loaded(tmp_path_factory):
     gpe.build()
     path = str(tmp_path_factory.mktemp("fake") / "libgpe_fake.so")
     objs = [os.path.join(buildlib.BUILD, s.replace(".cu", ".o")) for s in buildlib.SOURCES]
-    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-I" + os.path.join(CUDA, "include"),
+    # (symbolic: another runtime that is loaded already must not take the calls)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I" + os.path.join(CUDA, "include"),
                     os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-o", path, "-lpthread"], check=True)
     real = gpe.LIB_PATH, gpe._lib
     gpe.LIB_PATH, gpe._lib = path, None
@@ -38,6 +39,21 @@ def loaded(tmp_path_factory):
         yield gpe, Fake(gpe.lib())
     finally:
         gpe.LIB_PATH, gpe._lib = real
+        os.unlink(path)
+
+
+@pytest.fixture
+def unused(loaded, tmp_path):
+    """Another copy of the library, none of whose kernels has been asked for yet."""
+    gpe = loaded[0]
+    path = str(tmp_path / "libgpe_unused.so")
+    shutil.copy(gpe.LIB_PATH, path)
+    before = gpe.LIB_PATH, gpe._lib
+    gpe.LIB_PATH, gpe._lib = path, None
+    try:
+        yield gpe, Fake(gpe.lib())
+    finally:
+        gpe.LIB_PATH, gpe._lib = before
         os.unlink(path)
 
 
@@ -186,3 +202,23 @@ def test_tuner_times_the_sweeps_of_planes_stepped_on_chip(gpe, fake, clusters):
     fake.lib.fake_clusters(clusters)
     with Made(gpe, (128, 64 if clusters else 128)) as p:
         assert timed(gpe, fake, p) > 0
+
+
+BATCHES = {"resident": [((64, 64), 0)], "plane": [((64, 64), 1)], "sweeps": [((128, 128), 1)] * 9, "rows": [((512, 16), 0)],
+           "3d": [((128, 64, 16), 0)], "3d_c128": [((64, 128, 16), 1)], "lines": [((1024,), 0)], "few_lines": [((128,), 1)],
+           "many_lines": [((32,), 1)] * 310}
+
+
+@pytest.mark.parametrize("kind", BATCHES)
+def test_batch_resolves_its_kernels_before_capture(unused, kind):
+    gpe, fake = unused
+    made = [desc(gpe, n, prec) for n, prec in BATCHES[kind]]
+    bufs = [np.zeros(2 * int(np.prod(n)) + 2) for n, _ in BATCHES[kind]]
+    b = gpe.gpe_batch_create([m[0] for m in made], STREAM)
+    fake.lib.fake_reset()
+    gpe.gpe_batch_step_real(b, [(x.ctypes.data + 15) // 16 * 16 for x in bufs], 3, 1)
+    gpe.gpe_batch_destroy(b)
+    log = fake.log()
+    captured = log[log.index("begin"):log.index("end")]
+    assert any(line.startswith("kernel") for line in captured)
+    assert not [line for line in captured if line.startswith("resolve")]
