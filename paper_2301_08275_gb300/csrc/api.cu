@@ -2059,16 +2059,22 @@ gpe_status plan_prepare(gpe_plan *p, int imag)
 }
 
 // Give slot `slot` of a plan new interaction and trap parameters: host FP64
-// tables, uploaded on the plan stream.  Axes without a trap table keep none
-// (the caller groups instances by which axes are trapped).
+// tables, uploaded on the plan stream, which is waited for once.  Axes without a
+// trap table keep none (the caller groups instances by which axes are trapped).
 gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamma)
 {
     if (slot < 0 || slot >= p->batch) return fail(GPE_EINVAL, "slot out of range");
     DeviceGuard dg(p->device);
-    GPE_CUDA(cudaMemcpyAsync(p->g_dev + slot, &g, sizeof(double), cudaMemcpyHostToDevice, p->st));
+    std::vector<std::vector<unsigned char>> staged;      // sources of the copies in flight
+    auto put = [&](void *table, size_t entry, size_t count, const void *src) -> gpe_status {
+        const size_t len = entry * count;
+        staged.emplace_back(static_cast<const unsigned char *>(src), static_cast<const unsigned char *>(src) + len);
+        GPE_CUDA(cudaMemcpyAsync(static_cast<char *>(table) + (size_t)slot * len, staged.back().data(), len,
+                                 cudaMemcpyHostToDevice, p->st));
+        return GPE_OK;
+    };
     double gm[3] = {0, 0, 0};
     for (int a = 0; a < p->ndim; ++a) gm[a] = gamma[a];
-    GPE_CUDA(cudaMemcpyAsync(p->gamma_dev + 3 * slot, gm, sizeof(gm), cudaMemcpyHostToDevice, p->st));
     FxCoupling gx[2];
     float gf[2];
     for (int full = 0; full < 2; ++full) {
@@ -2076,44 +2082,41 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
         gx[full] = coupling_fx(g, c);
         gf[full] = (float)(g * c);
     }
-    if (p->prec == GPE_C128)
-        GPE_CUDA(cudaMemcpyAsync((FxCoupling *)p->gq + 2 * slot, gx, sizeof(gx), cudaMemcpyHostToDevice, p->st));
-    else
-        GPE_CUDA(cudaMemcpyAsync((float *)p->gq + 2 * slot, gf, sizeof(gf), cudaMemcpyHostToDevice, p->st));
-    GPE_CUDA(cudaStreamSynchronize(p->st));        // host staging goes out of scope
-    for (int a = 0; a < p->ndim; ++a) {
-        if (!p->trap[a]) continue;
-        const int64_t na = p->n[a];
-        if (p->prec == GPE_C128) {
-            std::vector<int64_t> vq(na), viq(na);
-            trap_fx(p, a, gm[a], vq.data(), viq.data());
-            const size_t len = (size_t)na * sizeof(int64_t);
-            GPE_CUDA(cudaMemcpyAsync((int64_t *)p->vq[a] + slot * na, vq.data(), len, cudaMemcpyHostToDevice, p->st));
-            GPE_CUDA(cudaMemcpyAsync((int64_t *)p->viq[a] + slot * na, viq.data(), len, cudaMemcpyHostToDevice, p->st));
-            std::vector<double> vi(na);
-            if (p->ndim == 1) {
-                trap_decay_host(p, a, gm[a], vi.data());
-                GPE_CUDA(cudaMemcpyAsync((double *)p->vi[a] + slot * na, vi.data(), na * sizeof(double),
-                                         cudaMemcpyHostToDevice, p->st));
+    auto copies = [&]() -> gpe_status {
+        GPE_TRY(put(p->g_dev, sizeof(double), 1, &g));
+        GPE_TRY(put(p->gamma_dev, sizeof(double), 3, gm));
+        if (p->prec == GPE_C128) GPE_TRY(put(p->gq, sizeof(FxCoupling), 2, gx));
+        else GPE_TRY(put(p->gq, sizeof(float), 2, gf));
+        for (int a = 0; a < p->ndim; ++a) {
+            if (!p->trap[a]) continue;
+            const size_t na = (size_t)p->n[a];
+            if (p->prec == GPE_C128) {
+                std::vector<int64_t> vq(na), viq(na);
+                trap_fx(p, a, gm[a], vq.data(), viq.data());
+                GPE_TRY(put(p->vq[a], sizeof(int64_t), na, vq.data()));
+                GPE_TRY(put(p->viq[a], sizeof(int64_t), na, viq.data()));
+                if (p->ndim == 1) {
+                    std::vector<double> vi(na);
+                    trap_decay_host(p, a, gm[a], vi.data());
+                    GPE_TRY(put(p->vi[a], sizeof(double), na, vi.data()));
+                }
+                continue;
             }
-            GPE_CUDA(cudaStreamSynchronize(p->st));
-            continue;
+            std::vector<double> vh(2 * na), vf(2 * na), vi(na);
+            trap_tables_host(p, a, gm[a], vh.data(), vf.data(), vi.data());
+            std::vector<unsigned char> bh, bf;
+            pack_cplx(p, vh, bh);
+            pack_cplx(p, vf, bf);
+            const std::vector<float> f(vi.begin(), vi.end());
+            GPE_TRY(put(p->vh[a], bh.size() / na, na, bh.data()));
+            GPE_TRY(put(p->vf[a], bf.size() / na, na, bf.data()));
+            GPE_TRY(put(p->vi[a], sizeof(float), na, f.data()));
         }
-        std::vector<double> vh(2 * na), vf(2 * na), vi(na);
-        trap_tables_host(p, a, gm[a], vh.data(), vf.data(), vi.data());
-        std::vector<unsigned char> bh, bf;
-        pack_cplx(p, vh, bh);
-        pack_cplx(p, vf, bf);
-        const size_t ce = bh.size() / (size_t)na;      // bytes per complex entry
-        GPE_CUDA(cudaMemcpyAsync((char *)p->vh[a] + slot * na * ce, bh.data(), bh.size(), cudaMemcpyHostToDevice, p->st));
-        GPE_CUDA(cudaMemcpyAsync((char *)p->vf[a] + slot * na * ce, bf.data(), bf.size(), cudaMemcpyHostToDevice, p->st));
-        std::vector<float> f(vi.begin(), vi.end());
-        GPE_CUDA(cudaMemcpyAsync((float *)p->vi[a] + slot * na, f.data(), f.size() * sizeof(float),
-                                 cudaMemcpyHostToDevice, p->st));
-        GPE_CUDA(cudaStreamSynchronize(p->st));    // host staging goes out of scope
-    }
+        return GPE_OK;
+    };
+    const gpe_status s = copies();
     GPE_CUDA(cudaStreamSynchronize(p->st));
-    return GPE_OK;
+    return s;
 }
 
 // Run `count` instances found through the device arrays dptrs (base pointers)

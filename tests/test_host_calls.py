@@ -222,3 +222,19 @@ def test_batch_resolves_its_kernels_before_capture(unused, kind):
     captured = log[log.index("begin"):log.index("end")]
     assert any(line.startswith("kernel") for line in captured)
     assert not [line for line in captured if line.startswith("resolve")]
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+@pytest.mark.parametrize("n", [(64,), (32, 64), (32, 16, 8)], ids=lambda n: "x".join(map(str, n)))
+def test_admission_waits_for_the_stream_once(gpe, fake, n, prec):
+    """Parameters and tables of a slot are uploaded without a wait between them."""
+    d, keep = desc(gpe, n, prec)
+    psi = np.zeros(n[::-1], dtype=np.complex128 if prec else np.complex64)
+    srv = gpe.gpe_server_create(1 << 30, max_active=4, chunk_steps=4)
+    t = gpe.gpe_serve_submit(srv, d, psi, imag=False, nsteps=3)
+    assert gpe.gpe_serve_poll(srv, t, -1, np.empty_like(psi)).status == 0
+    gpe.gpe_server_destroy(srv)
+    log = fake.log()
+    first = next(i for i, line in enumerate(log) if line.startswith("kernel"))
+    stream = log[first].split()[1]
+    assert log[:first].count("wait " + stream) == 1
