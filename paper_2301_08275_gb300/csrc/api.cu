@@ -100,7 +100,7 @@ struct gpe_plan {
     double *g_dev = nullptr, *gamma_dev = nullptr, *scale = nullptr, *partials = nullptr;
     double *sums = nullptr, *out6 = nullptr, *out4 = nullptr;
     double *csum = nullptr;                  // chunk sums of the line reductions
-    unsigned *red_count = nullptr;           // CTAs of a line reduction that are done
+    unsigned *red_count = nullptr;           // CTAs of a line reduction that are done, per instance
     // imaginary-time convergence on the device: [0] stop word (int), [8] steps done (int64_t)
     unsigned char *istate = nullptr;
     double *eprev = nullptr;                 // [batch] energies of the last check
@@ -569,7 +569,7 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
     {
         int64_t nch = 1;
         for (int a = 0; a < d->ndim; ++a) nch = std::max(nch, reduce_chunks(p->N / p->n[a]));
-        PLAN_TRY(dalloc(p, (void **)&p->csum, sizeof(double) * (NQ * B * nch + 1)));
+        PLAN_TRY(dalloc(p, (void **)&p->csum, sizeof(double) * NQ * B * nch + sizeof(unsigned) * B));
         p->red_count = reinterpret_cast<unsigned *>(p->csum + NQ * B * nch);
     }
     PLAN_TRY(dalloc(p, (void **)&p->istate, 16));
@@ -601,7 +601,7 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
     if (cudaMemcpy(p->g_dev, gs.data(), sizeof(double) * B, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(p->gamma_dev, gam.data(), sizeof(double) * 3 * B, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(p->red_count, 0, sizeof(unsigned)) != cudaSuccess) {
+        cudaMemset(p->red_count, 0, sizeof(unsigned) * B) != cudaSuccess) {
         destroy(p);
         return fail(GPE_ECUDA, "uploading plan parameters failed");
     }

@@ -223,7 +223,7 @@ cudaError_t launch_trap_level(int prec, void *const *tab, int ndim, const int64_
 // sums[b*NQ + q], q in [nq_first, nq_first + nq): per-instance sums of the
 // per-line partials, in a fixed order (chunks of REDUCE_CHUNK lines, then the
 // chunk sums); csum is scratch of batch * NQ * reduce_chunks(lines_per_inst)
-// doubles, counter a word that is zero before the first call on a stream.  With
+// doubles, counter a word per instance, zero before the first call on a stream.  With
 // scale set, the q = 0 sum also gives the renormalisation
 // factor scale[b] = sqrt(target / (sum * dv)) (err |= ERR_NUMERIC and
 // scale[b] = 1 for a zero or non-finite norm).

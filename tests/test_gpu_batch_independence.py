@@ -80,3 +80,28 @@ def test_imaginary_time_on_chip_and_as_sweeps(gpe, n, sampled, prec):
     for i in range(most + 1):
         assert np.array_equal(over[i], a[i % 3]), i
         assert i == most or np.array_equal(at[i], a[i % 3]), i
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+@pytest.mark.parametrize("n", [(8, 256, 256), (128, 64, 64), (128, 16, 128)], ids=lambda n: "x".join(map(str, n)))
+def test_sums_of_several_instances_of_several_chunks(gpe, n, prec):
+    """More than 4096 lines per instance and axis: chunk sums, added per instance."""
+    import torch
+    sp = gi.Spec(n=n, lo=(-6.0,) * 3, length=(12.0,) * 3, g=20.0, dt=1e-3, gamma=(1.0, 1.2, 1.4))
+    psi = np.stack([(1 + b) * gi.random_field(sp, seed=b, smooth=0.05) for b in range(5)])
+    psi = torch.from_numpy(psi).cuda().to(torch.complex128 if prec else torch.complex64)
+
+    def values(x, g):
+        p = gpe.Plan(sp.n, sp.lo, sp.length, g=0.0, dt=sp.dt, gamma=sp.gamma, prec=prec, batch=len(g), g_each=g)
+        x = x.clone()
+        out = [p.norm_energy(x), p.rms_size(x), p.norm_energy(x)]
+        _, e = p.step_imag(x, 3, 1.0, 0.0, 1)
+        torch.cuda.synchronize()
+        p.close()
+        return out + [np.reshape(e, -1), x.cpu().numpy()]
+
+    g = [5.0 * b for b in range(5)]
+    many = values(psi, g)
+    for b in range(5):
+        for m, one in zip(many, values(psi[b:b + 1], g[b:b + 1])):
+            assert np.array_equal(m[b], one[0])
