@@ -105,3 +105,65 @@ def test_sums_of_several_instances_of_several_chunks(gpe, n, prec):
     for b in range(5):
         for m, one in zip(many, values(psi[b:b + 1], g[b:b + 1])):
             assert np.array_equal(m[b], one[0])
+
+
+def planes(count, seed):
+    """2D instances that are stepped on chip when grouped, each with its own g and trap."""
+    rng = np.random.default_rng(seed)
+    shapes = [(128, 64), (64, 128), (128, 128), (64, 64)]
+    return [gi.Spec(n=shapes[i % 4], lo=(-6.0, -6.0), length=(12.0, 12.0), g=float(rng.uniform(0, 200)), dt=1e-3,
+                    gamma=tuple(float(v) for v in rng.uniform(1.0, 3.0, size=2))) for i in range(count)]
+
+
+def as_sweeps(gpe, sp, psi, prec, imag, nsteps, check_every=1):
+    import torch
+    p = gpe.Plan(sp.n, sp.lo, sp.length, g=sp.g, dt=sp.dt, gamma=sp.gamma[:2], prec=prec)
+    p.set_option(gpe.GPE_OPT_TILE_X, 0)
+    x = torch.from_numpy(psi.copy()).cuda()
+    if imag:
+        p.step_imag(x, nsteps, 1.0, 0.0, check_every)
+    else:
+        p.step_real(x, nsteps)
+    torch.cuda.synchronize()
+    p.close()
+    return x.cpu().numpy()
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+def test_planes_of_a_batch_keep_their_parameters(gpe, prec):
+    import torch
+    dt = np.complex128 if prec else np.complex64
+    specs = planes(16, seed=prec)
+    psi = [gi.random_field(sp, seed=i, smooth=0.05).astype(dt) for i, sp in enumerate(specs)]
+    xs = [torch.from_numpy(p.copy()).cuda() for p in psi]
+    descs = [gpe.make_desc(sp.n, sp.lo, sp.length, g=sp.g, dt=sp.dt, gamma=sp.gamma[:2], prec=prec)[0] for sp in specs]
+    b = gpe.gpe_batch_create(descs, torch.cuda.current_stream().cuda_stream)
+    gpe.gpe_batch_step_real(b, [x.data_ptr() for x in xs], 9, True)
+    torch.cuda.synchronize()
+    gpe.gpe_batch_destroy(b)
+    for i, sp in enumerate(specs):
+        assert np.array_equal(xs[i].cpu().numpy(), as_sweeps(gpe, sp, psi[i], prec, False, 9)), i
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["c64", "c128"])
+def test_planes_of_a_server_keep_their_slots(gpe, prec):
+    """More requests than places, of different lengths: slots are handed on, and the
+    members of a round are not in the order of their slots."""
+    dt = np.complex128 if prec else np.complex64
+    specs = [sp for sp in planes(40, seed=10 + prec) if sp.n in ((128, 64), (64, 64))]
+    psi = [gi.random_field(sp, seed=i, smooth=0.05).astype(dt) for i, sp in enumerate(specs)]
+    nsteps = [5 * (1 + (7 * i) % 11) for i in range(len(specs))]
+    srv = gpe.gpe_server_create(1 << 30, max_active=7, chunk_steps=5)
+    tickets = [gpe.gpe_serve_submit(srv, gpe.make_desc(sp.n, sp.lo, sp.length, g=sp.g, dt=sp.dt, gamma=sp.gamma[:2],
+                                                       prec=prec)[0], psi[i], imag=i % 3 > 0, nsteps=nsteps[i],
+                                    etol=0.0, check_every=5) for i, sp in enumerate(specs)]
+    for i, t in enumerate(tickets):
+        out = np.empty_like(psi[i])
+        r = gpe.gpe_serve_poll(srv, t, timeout_ms=-1, psi_out=out)
+        assert r.status == 0 and r.steps_done == nsteps[i]
+        if i % 3 > 0:
+            assert np.array_equal(out, as_sweeps(gpe, specs[i], psi[i], prec, True, nsteps[i], 5)), i
+        else:      # real-time requests advance in chunks; a chunk ends and opens the nonlinear half-step
+            assert np.linalg.norm(out - as_sweeps(gpe, specs[i], psi[i], prec, False, nsteps[i])) < \
+                (1e-12 if prec else 1e-4) * np.linalg.norm(out), i
+    gpe.gpe_server_destroy(srv)
