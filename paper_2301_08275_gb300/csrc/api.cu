@@ -201,21 +201,14 @@ static gpe_status upload_real(gpe_plan *p, void **dst, const std::vector<double>
     }
     return GPE_OK;
 }
-// v holds interleaved (re, im) of unit factors.  complex128: stored as is;
-// complex64: each value w becomes (hi, lo) = (fl(w), fl(w - fl(w))) so that
-// kernels can apply it without a per-application modulus error.
+// v holds interleaved (re, im) of unit factors: stored as is in complex128, by
+// pack_cplx in complex64
+static std::vector<float> pack_cplx(const std::vector<double> &v);
 static gpe_status upload_cplx(gpe_plan *p, void **dst, const std::vector<double> &v)
 {
     if (p->prec != GPE_C64) return upload_real(p, dst, v);
-    GPE_TRY(dalloc(p, dst, v.size() * 2 * sizeof(float)));
-    std::vector<float> f(v.size() * 2);
-    for (size_t i = 0; i + 1 < v.size(); i += 2) {
-        const float hx = (float)v[i], hy = (float)v[i + 1];
-        f[2 * i + 0] = hx;
-        f[2 * i + 1] = hy;
-        f[2 * i + 2] = (float)(v[i] - (double)hx);
-        f[2 * i + 3] = (float)(v[i + 1] - (double)hy);
-    }
+    const std::vector<float> f = pack_cplx(v);
+    GPE_TRY(dalloc(p, dst, f.size() * sizeof(float)));
     GPE_CUDA(cudaMemcpy(*dst, f.data(), f.size() * sizeof(float), cudaMemcpyHostToDevice));
     return GPE_OK;
 }
@@ -372,14 +365,11 @@ static void trap_tables_host(const gpe_plan *p, int a, double gamma, double *vh,
     }
 }
 
-// complex table values (re, im) in the device format of the plan's precision
-static void pack_cplx(const gpe_plan *p, const std::vector<double> &v, std::vector<unsigned char> &out)
+// unit factors (re, im) as the device tables of complex64 hold them: each value w
+// as (hi, lo) = (fl(w), fl(w - fl(w))), so that kernels can apply it without a
+// per-application modulus error
+static std::vector<float> pack_cplx(const std::vector<double> &v)
 {
-    if (p->prec != GPE_C64) {
-        out.resize(v.size() * sizeof(double));
-        memcpy(out.data(), v.data(), out.size());
-        return;
-    }
     std::vector<float> f(v.size() * 2);
     for (size_t i = 0; i + 1 < v.size(); i += 2) {
         const float hx = (float)v[i], hy = (float)v[i + 1];
@@ -388,8 +378,7 @@ static void pack_cplx(const gpe_plan *p, const std::vector<double> &v, std::vect
         f[2 * i + 2] = (float)(v[i] - (double)hx);
         f[2 * i + 3] = (float)(v[i + 1] - (double)hy);
     }
-    out.resize(f.size() * sizeof(float));
-    memcpy(out.data(), f.data(), out.size());
+    return f;
 }
 
 extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream, gpe_plan **out)
@@ -534,22 +523,24 @@ extern "C" gpe_status gpe_plan_create(const gpe_plan_desc *d, void *cuda_stream,
         PLAN_TRY(upload_real(p, &p->vsamp, std::vector<double>(d->V_host, d->V_host + p->N)));
         if (d->ndim == 1) {
             const int64_t na = p->n[0];
-            std::vector<double> vh(2 * na * B), vf(2 * na * B), vi(na * B);
+            std::vector<double> vi(na * B);
             for (int64_t b = 0; b < B; ++b)
-                for (int64_t j = 0; j < na; ++j) {
-                    const double th = d->V_host[j] * p->dt;
-                    vh[2 * (b * na + j)] = -2.0 * sin(0.25 * th) * sin(0.25 * th);
-                    vh[2 * (b * na + j) + 1] = -sin(0.5 * th);
-                    vf[2 * (b * na + j)] = -2.0 * sin(0.5 * th) * sin(0.5 * th);
-                    vf[2 * (b * na + j) + 1] = -sin(th);
-                    vi[b * na + j] = exp(-0.5 * th);
-                }
+                for (int64_t j = 0; j < na; ++j) vi[b * na + j] = exp(-0.5 * (d->V_host[j] * p->dt));
             if (p->prec == GPE_C128) {
                 std::vector<int64_t> vq(na * B);
                 for (int64_t b = 0; b < B; ++b)
                     for (int64_t j = 0; j < na; ++j) vq[b * na + j] = turns_fx(0.5 * d->V_host[j] * p->dt);
                 PLAN_TRY(upload_raw(p, &p->vq[0], vq.data(), vq.size() * sizeof(int64_t)));
             } else {
+                std::vector<double> vh(2 * na * B), vf(2 * na * B);
+                for (int64_t b = 0; b < B; ++b)
+                    for (int64_t j = 0; j < na; ++j) {
+                        const double th = d->V_host[j] * p->dt;
+                        vh[2 * (b * na + j)] = -2.0 * sin(0.25 * th) * sin(0.25 * th);
+                        vh[2 * (b * na + j) + 1] = -sin(0.5 * th);
+                        vf[2 * (b * na + j)] = -2.0 * sin(0.5 * th) * sin(0.5 * th);
+                        vf[2 * (b * na + j) + 1] = -sin(th);
+                    }
                 PLAN_TRY(upload_cplx(p, &p->vh[0], vh));
                 PLAN_TRY(upload_cplx(p, &p->vf[0], vf));
             }
@@ -2104,12 +2095,9 @@ gpe_status plan_set_slot(gpe_plan *p, int64_t slot, double g, const double *gamm
             }
             std::vector<double> vh(2 * na), vf(2 * na), vi(na);
             trap_tables_host(p, a, gm[a], vh.data(), vf.data(), vi.data());
-            std::vector<unsigned char> bh, bf;
-            pack_cplx(p, vh, bh);
-            pack_cplx(p, vf, bf);
-            const std::vector<float> f(vi.begin(), vi.end());
-            GPE_TRY(put(p->vh[a], bh.size() / na, na, bh.data()));
-            GPE_TRY(put(p->vf[a], bf.size() / na, na, bf.data()));
+            const std::vector<float> bh = pack_cplx(vh), bf = pack_cplx(vf), f(vi.begin(), vi.end());
+            GPE_TRY(put(p->vh[a], sizeof(float4), na, bh.data()));
+            GPE_TRY(put(p->vf[a], sizeof(float4), na, bf.data()));
             GPE_TRY(put(p->vi[a], sizeof(float), na, f.data()));
         }
         return GPE_OK;

@@ -112,10 +112,6 @@ __device__ __forceinline__ float2 cmadd1(float2 v, float2 w)
 {
     return mk(v.x + fmaf(v.x, w.x, -v.y * w.y), v.y + fmaf(v.x, w.y, v.y * w.x));
 }
-__device__ __forceinline__ double2 cmadd1(double2 v, double2 w)
-{
-    return mk(v.x + fma(v.x, w.x, -v.y * w.y), v.y + fma(v.x, w.y, v.y * w.x));
-}
 // same with the offset held as a hi + lo float pair (table entries)
 __device__ __forceinline__ float2 uomul(float2 v, float4 w)
 {
@@ -123,7 +119,6 @@ __device__ __forceinline__ float2 uomul(float2 v, float4 w)
     const float ty = fmaf(v.x, w.w, v.y * w.z);
     return mk(v.x + fmaf(v.x, w.x, fmaf(-v.y, w.y, tx)), v.y + fmaf(v.x, w.y, fmaf(v.y, w.x, ty)));
 }
-__device__ __forceinline__ double2 uomul(double2 v, double2 w) { return cmadd1(v, w); }
 // offset form of a product of two unit factors: (1+a)(1+b) - 1
 template <typename C> __device__ __forceinline__ C wcomb(C a, C b)
 {
@@ -314,82 +309,6 @@ template <int N> struct Radix4 {
 template <int N, int E> struct PassPlan { using T = Radix<N>; };
 template <int N> struct PassPlan<N, 4> { using T = Radix4<N>; };
 template <int N> struct PassPlan<N, 32> { using T = Radix32<N>; };
-
-// ---------------------------------------------------------------- tile engine
-// ROWS = true : lines are contiguous rows (x axis); shared layout row-major with
-//               the point index XOR-swizzled inside each 128-byte block
-//               (i ^ ((i / P) mod P), P points per 128 bytes), which keeps both
-//               the contiguous reads and the stride-r Stockham writes free of
-//               bank conflicts.
-// ROWS = false: lines are strided (y or z axis); L lines interleaved point by point.
-template <typename R, int N, int L, bool ROWS> struct Tile {
-    using C = typename CT<R>::C;
-    static constexpr int E = Radix<N>::E;
-    static constexpr int TPL = N / E;
-    static constexpr int NT = L * TPL;
-    static constexpr int P = 128 / (int)sizeof(C);      // points per 128-byte block
-    static constexpr int SMEM_POINTS = N * L;
-
-    __device__ __forceinline__ static int sidx(int i, int l)
-    {
-        if (ROWS) return l * N + (i ^ ((i / P) & (P - 1)));
-        return i * L + l;
-    }
-    __device__ __forceinline__ static int line_of(int t) { return ROWS ? t / TPL : t % L; }
-    __device__ __forceinline__ static int tl_of(int t) { return ROWS ? t % TPL : t / L; }
-
-    using U = typename UT<R>::U;
-
-    // One pass p of the transform.  v holds points tl + TPL*e.
-    template <int DIR, int p>
-    __device__ __forceinline__ static void pass(C (&v)[E], C *sm, int tl, int l, const U *__restrict__ tw)
-    {
-        constexpr int r = Radix<N>::radix(p);
-        constexpr int Ns = Radix<N>::ns(p);
-        constexpr int B = E / r;
-        constexpr bool last = (p == Radix<N>::P - 1);
-        if constexpr (p > 0) {
-            __syncthreads();                          // previous pass outputs visible
-#pragma unroll
-            for (int e = 0; e < E; ++e) v[e] = sm[sidx(tl + TPL * e, l)];
-            if constexpr (!last) __syncthreads();     // all reads done before rewriting
-        } else if constexpr (!last) {
-            __syncthreads();                          // earlier readers of sm are done
-        }
-#pragma unroll
-        for (int q = 0; q < B; ++q) {
-            const int j = tl + q * TPL;
-            const int k = j & (Ns - 1);
-            C x[r];
-#pragma unroll
-            for (int m = 0; m < r; ++m) x[m] = v[q + m * B];
-            if constexpr (Ns > 1) {
-#pragma unroll
-                for (int m = 1; m < r; ++m) x[m] = umul<(DIR > 0)>(x[m], tw[m * k * (N / (Ns * r))]);
-            }
-            Dft<r, DIR, C>::run(x);
-            if constexpr (last) {
-#pragma unroll
-                for (int m = 0; m < r; ++m) v[q + m * B] = x[m];
-            } else {
-                const int base = (j / Ns) * Ns * r + k;
-#pragma unroll
-                for (int m = 0; m < r; ++m) sm[sidx(base + m * Ns, l)] = x[m];
-            }
-        }
-    }
-
-    // Full N-point transform of the thread's line, in place in registers.
-    // DIR = -1 forward (unnormalised), +1 inverse (unnormalised).
-    template <int DIR, int p = 0>
-    __device__ __forceinline__ static void fft(C (&v)[E], C *sm, int tl, int l, const U *tw)
-    {
-        if constexpr (p < Radix<N>::P) {
-            pass<DIR, p>(v, sm, tl, l, tw);
-            fft<DIR, p + 1>(v, sm, tl, l, tw);
-        }
-    }
-};
 
 // ---------------------------------------------------------------- line groups
 // Strided tile in which each thread carries LPT adjacent lines: the points

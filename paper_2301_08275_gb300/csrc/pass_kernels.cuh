@@ -14,41 +14,15 @@
 
 namespace gpe {
 
-__device__ __forceinline__ void sincos_r(float x, float *s, float *c) { sincosf(x, s, c); }
-__device__ __forceinline__ void sincos_r(double x, double *s, double *c) { sincos(x, s, c); }
 __device__ __forceinline__ float exp_r(float x) { return expf(x); }
 __device__ __forceinline__ double exp_r(double x) { return exp(x); }
 
-// exp(-i th) - 1 = (cos th - 1, -sin th).  Double precision: from the half
-// angle, (-2 sin^2(th/2), -sin th).  Single precision, |th| <= 1/2: the
+// exp(-i th) - 1 = (cos th - 1, -sin th) of complex64 sweeps.  |th| <= 1/2: the
 // Maclaurin series of cos th - 1 and sin th to the th^10 / th^11 terms
 // (truncation below 1e-11 relative), evaluated by Horner's rule in th^2;
 // larger angles fall back to sincosf of the half angle.
-__device__ __forceinline__ double2 phase_offset(double th)
-{
-    double s, c;
-    sincos(0.5 * th, &s, &c);
-    return mk(-2.0 * s * s, -2.0 * s * c);
-}
-// short forms for |th| <= 1/16 (Maclaurin series of cos th - 1 and sin th).
-// double: terms to th^12 / th^13, truncation below 1e-27;
-// float: terms to th^6 / th^5, truncation below 1e-12 (sin) and 1e-14 (cos),
-// so the modulus of 1 + w stays one to about 1e-13
-__device__ __forceinline__ double2 phase_offset_small(double th)
-{
-    const double u = th * th;
-    const double cm =
-        u * fma(u, fma(u, fma(u, fma(u, fma(u, 1.0 / 479001600.0, -1.0 / 3628800.0), 1.0 / 40320.0), -1.0 / 720.0),
-                       1.0 / 24.0),
-                -0.5);
-    const double sn =
-        th * fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, 1.0 / 6227020800.0, -1.0 / 39916800.0), 1.0 / 362880.0),
-                                         -1.0 / 5040.0),
-                                 1.0 / 120.0),
-                         -1.0 / 6.0),
-                 1.0);
-    return mk(cm, -sn);
-}
+// Short form for |th| <= 1/16: terms to th^6 / th^5, truncation below 1e-12 (sin)
+// and 1e-14 (cos), so the modulus of 1 + w stays one to about 1e-13.
 __device__ __forceinline__ float2 phase_offset_small(float th)
 {
     const float u = th * th;
@@ -216,11 +190,6 @@ __device__ __forceinline__ float4 offset_product(float4 a, float4 b)
     two_sum(uy, ly, hy, gy);
     return make_float4(hx, hy, gx, gy);
 }
-__device__ __forceinline__ double2 offset_product(double2 a, double2 b)
-{
-    return make_double2(a.x + b.x + (a.x * b.x - a.y * b.y), a.y + b.y + (a.x * b.y + a.y * b.x));
-}
-
 // Component of the velocity (part 0: Im) or of the gradient of |psi| (part 1: Re)
 // from psi and a derivative d not yet divided by N; zero where |psi|^2 < 1e-30.
 template <typename R, typename C> __device__ __forceinline__ R velocity_of(C p, C d, int part, R invn)
@@ -231,7 +200,8 @@ template <typename R, typename C> __device__ __forceinline__ R velocity_of(C p, 
     return u;
 }
 
-// pointwise substep on the E points (indices tl + TPL*e on this axis) of one line
+// pointwise substep of a complex64 sweep (complex128: fx_sweep) on the E points
+// (indices tl + TPL*e on this axis) of one line
 // inst: position of the instance in this launch (renormalisation factor);
 // ti: its parameter/table slot
 // off: offset of the line's first point within its instance (sampled potential)
@@ -242,6 +212,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
                                          int ti, int c0, int c1, int tl, int64_t off,
                                          const typename UT<R>::U *vreg = nullptr)
 {
+    static_assert(sizeof(R) == 4, "complex64");
     using C = typename CT<R>::C;
     if (op == OP_NONE) return;
     using U = typename UT<R>::U;
@@ -259,10 +230,7 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
         // the factors of the line's other axes, combined once per line into
         // one offset to twice the working precision
         U fl = offset_product(k0 ? k0[c0] : U{}, k1 ? k1[c1] : U{});
-        if constexpr (sizeof(R) == 4) {
-            if (a.dither)
-                fl = offset_product(fl, make_float4(a.dk[0], a.dk[1], a.dk[2], a.dk[3]));
-        }
+        if (a.dither) fl = offset_product(fl, make_float4(a.dk[0], a.dk[1], a.dk[2], a.dk[3]));
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = cscale(uomul(uomul(v[e], kt[tl + TPL * e]), fl), invn);
         return;
@@ -276,23 +244,21 @@ __device__ __forceinline__ void point_op(int op, typename CT<R>::C (&v)[E], cons
         for (int e = 0; e < E; ++e) v[e] = cscale(v[e], fl * ki[tl + TPL * e]);
         return;
     }
-    if constexpr (sizeof(R) == 4) {
-        if (op == OP_DERIV) {
-            const float kl = a.dk_o0 ? a.dk_o0[c0] : a.dk_o1 ? a.dk_o1[c1] : 0.0f;
+    if (op == OP_DERIV) {
+        const float kl = a.dk_o0 ? a.dk_o0[c0] : a.dk_o1 ? a.dk_o1[c1] : 0.0f;
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const float k = a.dk_ax ? a.dk_ax[tl + TPL * e] : kl;
-                v[e] = mk(-k * v[e].y, k * v[e].x);
-            }
-            return;
+        for (int e = 0; e < E; ++e) {
+            const float k = a.dk_ax ? a.dk_ax[tl + TPL * e] : kl;
+            v[e] = mk(-k * v[e].y, k * v[e].x);
         }
-        if (op == OP_VEL) {                // rows
-            const C *psi = static_cast<const C *>(a.vel_psi) + off;
+        return;
+    }
+    if (op == OP_VEL) {                // rows
+        const C *psi = static_cast<const C *>(a.vel_psi) + off;
 #pragma unroll
-            for (int e = 0; e < E; ++e)
-                v[e] = mk(velocity_of<R>(psi[tl + TPL * e], v[e], a.vel_part, a.inv_n), 0.0f);
-            return;
-        }
+        for (int e = 0; e < E; ++e)
+            v[e] = mk(velocity_of<R>(psi[tl + TPL * e], v[e], a.vel_part, a.inv_n), 0.0f);
+        return;
     }
     if (op == OP_SCALE || op == OP_SCALE_NIMAG) {
         const R s = (R)a.scale[inst];
@@ -1306,40 +1272,44 @@ __global__ void __launch_bounds__(Line1DCfg<R, N, L>::NT) k_line1d(const Line1DA
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = valid ? psi[tl + TPL * e] : mk((R)0, (R)0);
         const double g = a.g[ib];
-        if (sizeof(R) == 4 && !a.imag) {        // complex128: k_line1d_fx
-            const U *kt = static_cast<const U *>(a.kt);
-            const U *vh = static_cast<const U *>(a.vh);
-            const U *vf = static_cast<const U *>(a.vf);
-            const R gh = (R)(g * 0.5 * a.dt), gf = (R)(g * a.dt);
-            const R invn = (R)(1.0 / N);
-            // first nonlinear half-step
-            {
-                R th[E];
+        const bool real = sizeof(R) == 4 && !a.imag;        // complex128: k_line1d_fx
+        if constexpr (sizeof(R) == 4) {
+            if (real) {
+                const U *kt = static_cast<const U *>(a.kt);
+                const U *vh = static_cast<const U *>(a.vh);
+                const U *vf = static_cast<const U *>(a.vf);
+                const R gh = (R)(g * 0.5 * a.dt), gf = (R)(g * a.dt);
+                const R invn = (R)(1.0 / N);
+                // first nonlinear half-step
+                {
+                    R th[E];
 #pragma unroll
-                for (int e = 0; e < E; ++e) th[e] = gh * cabs2(v[e]);
-                apply_phase<C, R, E>(v, th);
-            }
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                if (vh) v[e] = uomul(v[e], vh[ib * N + tl + TPL * e]);
-#pragma unroll 1
-            for (int64_t st = 0; st < a.nsteps; ++st) {
-                T::template fft<-1, PING>(w, sm, ss, tl, 0, twr);
-#pragma unroll
-                for (int e = 0; e < E; ++e) v[e] = cscale(uomul(v[e], kt[tl + TPL * e]), invn);
-                T::template fft<1, PING>(w, sm, ss, tl, 0, twr);
-                const bool last = (st == a.nsteps - 1);
-                const R gc = last ? gh : gf;
-                const U *vt = last ? (a.vh_last ? static_cast<const U *>(a.vh_last) : vh) : vf;
-                R th[E];
-#pragma unroll
-                for (int e = 0; e < E; ++e) th[e] = gc * cabs2(v[e]);
-                apply_phase<C, R, E>(v, th);
+                    for (int e = 0; e < E; ++e) th[e] = gh * cabs2(v[e]);
+                    apply_phase<C, R, E>(v, th);
+                }
 #pragma unroll
                 for (int e = 0; e < E; ++e)
-                    if (vt) v[e] = uomul(v[e], vt[ib * N + tl + TPL * e]);
+                    if (vh) v[e] = uomul(v[e], vh[ib * N + tl + TPL * e]);
+#pragma unroll 1
+                for (int64_t st = 0; st < a.nsteps; ++st) {
+                    T::template fft<-1, PING>(w, sm, ss, tl, 0, twr);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) v[e] = cscale(uomul(v[e], kt[tl + TPL * e]), invn);
+                    T::template fft<1, PING>(w, sm, ss, tl, 0, twr);
+                    const bool last = (st == a.nsteps - 1);
+                    const R gc = last ? gh : gf;
+                    const U *vt = last ? (a.vh_last ? static_cast<const U *>(a.vh_last) : vh) : vf;
+                    R th[E];
+#pragma unroll
+                    for (int e = 0; e < E; ++e) th[e] = gc * cabs2(v[e]);
+                    apply_phase<C, R, E>(v, th);
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (vt) v[e] = uomul(v[e], vt[ib * N + tl + TPL * e]);
+                }
             }
-        } else {
+        }
+        if (!real) {
             const R *ki = static_cast<const R *>(a.kt);
             const R *vi = static_cast<const R *>(a.vi);
             const R gh = (R)(g * 0.5 * a.dt);
