@@ -184,17 +184,22 @@ def cpu_sample(key, spec, max_seconds=25.0, steps=None, max_steps=None):
     return rec, psi, done
 
 
-def hbm_roofline(kind, avg_ms, state_bytes, kernels, traffic=None):
-    """Roofline of a sweep: it reads and writes every point once (a 1D launch
-    does so once for all its steps)."""
+def hbm_roofline(kind, avg_ms, state_bytes, kernels, traffic=None, c128=False):
+    """Roofline of a sweep: it reads and writes every point once (a launch that
+    holds the state on chip does so once for all its steps).  Where HBM is not what
+    bounds the launch, "frac" is None and the fraction stands under "hbm_frac"."""
     peak, src = measured_peaks()
     nbytes = 2.0 * state_bytes
     achieved = nbytes / (avg_ms / 1e3) / 1e9
     out = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
            "traffic": traffic, "kernel": kind, "kernel_avg_ms": avg_ms, "bytes_per_launch": nbytes,
            "peak_source": src, "kernels": kernels}
-    if kind.startswith("line1d"):
-        out["on_chip"] = "one launch runs every step of the call with the lines on chip: bound by latency"
+    on_chip = kind.startswith(("line1d", "plane", "resident"))
+    if on_chip or c128:
+        out["hbm_frac"], out["frac"] = out["frac"], None
+        out["bound"] = "latency" if on_chip else "integer issue"
+    if on_chip:
+        out["on_chip"] = "one launch runs the steps of the call with the state on chip: bound by latency"
     elif state_bytes < 100e6:
         out["l2_resident"] = ("the %.0f MiB state stays in L2 between launches: HBM bytes do not bind "
                               "these launches (each CTA runs one or two tiles; latency bound)"
@@ -362,7 +367,7 @@ def config_record(key, steps=None):
     kind, (cnt, tot) = max(tr.items(), key=lambda kv: kv[1][1])
     kernels = {k: {"launches": c, "avg_ms": t / c} for k, (c, t) in tr.items()}
     state_bytes = spec.N * (8 if prec == gpe.GPE_C64 else 16)
-    roof = hbm_roofline(kind, tot / cnt, state_bytes, kernels)
+    roof = hbm_roofline(kind, tot / cnt, state_bytes, kernels, c128=prec == gpe.GPE_C128)
     plan.close()
     return {"workload": wl["name"], "value": spec.N * steps / (ms / 1e3), "unit": UNIT, "steps": steps,
             "ms_per_step": ms / steps, "us_per_step": 1e3 * ms / steps, "dtype": wl["prec"], "tiles": tiles,
@@ -439,7 +444,7 @@ def run_ours(args, key, wl):
     kernels = {k: {"launches": c, "avg_ms": t / c, "share": t / sum(x[1] for x in tr.values())}
                for k, (c, t) in tr.items()}
     state_bytes = spec.N * (8 if prec == gpe.GPE_C64 else 16)
-    roofline = hbm_roofline(kind, avg_ms, state_bytes, kernels, read_traffic(kind, key))
+    roofline = hbm_roofline(kind, avg_ms, state_bytes, kernels, read_traffic(kind, key), prec == gpe.GPE_C128)
 
     # end to end through the host-buffer entry point: every step copies the
     # state in from pinned host memory and the result back

@@ -54,9 +54,13 @@ typedef enum gpe_status {
 } gpe_status;
 
 typedef enum gpe_precision {
-    GPE_C64 = 0,   /* complex64 bulk arithmetic, FP64 reductions and tables */
-    GPE_C128 = 1   /* complex128 state; the 2D/3D sweeps hold each line in 64-bit
-                      fixed point with a scale of its own (no less exact)    */
+    GPE_C64 = 0,   /* complex64 bulk arithmetic; tables from FP64; sums along a
+                      line and spectral parts in two-float, across lines FP64  */
+    GPE_C128 = 1   /* complex128 state; sweeps and 1D real-time steps hold each
+                      line in 64-bit fixed point with a scale of its own: 52 to
+                      55 bits below the line's rms value (FP64: 53 below each
+                      value), so values far under it carry fewer bits, as
+                      after any transform; errors in L2 are smaller          */
 } gpe_precision;
 
 /* Problem description (copied by gpe_plan_create). */
@@ -174,9 +178,10 @@ gpe_status gpe_spectrum(gpe_plan *plan, const void *psi_dev, unsigned kinds, dou
 /* Plan options (implementation choices, no counterpart in the paper).  2D grids
  * of 64 or 128 points per axis are stepped on chip by one cluster per instance;
  * setting any of the options 1 to 7 on such a plan selects the sweeps that the
- * option is about.  Every option takes 0 or 1; results are bit-identical for every setting (each
- * line's arithmetic does not depend on them, with the one exception noted at
- * GPE_OPT_GENERIC_PASSES), only the speed changes.
+ * option is about.  Every option takes 0 or 1.  Options 1 to 7 change the speed
+ * only: results are bit-identical for every setting (each line's arithmetic does
+ * not depend on them, with the one exception noted at GPE_OPT_GENERIC_PASSES),
+ * and so they are for any number of instances.
  *   GPE_OPT_TMA_STAGING  1 (default): tiles of the y and z sweeps are fetched
  *                        by the tensor-memory accelerator when the grid allows
  *                        it (n0 a multiple of the tile's line count, instances
@@ -190,11 +195,11 @@ gpe_status gpe_spectrum(gpe_plan *plan, const void *psi_dev, unsigned kinds, dou
  *                        reads its program (pointwise ops, transforms,
  *                        reduction) from the launch arguments; 0 (default):
  *                        the sweeps of the real- and imaginary-time steps on
- *                        complex64 lines of 256 to 1024 points run kernels
- *                        compiled for their program.  For tests and timing.
- *                        The one exception to bit-identical results: with
- *                        this option imaginary-time steps can differ in the
- *                        last place (real-time steps do not).
+ *                        lines of 64 points and more (complex128: 64 to 1024)
+ *                        run kernels compiled for their program.  For tests
+ *                        and timing.  The one exception to bit-identical
+ *                        results: with this option imaginary-time steps may
+ *                        differ in the last place (real-time steps do not).
  *   GPE_OPT_NO_DITHER    1: turns off the phase dither of complex64
  *                        real-time steps (the default, 0, keeps it): each
  *                        step's kinetic substep also turns the state by a
@@ -210,7 +215,8 @@ gpe_status gpe_spectrum(gpe_plan *plan, const void *psi_dev, unsigned kinds, dou
  *                        of 2, 4 or 8 CTAs (a latency path); 0: one CTA per
  *                        line.
  *                        The two factor the transform differently, so their
- *                        results differ in rounding (both agree with the
+ *                        results (and with 1, those of 32 and of 33 such
+ *                        lines) differ in rounding (both agree with the
  *                        FP64 reference to about 1e-14 per step).
  *   GPE_OPT_TEST_STALL_COPIES  test hook for the failure handling: 1 makes
  *                        every copy-engine tile wait, and every exchange wait
@@ -248,7 +254,8 @@ gpe_status gpe_plan_get_option(const gpe_plan *plan, int option, int64_t *value)
  * sampled or not) for the life of the process, so later plans of the same kind
  * tune without timing.  Needs two state-sized device
  * scratch arrays for the duration of the call; synchronises the plan stream.
- * 1D plans have nothing to tune (GPE_OK). */
+ * 1D plans have nothing to tune (GPE_OK).  2D plans that are stepped on chip have:
+ * steps in a trap schedule, diagnostics and spectra are sweeps. */
 #define GPE_TUNE_NO_TMA 1
 gpe_status gpe_plan_autotune(gpe_plan *plan, const void *psi_dev, int reps, int flags);
 

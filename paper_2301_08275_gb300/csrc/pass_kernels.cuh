@@ -784,9 +784,10 @@ __device__ __forceinline__ void fx_forward(double2 (&d)[PassTileFx<N, ROWS, VAR>
 // imaginary-time steps, with the first and last x sweeps of a real-time call.
 // Program 0 reads the slots from the arguments (every other sweep:
 // diagnostics, spectra, the final renormalisation).  The real-time programs
-// give the generic kernel's bits (tested); the imaginary-time ones (5-7) can
-// round differently from it in the last place (seen on the decay sweeps, cause
-// not identified), well inside the parity tolerances.
+// give the generic kernel's bits (tested); the imaginary-time ones (5-7) end in
+// plain products, which a compiler may fuse into what follows in one kernel and
+// not in another, and are held to the parity tolerances only (equal bits on the
+// seven grids tried in both precisions).
 struct SweepProg {
     int op_pre, fft1, op_mid, fft2, op_post, red;
 };

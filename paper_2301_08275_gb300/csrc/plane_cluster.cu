@@ -11,6 +11,11 @@
 // that owns its row, and one hardware cluster barrier follows each (what a
 // buffer held has been read before the barrier that precedes its next writes).
 //
+// Sizes: 64 and 128 points per axis, the small grids of the batched and ground-state
+// workloads.  32-point axes would leave a CTA of 8 with half a warp, and complex64
+// columns of 256 points take the sweeps' 32-point plan, whose threads would not be
+// those of the rows; 256 x 64 and 256 x 128 have not been tried.
+//
 // The lines run the same transforms, tables and pointwise code as the streaming
 // sweeps (pass_kernels.cuh), so their results are the same bits.
 // Measured, us per step on chip / as sweeps, one instance: 64^2 complex64 real
