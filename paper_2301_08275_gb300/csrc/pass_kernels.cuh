@@ -664,7 +664,8 @@ __device__ __forceinline__ void fx_nreal(fx2 (&v)[E], int q, const PassArgs &a, 
 // Three terms (the sweep's own axis, the other axes together, interaction with a
 // sampled potential), each held within +-FX_EXP_MAX: their sum stays below 2^10,
 // and a state whose norm is a double (its factors are then above 2^-256 where
-// it is, in each of a step's two half-steps) meets no limit.
+// it is, in each of a step's two half-steps) meets no limit unless terms of
+// opposite sign beyond 2^340 cancel.
 template <int E, int TPL>
 __device__ __forceinline__ void fx_nimag(double2 (&d)[E], double s, const PassArgs &a, const LineGeom &g, int tl)
 {
